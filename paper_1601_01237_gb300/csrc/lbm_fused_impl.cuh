@@ -40,6 +40,7 @@
 
 #include <atomic>
 
+#include "collide.cuh"
 #include "d3q19.cuh"
 #include "lbm_internal.h"
 
@@ -52,15 +53,35 @@ constexpr int kThreadsF = kTX * kTY;
 constexpr int kHalo = 2 * (kTX + 2) + 2 * kTY;   // perimeter cells of the (TX+2) x (TY+2) box
 constexpr int kGroups = 3;                        // halo directions split 7 + 6 + 6 (both components each)
 constexpr int kPer = 14;
-constexpr int Q2 = 2 * Q;
 static_assert(kGroups * kHalo <= kThreadsF, "one halo group per thread");
 
-template <class R>
+// What a plane leaves in shared memory for its collision.  BGK relaxes the
+// populations themselves: 19 pairs per cell, 78 KB per CTA.  The regularized
+// operators need only the second (and third) moments of them, formed in
+// registers while the populations are there: 6 (12) pairs, 25 (49) KB.  At tau
+// = 1 nothing but the densities and the momentum is needed.  The instances were
+// held back by shared-memory traffic (38 eight-byte accesses per cell, MIO
+// throttle) and by the L1 that the stash takes: per step at 256^3 FP32, us,
+// before and after: regularized 1043 -> 878, third-order 1188 -> 916, tau = 1
+// 1020 -> 876 (512^3: 8139 -> 7018, 86 % of the measured copy bandwidth);
+// FP16 deviations regularized 909 -> 701, FP16 relative 1336 -> 936.
+template <int REG> constexpr int kStash = REG == COLL_BGK ? Q : (REG == COLL_EQ ? 0 : RegMoments<float, REG>::n);
+
+// Resident CTAs per SM each instance is compiled for (registers: 128 a thread
+// at 2, 80 at 3).  The 16-bit deviation instances without a BGK stash carry 19
+// registers of raw pairs across the collision and fit 3 (256^3, us per step at
+// 2 / 3: tau = 1 675 / 594, regularized 722 / 701); the FP32 ones carry 38 and
+// spill there (876 / 1003, 878 / 1180).  The relative formats' four planes of
+// reciprocals and the BGK stash leave room for 2.
+template <int S, int REG>
+constexpr int kBlocks = Store<S>::kDev && REG != COLL_BGK ? 3 : 2;
+
+template <int NS>
 struct FusedSmem {
     float2 ring[4][kTY + 2][kTX + 2];      // (rho^1, rho^2) of planes z-1 .. z+2 (+ halo)
-    R hpart[2][kGroups][2][kHalo];         // halo partial densities of the next two planes
-    R mom[2][3][kThreadsF];                // sum_a sum_i c_i f_i of the stashed planes
-    float2 stash[2][Q][kThreadsF];         // pre-collision (f^1_i, f^2_i) of planes z, z+1
+    float hpart[2][kGroups][2][kHalo];     // halo partial densities of the next two planes
+    float mom[2][3][kThreadsF];            // sum_a sum_i c_i f_i of the stashed planes
+    float2 stash[2][NS > 0 ? NS : 1][NS > 0 ? kThreadsF : 1];   // populations or moments of planes z, z+1
     unsigned char hsolid[2][kHalo];        // under a mask: the halo cell is a solid site
 };
 
@@ -71,15 +92,15 @@ struct FusedSmem {
 // the ring is written.
 using InvRing = float2[kTY + 2][kTX + 2];
 
-template <int S>
+template <int S, int REG>
 constexpr size_t smem_bytes()
 {
-    return sizeof(FusedSmem<float>) + (Store<S>::kRel ? 4 * sizeof(InvRing) : 0);
+    return sizeof(FusedSmem<kStash<REG>>) + (Store<S>::kRel ? 4 * sizeof(InvRing) : 0);
 }
 
 // Writes one ring density pair (and, for the *_REL formats, its reciprocals).
-template <int S>
-__device__ __forceinline__ void put_ring(FusedSmem<typename Store<S>::R> &sm, InvRing *inv, int slot, int y, int x,
+template <int S, class SM>
+__device__ __forceinline__ void put_ring(SM &sm, InvRing *inv, int slot, int y, int x,
                                          float r1, float r2)
 {
     sm.ring[slot][y][x] = make_float2(r1, r2);
@@ -171,23 +192,23 @@ __device__ __forceinline__ float2 gather_ref(const typename Store<S>::T *__restr
 template <int S, int I>
 __device__ __forceinline__ void load_dir(const typename Store<S>::T *__restrict__ f, long long N,
                                          float2 rr, const PlaneRef &pr, const Col &c, unsigned lw,
-                                         typename Store<S>::R (&v)[Q2])
+                                         float2 (&v)[Q])
 {
     using R = typename Store<S>::R;
     int d;
     const int e = gather_elem<I>(pr, c, lw, d);
     const unsigned idx = (unsigned)d * (unsigned)N + (unsigned)e;
     if constexpr (Store<S>::kDev)   // the deviation formats compute in d = f - w rho0
-        Store<S>::load2_d(f + 2 * (size_t)idx, v[I], v[Q + I]);
+        Store<S>::load2_d(f + 2 * (size_t)idx, v[I].x, v[I].y);
     else
-        Store<S>::load2(f + 2 * (size_t)idx, w<R>(I) * rr.x, w<R>(I) * rr.y, v[I], v[Q + I]);
+        Store<S>::load2(f + 2 * (size_t)idx, w<R>(I) * rr.x, w<R>(I) * rr.y, v[I].x, v[I].y);
 }
 
 template <int S, int I>
 struct GatherAll {
     __device__ __forceinline__ static void run(const typename Store<S>::T *__restrict__ f, long long N,
                                                float2 rr, const PlaneRef &pr, const Col &c, unsigned lw,
-                                               typename Store<S>::R (&v)[Q2])
+                                               float2 (&v)[Q])
     {
         load_dir<S, I>(f, N, rr, pr, c, lw, v);
         GatherAll<S, I + 1>::run(f, N, rr, pr, c, lw, v);
@@ -197,7 +218,7 @@ template <int S>
 struct GatherAll<S, Q> {
     __device__ __forceinline__ static void run(const typename Store<S>::T *__restrict__, long long,
                                                float2, const PlaneRef &, const Col &, unsigned,
-                                               typename Store<S>::R (&)[Q2]) {}
+                                               float2 (&)[Q]) {}
 };
 
 // The same gather with the pairs kept as stored (one 32-bit word per pair in
@@ -223,50 +244,70 @@ struct GatherRaw<S, Q> {
 
 template <int S>
 __device__ __forceinline__ void decode_all(const typename Store<S>::Raw (&r)[Q], float2 rr,
-                                           typename Store<S>::R (&v)[Q2])
+                                           float2 (&v)[Q])
 {
     using R = typename Store<S>::R;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         if constexpr (Store<S>::kDev)
-            Store<S>::decode2_d(r[i], v[i], v[Q + i]);
+            Store<S>::decode2_d(r[i], v[i].x, v[i].y);
         else
-            Store<S>::decode2(r[i], w<R>(i) * rr.x, w<R>(i) * rr.y, v[i], v[Q + i]);
+            Store<S>::decode2(r[i], w<R>(i) * rr.x, w<R>(i) * rr.y, v[i].x, v[i].y);
     }
 }
 
-// rho^1, rho^2 and momentum of a gathered population set.  The densities are
-// summed in the grouping of the halo partial gathers, (directions 0-6 +
-// directions 7-12) + directions 13-18, so that a cell's density is the same
-// bit for bit whether its own CTA forms it or a neighbouring CTA forms it as a
-// halo cell.  The momentum is summed over opposite pairs,
-// sum_{i odd} c_i (t_i - t_opp(i)) with t_i = f^1_i + f^2_i: the same sum, but
-// each difference of two nearly equal populations is taken first (exactly,
-// in FP32, when they are within a factor of two), so the rounding of the
-// result scales with the momentum, not with the density.
-template <class R>
-__device__ __forceinline__ void sums(const R (&v)[Q2], R &r1, R &r2, R &jx, R &jy, R &jz)
+// Densities and momentum of the *_REL formats in their fixed order (see
+// collide_rel): as sums2, with the two components added before the opposite
+// directions are subtracted.
+__device__ __forceinline__ void sums_rel(const float2 (&v)[Q], float2 &r, float &jx, float &jy, float &jz)
 {
-    R s1 = 0, s2 = 0, ax = 0, ay = 0, az = 0;
-    {
-        R g1[3] = {0, 0, 0}, g2[3] = {0, 0, 0};
+    float2 g[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int k = i < 7 ? 0 : (i < 13 ? 1 : 2);
-            g1[k] += v[i];
-            g2[k] += v[Q + i];
-        }
-        s1 = g1[0] + g1[1] + g1[2];
-        s2 = g2[0] + g2[1] + g2[2];
+    for (int i = 0; i < Q; ++i) {
+        const int k = i < 7 ? 0 : (i < 13 ? 1 : 2);
+        g[k].x += v[i].x;
+        g[k].y += v[i].y;
     }
+    r.x = g[0].x + g[1].x + g[2].x;
+    r.y = g[0].y + g[1].y + g[2].y;
+    float ax = 0, ay = 0, az = 0;
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
-        const R t = (v[i] + v[Q + i]) - (v[i + 1] + v[Q + i + 1]);
+        const float t = (v[i].x + v[i].y) - (v[i + 1].x + v[i + 1].y);
         if (cx(i) == 1) ax += t; else if (cx(i) == -1) ax -= t;
         if (cy(i) == 1) ay += t; else if (cy(i) == -1) ay -= t;
         if (cz(i) == 1) az += t; else if (cz(i) == -1) az -= t;
     }
-    r1 = s1; r2 = s2; jx = ax; jy = ay; jz = az;
+    jx = ax; jy = ay; jz = az;
+}
+
+// Raw moments of the regularized operators in the *_REL formats' fixed order.
+template <int REG>
+__device__ __forceinline__ void moments_rel(const float2 (&v)[Q], RegMoments<float, REG> &mo)
+{
+    float P1[6] = {0, 0, 0, 0, 0, 0}, P2[6] = {0, 0, 0, 0, 0, 0};
+    Third<float> th1, th2;
+    th1.zero(); th2.zero();
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+        const float fa = v[i].x, fb = v[i].y;
+        if (REG == 2) { th1.add(i, fa); th2.add(i, fb); }
+        if (cx(i)) { P1[0] += fa; P2[0] += fb; }
+        if (cy(i)) { P1[1] += fa; P2[1] += fb; }
+        if (cz(i)) { P1[2] += fa; P2[2] += fb; }
+        if (cx(i) && cy(i)) { if (cx(i) == cy(i)) { P1[3] += fa; P2[3] += fb; } else { P1[3] -= fa; P2[3] -= fb; } }
+        if (cx(i) && cz(i)) { if (cx(i) == cz(i)) { P1[4] += fa; P2[4] += fb; } else { P1[4] -= fa; P2[4] -= fb; } }
+        if (cy(i) && cz(i)) { if (cy(i) == cz(i)) { P1[5] += fa; P2[5] += fb; } else { P1[5] -= fa; P2[5] -= fb; } }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) mo.m[k] = make_float2(P1[k], P2[k]);
+    if constexpr (REG == 2) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            mo.m[6 + k] = make_float2(th1.s[k], th2.s[k]);
+            mo.m[9 + k] = make_float2(th1.d[k], th2.d[k]);
+        }
+    }
 }
 
 // Partial gather of one halo cell: directions [D, D1) of both components
@@ -326,46 +367,20 @@ __device__ __forceinline__ void halo_sum(const typename Store<S>::R (&v)[kPer], 
     else HaloRange<S, 13, Q>::sum(v, 0, s0, s1);
 }
 
-// Collision of both components at the thread's interior cell of plane z (the
-// populations come from the stash, densities from the ring, momentum from the
-// moment buffer), forcing term included, result stored at the cell.
-// With the *_REL formats each stored population is coded relative to the
-// density of the cell that reads it next: x + c_i (from the ring), or the
-// cell itself when x + c_i lies behind a wall (lo_wall / hi_wall: plane z is
-// next to the lower / upper wall); the cell's own densities are stored as the
-// reference of the populations it will gather.
-// Under a solid mask, lw is the cell's link word: a solid site (bit 0) stores
-// zero populations (reference densities 1 for the *_REL formats) and zero
-// interaction sums, and a population whose destination x + c_i is solid
-// (bit opp(i)) returns to the cell itself.
+// Collision of the *_REL formats.  A relative code is a function of two rounded
+// densities and amplifies the rounding of the step that produced it (one code
+// of a BF16 population is 2^-9 of it, and a flipped code moves all its readers),
+// so two orders of the same sums part by some 1e-3 within 20 steps.  These
+// instances keep one fixed order of operations, component by component, so
+// that their runs and checkpoints reproduce bit for bit.
 template <int S, int REG, int FORCE>
-__device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ fout, const Phys<typename Store<S>::R> &p,
-                                             const FusedSmem<typename Store<S>::R> &sm, const InvRing *rinv,
-                                             int sl_m, int sl_c, int sl_p,
-                                             int st, long long cell, typename Store<S>::R *__restrict__ s_out,
-                                             bool lo_wall, bool hi_wall, unsigned lw = 0u)
+__device__ __forceinline__ void collide_rel(typename Store<S>::T *__restrict__ fout, const Phys<typename Store<S>::R> &p,
+                                            const FusedSmem<kStash<REG>> &sm, const InvRing *rinv, int sl_m, int sl_c,
+                                            int sl_p, int st, long long cell, typename Store<S>::R *__restrict__ s_out,
+                                            bool lo_wall, bool hi_wall, unsigned lw)
 {
     using R = typename Store<S>::R;
     const int tid = threadIdx.x;
-    if (lw & 1u) {   // solid site
-        typename Store<S>::T *os = fout + 2 * cell;
-        const unsigned n32 = (unsigned)p.N;
-#pragma unroll
-        for (int i = 0; i < Q && fout; ++i) {
-            // zero in every format: the deviation formats code it against w_i rho0,
-            // the relative ones code 0 as 0 whatever their parameter
-            const R ref = Store<S>::kRel ? R(1) : w<R>(i) * R(p.rho0);
-            Store<S>::store2(os + 2 * (size_t)((unsigned)i * n32), R(0), R(0), ref, ref);
-        }
-        if constexpr (Store<S>::kRel) {
-            if (fout) state_ref(fout, p.ref_off)[cell] = make_float2(1.0f, 1.0f);
-        }
-        if (s_out) {
-#pragma unroll
-            for (int k = 0; k < 6; ++k) s_out[(long long)k * p.N + cell] = R(0);
-        }
-        return;
-    }
     const int lx = tid % kTX + 1, ly = tid / kTX + 1;
     const float2 rr = sm.ring[sl_c][ly][lx];
     const R r1 = rr.x, r2 = rr.y;
@@ -432,39 +447,21 @@ __device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ 
     const R rq1 = r1 / R(36), rq2 = r2 / R(36);   // rho w_i = (rho / 36) k_i
     typename Store<S>::T *o = fout + 2 * cell;   // (component 1, component 2) of direction 0
     const unsigned N32 = (unsigned)p.N;
-    const R ref0 = p.rho0;
-    // Deviation formats: the stash holds d = f - w rho0 and the outputs are
-    // stored as f* - w rho0; that adds to each output a constant per unit
-    // weight: -omega rho0 under BGK (keep f = keep d + keep w rho0), -rho0
-    // under the regularized filter (which keeps no f of its own)
-    const R dc1 = Store<S>::kDev ? (REG ? ref0 : p.omega[0] * ref0) : R(0);
-    const R dc2 = Store<S>::kDev ? (REG ? ref0 : p.omega[1] * ref0) : R(0);
-
     // Regularized: second moments of f - f^eq(u): Pi = sum c c f - rho (T0 I + u u)
     R P1[6], P2[6], t1 = 0, t2 = 0;
     Third<R> th1, th2;   // REG = 2: third-order moments of f - f^eq(u)
     if (REG) {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) { P1[k] = 0; P2[k] = 0; }
-        if (REG == 2) { th1.zero(); th2.zero(); }
+        for (int k = 0; k < 6; ++k) { const float2 m = s0[k * kThreadsF]; P1[k] = m.x; P2[k] = m.y; }
+        if (REG == 2) {
 #pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            const float2 fp = s0[i * kThreadsF];
-            const R fa = fp.x, fb = fp.y;
-            if (REG == 2) { th1.add(i, fa); th2.add(i, fb); }
-            if (cx(i)) { P1[0] += fa; P2[0] += fb; }
-            if (cy(i)) { P1[1] += fa; P2[1] += fb; }
-            if (cz(i)) { P1[2] += fa; P2[2] += fb; }
-            if (cx(i) && cy(i)) { if (cx(i) == cy(i)) { P1[3] += fa; P2[3] += fb; } else { P1[3] -= fa; P2[3] -= fb; } }
-            if (cx(i) && cz(i)) { if (cx(i) == cz(i)) { P1[4] += fa; P2[4] += fb; } else { P1[4] -= fa; P2[4] -= fb; } }
-            if (cy(i) && cz(i)) { if (cy(i) == cz(i)) { P1[5] += fa; P2[5] += fb; } else { P1[5] -= fa; P2[5] -= fb; } }
+            for (int k = 0; k < 3; ++k) {
+                const float2 m = s0[(6 + k) * kThreadsF], q = s0[(9 + k) * kThreadsF];
+                th1.s[k] = m.x; th2.s[k] = m.y;
+                th1.d[k] = q.x; th2.d[k] = q.y;
+            }
         }
         const R T0 = R(1) / R(3);
-        if constexpr (Store<S>::kDev) {   // sum_i c_i c_i w_i rho0 = rho0 T0 I
-            const R d = ref0 * T0;
-            P1[0] += d; P1[1] += d; P1[2] += d;
-            P2[0] += d; P2[1] += d; P2[2] += d;
-        }
         P1[0] -= r1 * (T0 + ux * ux); P2[0] -= r2 * (T0 + ux * ux);
         P1[1] -= r1 * (T0 + uy * uy); P2[1] -= r2 * (T0 + uy * uy);
         P1[2] -= r1 * (T0 + uz * uz); P2[2] -= r2 * (T0 + uz * uz);
@@ -484,7 +481,6 @@ __device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ 
     }
     // rest population (k_0 = 12)
     {
-        const R w0 = w<R>(0);
         R o1, o2v;
         if (!REG) {
             const float2 f0 = s0[0];
@@ -498,15 +494,9 @@ __device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ 
             o1 += cf1 * (R(-1) * uF1);
             o2v += cf2 * (R(-1) * uF2);
         }
-        if constexpr (Store<S>::kRel) {
-            const float2 iv = rinv[sl_c][ly][lx];   // 1/rho of the cell itself; 1/w_0 = 3
-            Store<S>::store2(o, o1, o2v, R(3) * iv.x, R(3) * iv.y);
-            state_ref(fout, p.ref_off)[cell] = rr;
-        } else if constexpr (Store<S>::kDev) {
-            Store<S>::store2_d(o, o1 - w0 * dc1, o2v - w0 * dc2);
-        } else {
-            Store<S>::store2(o, o1, o2v, w0 * ref0, w0 * ref0);
-        }
+        const float2 iv = rinv[sl_c][ly][lx];   // 1/rho of the cell itself; 1/w_0 = 3
+        Store<S>::store2(o, o1, o2v, R(3) * iv.x, R(3) * iv.y);
+        state_ref(fout, p.ref_off)[cell] = rr;
     }
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
@@ -523,7 +513,6 @@ __device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ 
             const R Eu = Au + R(4.5) * cu * cu, Ou = cu * (Bu + R(4.5) * cu * cu);
             R P1e = rw1 * (E1 - keep1 * Eu), M1 = rw1 * (O1 - keep1 * Ou);
             R P2e = rw2 * (E2 - keep2 * Eu), M2 = rw2 * (O2 - keep2 * Ou);
-            if constexpr (Store<S>::kDev) { P1e -= w<R>(i) * dc1; P2e -= w<R>(i) * dc2; }
             const float2 fp = s0[i * kThreadsF], fm = s0[(i + 1) * kThreadsF];
             o1p = P1e + M1 + keep1 * fp.x;
             o1m = P1e - M1 + keep1 * fm.x;
@@ -540,7 +529,6 @@ __device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ 
             if (cy(i) && cz(i)) { const R sg = cy(i) == cz(i) ? R(2) : R(-2); cc1 += sg * P1[5]; cc2 += sg * P2[5]; }
             R n1 = keep1 * (R(k36(i)) * R(0.125)) * (cc1 - t1);
             R n2 = keep2 * (R(k36(i)) * R(0.125)) * (cc2 - t2);
-            if constexpr (Store<S>::kDev) { n1 -= w<R>(i) * dc1; n2 -= w<R>(i) * dc2; }
             // third-order part, odd in c_i: + for i, - for opp(i)
             const R m1 = REG == 2 ? keep1 * th1.odd(i) : R(0);
             const R m2 = REG == 2 ? keep2 * th2.odd(i) : R(0);
@@ -558,36 +546,110 @@ __device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ 
             o2p += e2 + d2; o2m += e2 - d2;
         }
         const size_t ip = 2 * (size_t)((unsigned)i * N32), im = 2 * (size_t)((unsigned)(i + 1) * N32);
+        // destinations: x + c_i for i, x - c_i for opp(i), or x across a wall
+        const bool wp = (cz(i) == -1 && lo_wall) || (cz(i) == 1 && hi_wall) || ((lw >> (i + 1)) & 1u);
+        const bool wm = (cz(i) == 1 && lo_wall) || (cz(i) == -1 && hi_wall) || ((lw >> i) & 1u);
+        const int slp = cz(i) == -1 ? sl_m : (cz(i) == 1 ? sl_p : sl_c);
+        const int slm = cz(i) == -1 ? sl_p : (cz(i) == 1 ? sl_m : sl_c);
+        const float2 dp = wp ? rinv[sl_c][ly][lx] : rinv[slp][ly + cy(i)][lx + cx(i)];
+        const float2 dm = wm ? rinv[sl_c][ly][lx] : rinv[slm][ly - cy(i)][lx - cx(i)];
+        const R sk = R(36 / k36(i));   // 1 / w_i: the code parameter is 1 / (w_i rho~)
+        Store<S>::store2(o + ip, o1p, o2p, sk * dp.x, sk * dp.y);
+        Store<S>::store2(o + im, o1m, o2m, sk * dm.x, sk * dm.y);
+    }
+}
+
+// Collision of both components at the thread's interior cell of plane z (the
+// populations come from the stash, densities from the ring, momentum from the
+// moment buffer), forcing term included, result stored at the cell.
+// With the *_REL formats each stored population is coded relative to the
+// density of the cell that reads it next: x + c_i (from the ring), or the
+// cell itself when x + c_i lies behind a wall (lo_wall / hi_wall: plane z is
+// next to the lower / upper wall); the cell's own densities are stored as the
+// reference of the populations it will gather.
+// Under a solid mask, lw is the cell's link word: a solid site (bit 0) stores
+// zero populations (reference densities 1 for the *_REL formats) and zero
+// interaction sums, and a population whose destination x + c_i is solid
+// (bit opp(i)) returns to the cell itself.
+template <int S, int REG, int FORCE>
+__device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ fout, const Phys<typename Store<S>::R> &p,
+                                             const FusedSmem<kStash<REG>> &sm, const InvRing *rinv,
+                                             int sl_m, int sl_c, int sl_p,
+                                             int st, long long cell, typename Store<S>::R *__restrict__ s_out,
+                                             bool lo_wall, bool hi_wall, unsigned lw = 0u)
+{
+    using R = typename Store<S>::R;
+    const int tid = threadIdx.x;
+    if (lw & 1u) {   // solid site
+        typename Store<S>::T *os = fout + 2 * cell;
+        const unsigned n32 = (unsigned)p.N;
+#pragma unroll
+        for (int i = 0; i < Q && fout; ++i) {
+            // zero in every format: the deviation formats code it against w_i rho0,
+            // the relative ones code 0 as 0 whatever their parameter
+            const R ref = Store<S>::kRel ? R(1) : w<R>(i) * R(p.rho0);
+            Store<S>::store2(os + 2 * (size_t)((unsigned)i * n32), R(0), R(0), ref, ref);
+        }
         if constexpr (Store<S>::kRel) {
-            // destinations: x + c_i for i, x - c_i for opp(i), or x across a wall
-            const bool wp = (cz(i) == -1 && lo_wall) || (cz(i) == 1 && hi_wall) || ((lw >> (i + 1)) & 1u);
-            const bool wm = (cz(i) == 1 && lo_wall) || (cz(i) == -1 && hi_wall) || ((lw >> i) & 1u);
-            const int slp = cz(i) == -1 ? sl_m : (cz(i) == 1 ? sl_p : sl_c);
-            const int slm = cz(i) == -1 ? sl_p : (cz(i) == 1 ? sl_m : sl_c);
-            const float2 dp = wp ? rinv[sl_c][ly][lx] : rinv[slp][ly + cy(i)][lx + cx(i)];
-            const float2 dm = wm ? rinv[sl_c][ly][lx] : rinv[slm][ly - cy(i)][lx - cx(i)];
-            const R sk = R(36 / k36(i));   // 1 / w_i: the code parameter is 1 / (w_i rho~)
-            Store<S>::store2(o + ip, o1p, o2p, sk * dp.x, sk * dp.y);
-            Store<S>::store2(o + im, o1m, o2m, sk * dm.x, sk * dm.y);
-        } else if constexpr (Store<S>::kDev) {
-            Store<S>::store2_d(o + ip, o1p, o2p);
-            Store<S>::store2_d(o + im, o1m, o2m);
+            if (fout) state_ref(fout, p.ref_off)[cell] = make_float2(1.0f, 1.0f);
+        }
+        if (s_out) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) s_out[(long long)k * p.N + cell] = R(0);
+        }
+        return;
+    }
+    if constexpr (Store<S>::kRel) {
+        collide_rel<S, REG, FORCE>(fout, p, sm, rinv, sl_m, sl_c, sl_p, st, cell, s_out, lo_wall, hi_wall, lw);
+        return;
+    } else {
+    const int lx = tid % kTX + 1, ly = tid / kTX + 1;
+    const float2 rr = sm.ring[sl_c][ly][lx];
+    // S^b = sum_{i != 0} w_i c_i rho^b(x + c_i)  (Eq. 7; ghost planes carry Eq. 13's rho')
+    float2 Sb[3];
+    interaction2<float>([&](int i) {
+        const int slp = cz(i) == -1 ? sl_m : (cz(i) == 1 ? sl_p : sl_c);
+        const int slm = cz(i) == -1 ? sl_p : (cz(i) == 1 ? sl_m : sl_c);
+        return vsub(sm.ring[slp][ly + cy(i)][lx + cx(i)], sm.ring[slm][ly - cy(i)][lx - cx(i)]);
+    }, Sb);
+    if (s_out) {   // interaction sums of this step (reverse-mode replay)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            s_out[(long long)d * p.N + cell] = Sb[d].x;
+            s_out[(long long)(3 + d) * p.N + cell] = Sb[d].y;
+        }
+    }
+    if (!fout) return;   // the interaction sums alone (the last step of a replayed segment)
+    const R inv = R(1) / (rr.x + rr.y);
+    const R ux = sm.mom[st][0][tid] * inv, uy = sm.mom[st][1][tid] * inv, uz = sm.mom[st][2][tid] * inv;
+    const float2 *s0 = &sm.stash[st][0][tid];
+    RegMoments<float, REG> mo;
+#pragma unroll
+    for (int k = 0; k < RegMoments<float, REG>::n; ++k) mo.m[k] = s0[k * kThreadsF];
+    typename Store<S>::T *o = fout + 2 * cell;   // (component 1, component 2) of direction 0
+    const unsigned N32 = (unsigned)p.N;
+    const R ref0 = p.rho0;
+    auto get = [&](int i) { return s0[i * kThreadsF]; };
+    auto put = [&](int i, float2 f) {
+        typename Store<S>::T *q = o + 2 * (size_t)((unsigned)i * N32);
+        if constexpr (Store<S>::kDev) {
+            Store<S>::store2_d(q, f.x, f.y);
         } else {
             const R ref = w<R>(i) * ref0;
-            Store<S>::store2(o + ip, o1p, o2p, ref, ref);
-            Store<S>::store2(o + im, o1m, o2m, ref, ref);
+            Store<S>::store2(q, f.x, f.y, ref, ref);
         }
+    };
+    collide2<float, REG, FORCE, Store<S>::kDev>(p, rr, inv, ux, uy, uz, Sb, mo, get, put);
     }
 }
 
 // Interior part of plane zp for this thread's column: rho^1, rho^2 into ring
 // slot `slot`; when st >= 0 the populations and momentum into stash slot st.
 // A solid site of a mask (solid) presents its wall density wd instead.
-template <int S>
-__device__ __forceinline__ void interior_plane(const typename Store<S>::T *__restrict__ f,
-                                               const Phys<typename Store<S>::R> &p, FusedSmem<typename Store<S>::R> &sm,
+template <int S, int REG>
+__device__ __forceinline__ void interior_plane(const Phys<typename Store<S>::R> &p, FusedSmem<kStash<REG>> &sm,
                                                InvRing *inv,
-                                               int slot, int st, const PlaneRef &pr, const typename Store<S>::R (&v)[Q2],
+                                               int slot, int st, const PlaneRef &pr, const float2 (&v)[Q],
                                                bool solid = false, float2 wd = make_float2(0.f, 0.f))
 {
     using R = typename Store<S>::R;
@@ -598,16 +660,26 @@ __device__ __forceinline__ void interior_plane(const typename Store<S>::T *__res
         r1 = wd.x;
         r2 = wd.y;
     } else if (!pr.constant) {
-        R a1, a2, jx, jy, jz;
-        sums(v, a1, a2, jx, jy, jz);
-        if constexpr (Store<S>::kDev) { a1 += p.rho0; a2 += p.rho0; }   // sum_i w_i rho0 = rho0
+        float2 a;
+        R jx, jy, jz;
+        if constexpr (Store<S>::kRel) sums_rel(v, a, jx, jy, jz);
+        else sums2<float>(v, a, jx, jy, jz);
+        if constexpr (Store<S>::kDev) { a.x += p.rho0; a.y += p.rho0; }   // sum_i w_i rho0 = rho0
         if (pr.ghost) {
-            r1 += a1; r2 += a2;
+            r1 += a.x; r2 += a.y;
         } else {
-            r1 = a1; r2 = a2;
+            r1 = a.x; r2 = a.y;
             if (st >= 0) {
+                if constexpr (REG == COLL_BGK) {
 #pragma unroll
-                for (int k = 0; k < Q; ++k) sm.stash[st][k][tid] = make_float2(v[k], v[Q + k]);
+                    for (int k = 0; k < Q; ++k) sm.stash[st][k][tid] = v[k];
+                } else if constexpr (REG != COLL_EQ) {
+                    RegMoments<float, REG> mo;
+                    if constexpr (Store<S>::kRel) moments_rel<REG>(v, mo);
+                    else mo.of(v);
+#pragma unroll
+                    for (int k = 0; k < RegMoments<float, REG>::n; ++k) sm.stash[st][k][tid] = mo.m[k];
+                }
                 sm.mom[st][0][tid] = jx; sm.mom[st][1][tid] = jy; sm.mom[st][2][tid] = jz;
             }
         }
@@ -618,8 +690,8 @@ __device__ __forceinline__ void interior_plane(const typename Store<S>::T *__res
 // Halo densities of a plane in ring slot `slot` from the partials of the
 // population groups (mask: the kernel runs a solid mask, whose solid halo
 // cells are marked in hsolid).
-template <int S, class R>
-__device__ __forceinline__ void halo_combine(const Phys<R> &p, FusedSmem<R> &sm, InvRing *inv, int slot, int hs,
+template <int S, class SM, class R>
+__device__ __forceinline__ void halo_combine(const Phys<R> &p, SM &sm, InvRing *inv, int slot, int hs,
                                              const PlaneRef &pr, int h, int hx, int hy, bool mask = false)
 {
     R r1, r2;
@@ -646,7 +718,7 @@ __device__ __forceinline__ void halo_combine(const Phys<R> &p, FusedSmem<R> &sm,
 // site puts its wall density into the ring (a solid halo cell through its
 // first partial, the others zero) and stores zero populations.
 template <int S, int REG, bool WALLZ, bool MASK, int FORCE>
-__global__ void __launch_bounds__(kThreadsF, 2)
+__global__ void __launch_bounds__(kThreadsF, kBlocks<S, REG>)
 k_step_fused(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T *__restrict__ fout,
              Phys<typename Store<S>::R> p, int ntx, int lz, typename Store<S>::R *__restrict__ s_out,
              const unsigned *__restrict__ links, const float2 *__restrict__ wrho)
@@ -655,8 +727,9 @@ k_step_fused(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T 
     static_assert(sizeof(R) == sizeof(float), "the fused step runs FP32 arithmetic");
     static_assert(!(MASK && WALLZ), "a solid mask needs a lattice periodic along z");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    FusedSmem<R> &sm = *reinterpret_cast<FusedSmem<R> *>(smem_raw);
-    InvRing *inv = reinterpret_cast<InvRing *>(smem_raw + sizeof(FusedSmem<R>));   // *_REL formats only
+    using SM = FusedSmem<kStash<REG>>;
+    SM &sm = *reinterpret_cast<SM *>(smem_raw);
+    InvRing *inv = reinterpret_cast<InvRing *>(smem_raw + sizeof(SM));   // *_REL formats only
     const int tid = threadIdx.x;
     const int tx0 = (blockIdx.x % ntx) * kTX;
     const int ty0 = (blockIdx.x / ntx) * kTY;
@@ -729,10 +802,10 @@ k_step_fused(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T 
         const PlaneRef pr = plane_ref<WALLZ>(p, q);
         const unsigned lw = link_of(pr, ci);
         if (q == z0) lwA = lw;
-        R v[Q2];
+        float2 v[Q];
         if (!pr.constant) GatherAll<S, 0>::run(fin, p.N, gather_ref<S>(fin, p, pr, ci), pr, ci, lw, v);
         const bool sol = MASK && (lw & 1u);
-        interior_plane<S>(fin, p, sm, inv, q - z0 + 1, q == z0 ? 0 : -1, pr, v, sol,
+        interior_plane<S, REG>(p, sm, inv, q - z0 + 1, q == z0 ? 0 : -1, pr, v, sol,
                           sol ? wall_rho(pr, ci) : make_float2(0.f, 0.f));
         if (tid < kHalo) {
             R r1 = p.rho_s[0], r2 = p.rho_s[1];
@@ -742,12 +815,12 @@ k_step_fused(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T 
                 r1 = wd.x;
                 r2 = wd.y;
             } else if (!pr.constant) {
-                R hv[Q2];
+                float2 hv[Q], a;
                 GatherAll<S, 0>::run(fin, p.N, gather_ref<S>(fin, p, pr, ch), pr, ch, hl, hv);
-                R a1, a2, jx, jy, jz;
-                sums(hv, a1, a2, jx, jy, jz);
-                if constexpr (Store<S>::kDev) { a1 += p.rho0; a2 += p.rho0; }
-                if (pr.ghost) { r1 += a1; r2 += a2; } else { r1 = a1; r2 = a2; }
+                R jx, jy, jz;
+                sums2<float>(hv, a, jx, jy, jz);
+                if constexpr (Store<S>::kDev) { a.x += p.rho0; a.y += p.rho0; }
+                if (pr.ghost) { r1 += a.x; r2 += a.y; } else { r1 = a.x; r2 = a.y; }
             }
             put_ring<S>(sm, inv, q - z0 + 1, hy, hx, r1, r2);
         }
@@ -782,7 +855,7 @@ k_step_fused(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T 
     // measured to gain from it), as stored (rv, with the reference densities
     // rrv), which keeps 19 registers instead of 38 live across the collision.
     constexpr bool kRaw = sizeof(typename Store<S>::Raw) < sizeof(float2) && !WALLZ && !MASK;
-    R v[Q2];
+    float2 v[Q];
     typename Store<S>::Raw rv[Q];
     float2 rrv = make_float2(0.f, 0.f);
     unsigned lwB, lwC = 0, hlw = 0;   // link words: column at z+1, z+2; halo task cell at z+2
@@ -827,7 +900,7 @@ k_step_fused(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T 
         if constexpr (kRaw) {
             if (!pr1.constant) decode_all<S>(rv, rrv, v);
         }
-        interior_plane<S>(fin, p, sm, inv, s_p, z + 1 < z1 ? ((k + 1) & 1) : -1, pr1, v, sol, wdB);
+        interior_plane<S, REG>(p, sm, inv, s_p, z + 1 < z1 ? ((k + 1) & 1) : -1, pr1, v, sol, wdB);
         if (need2 && has_halo) {
             R s1 = 0, s2 = 0;
             if (hsol) {
@@ -898,11 +971,11 @@ cudaError_t launch_inst(dim3 grid, cudaStream_t s, const typename Store<S>::T *f
     const bool cached = dev >= 0 && dev < kMaxAttrDevices;
     if (!cached || !attr_set[dev].load(std::memory_order_acquire)) {
         e = cudaFuncSetAttribute((const void *)k_step_fused<S, REG, WALLZ, MASK, FORCE>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<S>());
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<S, REG>());
         if (e != cudaSuccess) return e;
         if (cached) attr_set[dev].store(1, std::memory_order_release);
     }
-    k_step_fused<S, REG, WALLZ, MASK, FORCE><<<grid, kThreadsF, smem_bytes<S>(), s>>>(fi, fo, p, ntx, lz, s_out, links, wrho);
+    k_step_fused<S, REG, WALLZ, MASK, FORCE><<<grid, kThreadsF, smem_bytes<S, REG>(), s>>>(fi, fo, p, ntx, lz, s_out, links, wrho);
     return cudaSuccess;
 }
 
@@ -923,6 +996,10 @@ cudaError_t launch_coll(const HostPhys &h, int lz, dim3 grid, cudaStream_t s, co
                         typename Store<S>::T *fo, const Phys<typename Store<S>::R> &p, int ntx,
                         typename Store<S>::R *s_out)
 {
+    if constexpr (!Store<S>::kRel) {   // tau = 1: the three operators coincide
+        if (p.omega[0] == 1.0f && p.omega[1] == 1.0f)
+            return launch_geom<S, COLL_EQ, FORCE>(h, lz, grid, s, fi, fo, p, ntx, s_out);
+    }
     switch (h.collision) {
     case LBM_REGULARIZED: return launch_geom<S, 1, FORCE>(h, lz, grid, s, fi, fo, p, ntx, s_out);
     case LBM_REGULARIZED3: return launch_geom<S, 2, FORCE>(h, lz, grid, s, fi, fo, p, ntx, s_out);
