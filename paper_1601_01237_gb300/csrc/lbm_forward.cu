@@ -19,6 +19,7 @@
 
 #include <atomic>
 
+#include "collide.cuh"
 #include "d3q19.cuh"
 #include "lbm_internal.h"
 
@@ -314,6 +315,143 @@ k_collide(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T *__
     }
 }
 
+// ---------------------------------------------------------------------------
+// The two-kernel step in FP64, one component of a cell per lane (LaneF64 of
+// collide.cuh) and 32-bit indices (19 N < 2^32).  FP64 arithmetic is scarce on
+// this GPU: a scheduler retires one FP64 warp instruction per 64 cycles, so
+// the step is bound by the FP64 instructions of the busiest scheduler at every
+// size (34^3: 37 us of them against 3.5 us of memory traffic).  Hence
+//   - small CTAs of half-cell lanes: 256-thread CTAs of whole cells put all of a
+//     34^3 lattice on 2 CTAs per busy SM, and a 64^2 one on 16 SMs;
+//   - the densities are formed once, in the density pass, and the collision
+//     reads its own back instead of summing them again;
+//   - the seven-operations-per-pair form of the collision;
+//   - warps inside a wall do no arithmetic.
+// Of CTAs of 32, 64 and 128 threads the smallest leaves the least imbalance
+// (34^3 39.5 / 42.7 / 42.7 us per step).  us per step before and now: 1 x 64 x 64
+// 39.8 / 8.8, 1 x 300 x 300 115 / 60, 34^3 periodic 94.7 / 39.5, 128^3 2046 / 1225.
+constexpr int kThreads64 = 32;
+
+struct Nbr32 {
+    unsigned cell;
+    unsigned xo[3], yo[3], zo[3];
+    bool zlo, zhi;   // z - 1 (z + 1) is a wall site
+};
+
+template <class P>
+__device__ __forceinline__ Nbr32 neighbours32(const P &p, unsigned cell)
+{
+    const unsigned nx = (unsigned)p.nx, ny = (unsigned)p.ny, nz = (unsigned)p.nz, plane = nx * ny;
+    const unsigned z = cell / plane, rem = cell - z * plane, y = rem / nx, x = rem - y * nx;
+    Nbr32 n;
+    n.cell = cell;
+    n.xo[0] = x == 0 ? nx - 1 : x - 1;
+    n.xo[1] = x;
+    n.xo[2] = x == nx - 1 ? 0 : x + 1;
+    n.yo[0] = (y == 0 ? ny - 1 : y - 1) * nx;
+    n.yo[1] = y * nx;
+    n.yo[2] = (y == ny - 1 ? 0 : y + 1) * nx;
+    n.zo[0] = (z == 0 ? nz - 1 : z - 1) * plane;
+    n.zo[1] = z * plane;
+    n.zo[2] = (z == nz - 1 ? 0 : z + 1) * plane;
+    n.zlo = p.wall_z && z == 0;
+    n.zhi = p.wall_z && z == nz - 1;
+    return n;
+}
+
+__device__ __forceinline__ void gather64(const double *__restrict__ f, const PhysF<double> &p, const Nbr32 &n,
+                                         unsigned lf, int a, double (&v)[Q])
+{
+    const unsigned N32 = (unsigned)p.N;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const unsigned src = n.zo[1 - cz(i)] + n.yo[1 - cy(i)] + n.xo[1 - cx(i)];
+        const bool wall = (cz(i) == 1 && n.zlo) || (cz(i) == -1 && n.zhi) || (i != 0 && ((lf >> i) & 1u));
+        v[i] = __ldg(f + 2 * (size_t)(wall ? (unsigned)opp(i) * N32 + n.cell : (unsigned)i * N32 + src) + a);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads64)
+k_density64(const double *__restrict__ f, double *__restrict__ rho, PhysF<double> p)
+{
+    const unsigned t = blockIdx.x * kThreads64 + threadIdx.x, cell = t >> 1;
+    if (cell >= (unsigned)p.N) return;
+    const unsigned lf = p.links ? __ldg(p.links + cell) : 0u;
+    const int a = (int)(t & 1u);
+    const Nbr32 n = neighbours32(p, cell);
+    if (lf & 1u) return;   // k_wall_rho64 writes the solid sites that are read
+    double v[Q];
+    gather64(f, p, n, lf, a, v);
+    rho[(size_t)a * (unsigned)p.N + cell] = density(v);
+}
+
+// k_wall_rho over the solid sites next to fluid, the only ones that are read,
+// one component per lane.
+__global__ void __launch_bounds__(kThreads64)
+k_wall_rho64(double *__restrict__ rho, PhysF<double> p, const unsigned *__restrict__ sites, unsigned n_sites)
+{
+    const unsigned t = blockIdx.x * kThreads64 + threadIdx.x;
+    if ((t >> 1) >= n_sites) return;
+    const int a = (int)(t & 1u);
+    const Nbr32 n = neighbours32(p, sites[t >> 1]);
+    double *r = rho + (size_t)a * (unsigned)p.N;
+    double num = 0;
+    int den36 = 0;
+    if (p.wall_mirror) {
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+            const unsigned nb = n.zo[1 + cz(i)] + n.yo[1 + cy(i)] + n.xo[1 + cx(i)];
+            if (__ldg(p.solid + nb)) continue;
+            num += (double)k36(i) * r[nb];
+            den36 += k36(i);
+        }
+    }
+    r[n.cell] = (den36 ? num / (double)den36 : 0.0) + p.rho_s[a];
+}
+
+template <int KIND, int FORCE>
+__global__ void __launch_bounds__(kThreads64)
+k_collide64(const double *__restrict__ fin, double *__restrict__ fout, const double *__restrict__ rho, PhysF<double> p)
+{
+    const unsigned t = blockIdx.x * kThreads64 + threadIdx.x, N32 = (unsigned)p.N;
+    // both lanes of every cell stay for the shuffles; lanes past the end repeat the last cell
+    const unsigned cell = min(t >> 1, N32 - 1u);
+    const bool store = (t >> 1) < N32;
+    const LaneF64 c{(int)(t & 1u)};
+    const Nbr32 n = neighbours32(p, cell);
+    const unsigned lf = p.links ? __ldg(p.links + cell) : 0u;
+    const bool solid = lf & 1u;
+    double *o = fout + 2 * (size_t)cell + c.a;
+    if (__all_sync(0xffffffffu, solid)) {   // inside a wall: no arithmetic
+#pragma unroll
+        for (int i = 0; i < Q && store; ++i) o[2 * (size_t)((unsigned)i * N32)] = 0.0;
+        return;
+    }
+    double f[Q];
+    gather64(fin, p, n, lf, c.a, f);
+    double r = __ldg(rho + (size_t)c.a * N32 + cell);
+    if (solid) r = 1.0;   // (nothing of a solid site's arithmetic is kept)
+    const double *ro = rho + (size_t)(1 - c.a) * N32;
+    const double rs = c.of(p.rho_s[1], p.rho_s[0]);   // of the other component
+    double So[3];
+    auto at = [&](int dx, int dy, int dz) {
+        const bool wall = (dz == -1 && n.zlo) || (dz == 1 && n.zhi);
+        if (wall) return p.wall_mirror ? rs + __ldg(ro + n.zo[1] + n.yo[1 + dy] + n.xo[1 + dx]) : rs;
+        return __ldg(ro + n.zo[1 + dz] + n.yo[1 + dy] + n.xo[1 + dx]);
+    };
+    interaction<LaneF64>([&](int i) { return at(cx(i), cy(i), cz(i)) - at(-cx(i), -cy(i), -cz(i)); }, So);
+    double jx, jy, jz;
+    momentum(c, f, jx, jy, jz);
+    RegMoments<LaneF64, KIND> mom;
+    mom.of(f);
+    const double inv = 1.0 / c.both(r);
+    auto get = [&](int i) { return f[i]; };
+    auto put = [&](int i, double v) {
+        if (store) o[2 * (size_t)((unsigned)i * N32)] = solid ? 0.0 : v;
+    };
+    collide_cell<LaneF64, KIND, FORCE, false>(c, p, r, inv, jx * inv, jy * inv, jz * inv, So, mom, get, put);
+}
+
 // Rest-state values of one cell, formed once per cell in FP64 and rounded to
 // the arithmetic type: rho^a w for the three weight classes (w = 1/3, 1/18,
 // 1/36) and rho^a itself, at slot (2 q + a) N + c (q = 0, 1, 2, 3).  The
@@ -575,6 +713,11 @@ PhysF<R> make_phys(const HostPhys &h)
 
 inline unsigned grid_for(long long N) { return (unsigned)((N + kThreads - 1) / kThreads); }
 
+// FP64 lattices that the half-cell kernels take: 32-bit element indices (and,
+// with a mask, the lists of its boundary, which lbm_set_solid makes).
+inline bool lanes64(const HostPhys &h) { return (long long)Q * h.N < (1LL << 32) && (!h.links || h.bsolid); }
+inline unsigned grid64(long long cells) { return (unsigned)((2 * cells + kThreads64 - 1) / kThreads64); }
+
 // Density pass: rho^a of every fluid cell, then (with a mask) the densities
 // the solid sites present to Eq. 13.
 template <int S>
@@ -582,6 +725,14 @@ void density_pass(const HostPhys &h, const typename Store<S>::T *f, typename Sto
 {
     using R = typename Store<S>::R;
     const PhysF<R> p = make_phys<R>(h);
+    if constexpr (S == ST_F64) {
+        if (lanes64(h)) {
+            k_density64<<<grid64(h.N), kThreads64, 0, s>>>(f, rho, p);
+            if (h.solid && h.n_bsolid > 0)
+                k_wall_rho64<<<grid64(h.n_bsolid), kThreads64, 0, s>>>(rho, p, h.bsolid, (unsigned)h.n_bsolid);
+            return;
+        }
+    }
     k_density<S><<<grid_for(h.N), kThreads, 0, s>>>(f, rho, p);
     if (h.solid) k_wall_rho<R><<<grid_for(h.N), kThreads, 0, s>>>(rho, p);
 }
@@ -597,6 +748,24 @@ cudaError_t step_split_t(const HostPhys &h, const void *fin, void *fout, void *r
     if (ev) cudaEventRecord(ev[0], s);
     density_pass<S>(h, (const T *)fin, (R *)rho, s);
     if (ev) cudaEventRecord(ev[1], s);
+    if constexpr (S == ST_F64) {
+        if (lanes64(h)) {
+            const unsigned g64 = grid64(h.N);
+            const bool guo = h.forcing == FORCE_GUO;
+#define LBM_COLLIDE64(K_)                                                                                            \
+    do {                                                                                                             \
+        if (guo) k_collide64<K_, FORCE_GUO><<<g64, kThreads64, 0, s>>>((const T *)fin, (T *)fout, (const R *)rho, p); \
+        else k_collide64<K_, FORCE_EDM><<<g64, kThreads64, 0, s>>>((const T *)fin, (T *)fout, (const R *)rho, p);     \
+    } while (0)
+            if (h.tau[0] == 1.0 && h.tau[1] == 1.0) LBM_COLLIDE64(COLL_EQ);
+            else if (h.collision == LBM_REGULARIZED) LBM_COLLIDE64(COLL_REG);
+            else if (h.collision == LBM_REGULARIZED3) LBM_COLLIDE64(COLL_REG3);
+            else LBM_COLLIDE64(COLL_BGK);
+#undef LBM_COLLIDE64
+            if (ev) cudaEventRecord(ev[2], s);
+            return cudaGetLastError();
+        }
+    }
 #define LBM_COLLIDE(REG_, F_) k_collide<S, REG_, F_><<<g, kThreads, 0, s>>>((const T *)fin, (T *)fout, (const R *)rho, p)
     const int reg = h.collision == LBM_REGULARIZED ? 1 : (h.collision == LBM_REGULARIZED3 ? 2 : 0);
     if (h.forcing == FORCE_GUO) {

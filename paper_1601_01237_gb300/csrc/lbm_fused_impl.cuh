@@ -39,6 +39,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "collide.cuh"
 #include "d3q19.cuh"
@@ -65,16 +66,29 @@ static_assert(kGroups * kHalo <= kThreadsF, "one halo group per thread");
 // before and after: regularized 1043 -> 878, third-order 1188 -> 916, tau = 1
 // 1020 -> 876 (512^3: 8139 -> 7018, 86 % of the measured copy bandwidth);
 // FP16 deviations regularized 909 -> 701, FP16 relative 1336 -> 936.
-template <int REG> constexpr int kStash = REG == COLL_BGK ? Q : (REG == COLL_EQ ? 0 : RegMoments<float, REG>::n);
+template <int REG> constexpr int kStash = REG == COLL_BGK ? Q : (REG == COLL_EQ ? 0 : RegMoments<PairF32, REG>::n);
+
+// Whether an instance carries the next plane's gathers across the collision as
+// stored (see k_step_fused).
+template <int S, int REG, bool WALLZ, bool MASK>
+constexpr bool kRawCarry = sizeof(typename Store<S>::Raw) < sizeof(float2) &&
+                           ((Store<S>::kDev && REG != COLL_BGK) || (!WALLZ && !MASK));
 
 // Resident CTAs per SM each instance is compiled for (registers: 128 a thread
 // at 2, 80 at 3).  The 16-bit deviation instances without a BGK stash carry 19
 // registers of raw pairs across the collision and fit 3 (256^3, us per step at
 // 2 / 3: tau = 1 675 / 594, regularized 722 / 701); the FP32 ones carry 38 and
-// spill there (876 / 1003, 878 / 1180).  The relative formats' four planes of
+// spill there (876 / 1003, 878 / 1180), and so do the 16-bit ones with z walls
+// (192 x 256 x 256, regularized: 585 / 718).  The relative formats' four planes of
 // reciprocals and the BGK stash leave room for 2.
+template <int S, int REG, bool WALLZ>
+constexpr int kBlocks = Store<S>::kDev && REG != COLL_BGK ? (WALLZ ? 2 : 3) : 2;
+
+// Instances that keep the component-by-component order of operations (see
+// collide_scalar): the relative formats, and the deviation formats' BGK, which
+// the packed form does not speed up (256^3 FP16, us per step: 820, packed 877).
 template <int S, int REG>
-constexpr int kBlocks = Store<S>::kDev && REG != COLL_BGK ? 3 : 2;
+constexpr bool kScalar = Store<S>::kRel || (Store<S>::kDev && REG == COLL_BGK);
 
 template <int NS>
 struct FusedSmem {
@@ -256,10 +270,9 @@ __device__ __forceinline__ void decode_all(const typename Store<S>::Raw (&r)[Q],
     }
 }
 
-// Densities and momentum of the *_REL formats in their fixed order (see
-// collide_rel): as sums2, with the two components added before the opposite
+// Densities and momentum in the fixed order of collide_scalar: as density and momentum, with the two components added before the opposite
 // directions are subtracted.
-__device__ __forceinline__ void sums_rel(const float2 (&v)[Q], float2 &r, float &jx, float &jy, float &jz)
+__device__ __forceinline__ void sums_scalar(const float2 (&v)[Q], float2 &r, float &jx, float &jy, float &jz)
 {
     float2 g[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
@@ -281,9 +294,9 @@ __device__ __forceinline__ void sums_rel(const float2 (&v)[Q], float2 &r, float 
     jx = ax; jy = ay; jz = az;
 }
 
-// Raw moments of the regularized operators in the *_REL formats' fixed order.
+// Raw moments of the regularized operators in that order.
 template <int REG>
-__device__ __forceinline__ void moments_rel(const float2 (&v)[Q], RegMoments<float, REG> &mo)
+__device__ __forceinline__ void moments_scalar(const float2 (&v)[Q], RegMoments<PairF32, REG> &mo)
 {
     float P1[6] = {0, 0, 0, 0, 0, 0}, P2[6] = {0, 0, 0, 0, 0, 0};
     Third<float> th1, th2;
@@ -367,16 +380,16 @@ __device__ __forceinline__ void halo_sum(const typename Store<S>::R (&v)[kPer], 
     else HaloRange<S, 13, Q>::sum(v, 0, s0, s1);
 }
 
-// Collision of the *_REL formats.  A relative code is a function of two rounded
-// densities and amplifies the rounding of the step that produced it (one code
-// of a BF16 population is 2^-9 of it, and a flipped code moves all its readers),
-// so two orders of the same sums part by some 1e-3 within 20 steps.  These
-// instances keep one fixed order of operations, component by component, so
-// that their runs and checkpoints reproduce bit for bit.
+// Collision in scalar operations, component by component (kScalar).  A relative
+// code is a function of two rounded densities and amplifies the rounding of the
+// step that produced it (one code of a BF16 population is 2^-9 of it, and a
+// flipped code moves all its readers), so two orders of the same sums part by
+// some 1e-3 within 20 steps: these instances keep one fixed order of
+// operations, so that their runs and checkpoints reproduce bit for bit.
 template <int S, int REG, int FORCE>
-__device__ __forceinline__ void collide_rel(typename Store<S>::T *__restrict__ fout, const Phys<typename Store<S>::R> &p,
-                                            const FusedSmem<kStash<REG>> &sm, const InvRing *rinv, int sl_m, int sl_c,
-                                            int sl_p, int st, long long cell, typename Store<S>::R *__restrict__ s_out,
+__device__ __forceinline__ void collide_scalar(typename Store<S>::T *__restrict__ fout, const Phys<typename Store<S>::R> &p,
+                                               const FusedSmem<kStash<REG>> &sm, const InvRing *rinv, int sl_m,
+                                               int sl_c, int sl_p, int st, long long cell, typename Store<S>::R *__restrict__ s_out,
                                             bool lo_wall, bool hi_wall, unsigned lw)
 {
     using R = typename Store<S>::R;
@@ -447,6 +460,11 @@ __device__ __forceinline__ void collide_rel(typename Store<S>::T *__restrict__ f
     const R rq1 = r1 / R(36), rq2 = r2 / R(36);   // rho w_i = (rho / 36) k_i
     typename Store<S>::T *o = fout + 2 * cell;   // (component 1, component 2) of direction 0
     const unsigned N32 = (unsigned)p.N;
+    // Deviation formats (BGK): the stash holds d = f - w rho0 and the outputs are
+    // stored as f* - w rho0, a constant -omega rho0 per unit weight in each output
+    // (keep f = keep d + keep w rho0)
+    const R dc1 = Store<S>::kDev ? p.omega[0] * R(p.rho0) : R(0);
+    const R dc2 = Store<S>::kDev ? p.omega[1] * R(p.rho0) : R(0);
     // Regularized: second moments of f - f^eq(u): Pi = sum c c f - rho (T0 I + u u)
     R P1[6], P2[6], t1 = 0, t2 = 0;
     Third<R> th1, th2;   // REG = 2: third-order moments of f - f^eq(u)
@@ -494,9 +512,13 @@ __device__ __forceinline__ void collide_rel(typename Store<S>::T *__restrict__ f
             o1 += cf1 * (R(-1) * uF1);
             o2v += cf2 * (R(-1) * uF2);
         }
-        const float2 iv = rinv[sl_c][ly][lx];   // 1/rho of the cell itself; 1/w_0 = 3
-        Store<S>::store2(o, o1, o2v, R(3) * iv.x, R(3) * iv.y);
-        state_ref(fout, p.ref_off)[cell] = rr;
+        if constexpr (Store<S>::kRel) {
+            const float2 iv = rinv[sl_c][ly][lx];   // 1/rho of the cell itself; 1/w_0 = 3
+            Store<S>::store2(o, o1, o2v, R(3) * iv.x, R(3) * iv.y);
+            state_ref(fout, p.ref_off)[cell] = rr;
+        } else {
+            Store<S>::store2_d(o, o1 - w<R>(0) * dc1, o2v - w<R>(0) * dc2);
+        }
     }
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
@@ -513,6 +535,7 @@ __device__ __forceinline__ void collide_rel(typename Store<S>::T *__restrict__ f
             const R Eu = Au + R(4.5) * cu * cu, Ou = cu * (Bu + R(4.5) * cu * cu);
             R P1e = rw1 * (E1 - keep1 * Eu), M1 = rw1 * (O1 - keep1 * Ou);
             R P2e = rw2 * (E2 - keep2 * Eu), M2 = rw2 * (O2 - keep2 * Ou);
+            if constexpr (Store<S>::kDev) { P1e -= w<R>(i) * dc1; P2e -= w<R>(i) * dc2; }
             const float2 fp = s0[i * kThreadsF], fm = s0[(i + 1) * kThreadsF];
             o1p = P1e + M1 + keep1 * fp.x;
             o1m = P1e - M1 + keep1 * fm.x;
@@ -546,16 +569,21 @@ __device__ __forceinline__ void collide_rel(typename Store<S>::T *__restrict__ f
             o2p += e2 + d2; o2m += e2 - d2;
         }
         const size_t ip = 2 * (size_t)((unsigned)i * N32), im = 2 * (size_t)((unsigned)(i + 1) * N32);
-        // destinations: x + c_i for i, x - c_i for opp(i), or x across a wall
-        const bool wp = (cz(i) == -1 && lo_wall) || (cz(i) == 1 && hi_wall) || ((lw >> (i + 1)) & 1u);
-        const bool wm = (cz(i) == 1 && lo_wall) || (cz(i) == -1 && hi_wall) || ((lw >> i) & 1u);
-        const int slp = cz(i) == -1 ? sl_m : (cz(i) == 1 ? sl_p : sl_c);
-        const int slm = cz(i) == -1 ? sl_p : (cz(i) == 1 ? sl_m : sl_c);
-        const float2 dp = wp ? rinv[sl_c][ly][lx] : rinv[slp][ly + cy(i)][lx + cx(i)];
-        const float2 dm = wm ? rinv[sl_c][ly][lx] : rinv[slm][ly - cy(i)][lx - cx(i)];
-        const R sk = R(36 / k36(i));   // 1 / w_i: the code parameter is 1 / (w_i rho~)
-        Store<S>::store2(o + ip, o1p, o2p, sk * dp.x, sk * dp.y);
-        Store<S>::store2(o + im, o1m, o2m, sk * dm.x, sk * dm.y);
+        if constexpr (Store<S>::kRel) {
+            // destinations: x + c_i for i, x - c_i for opp(i), or x across a wall
+            const bool wp = (cz(i) == -1 && lo_wall) || (cz(i) == 1 && hi_wall) || ((lw >> (i + 1)) & 1u);
+            const bool wm = (cz(i) == 1 && lo_wall) || (cz(i) == -1 && hi_wall) || ((lw >> i) & 1u);
+            const int slp = cz(i) == -1 ? sl_m : (cz(i) == 1 ? sl_p : sl_c);
+            const int slm = cz(i) == -1 ? sl_p : (cz(i) == 1 ? sl_m : sl_c);
+            const float2 dp = wp ? rinv[sl_c][ly][lx] : rinv[slp][ly + cy(i)][lx + cx(i)];
+            const float2 dm = wm ? rinv[sl_c][ly][lx] : rinv[slm][ly - cy(i)][lx - cx(i)];
+            const R sk = R(36 / k36(i));   // 1 / w_i: the code parameter is 1 / (w_i rho~)
+            Store<S>::store2(o + ip, o1p, o2p, sk * dp.x, sk * dp.y);
+            Store<S>::store2(o + im, o1m, o2m, sk * dm.x, sk * dm.y);
+        } else {
+            Store<S>::store2_d(o + ip, o1p, o2p);
+            Store<S>::store2_d(o + im, o1m, o2m);
+        }
     }
 }
 
@@ -599,15 +627,15 @@ __device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ 
         }
         return;
     }
-    if constexpr (Store<S>::kRel) {
-        collide_rel<S, REG, FORCE>(fout, p, sm, rinv, sl_m, sl_c, sl_p, st, cell, s_out, lo_wall, hi_wall, lw);
+    if constexpr (kScalar<S, REG>) {
+        collide_scalar<S, REG, FORCE>(fout, p, sm, rinv, sl_m, sl_c, sl_p, st, cell, s_out, lo_wall, hi_wall, lw);
         return;
     } else {
     const int lx = tid % kTX + 1, ly = tid / kTX + 1;
     const float2 rr = sm.ring[sl_c][ly][lx];
     // S^b = sum_{i != 0} w_i c_i rho^b(x + c_i)  (Eq. 7; ghost planes carry Eq. 13's rho')
     float2 Sb[3];
-    interaction2<float>([&](int i) {
+    interaction<PairF32>([&](int i) {
         const int slp = cz(i) == -1 ? sl_m : (cz(i) == 1 ? sl_p : sl_c);
         const int slm = cz(i) == -1 ? sl_p : (cz(i) == 1 ? sl_m : sl_c);
         return vsub(sm.ring[slp][ly + cy(i)][lx + cx(i)], sm.ring[slm][ly - cy(i)][lx - cx(i)]);
@@ -623,11 +651,14 @@ __device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ 
     const R inv = R(1) / (rr.x + rr.y);
     const R ux = sm.mom[st][0][tid] * inv, uy = sm.mom[st][1][tid] * inv, uz = sm.mom[st][2][tid] * inv;
     const float2 *s0 = &sm.stash[st][0][tid];
-    RegMoments<float, REG> mo;
+    RegMoments<PairF32, REG> mo;
+    if constexpr (RegMoments<PairF32, REG>::n > 0) {
 #pragma unroll
-    for (int k = 0; k < RegMoments<float, REG>::n; ++k) mo.m[k] = s0[k * kThreadsF];
+        for (int k = 0; k < RegMoments<PairF32, REG>::n; ++k) mo.m[k] = s0[k * kThreadsF];
+    }
     typename Store<S>::T *o = fout + 2 * cell;   // (component 1, component 2) of direction 0
-    const unsigned N32 = (unsigned)p.N;
+    unsigned N32 = (unsigned)p.N;
+    if constexpr (Store<S>::kDev) asm volatile("" : "+r"(N32));   // keeps i N out of the loop's invariants (spills)
     const R ref0 = p.rho0;
     auto get = [&](int i) { return s0[i * kThreadsF]; };
     auto put = [&](int i, float2 f) {
@@ -639,7 +670,8 @@ __device__ __forceinline__ void collide_cell(typename Store<S>::T *__restrict__ 
             Store<S>::store2(q, f.x, f.y, ref, ref);
         }
     };
-    collide2<float, REG, FORCE, Store<S>::kDev>(p, rr, inv, ux, uy, uz, Sb, mo, get, put);
+    const float2 So[3] = {vswap(Sb[0]), vswap(Sb[1]), vswap(Sb[2])};
+    lbm::collide_cell<PairF32, REG, FORCE, Store<S>::kDev>(PairF32(), p, rr, inv, ux, uy, uz, So, mo, get, put);
     }
 }
 
@@ -662,8 +694,11 @@ __device__ __forceinline__ void interior_plane(const Phys<typename Store<S>::R> 
     } else if (!pr.constant) {
         float2 a;
         R jx, jy, jz;
-        if constexpr (Store<S>::kRel) sums_rel(v, a, jx, jy, jz);
-        else sums2<float>(v, a, jx, jy, jz);
+        if constexpr (kScalar<S, REG>) sums_scalar(v, a, jx, jy, jz);
+        else {
+            a = density(v);
+            momentum(PairF32(), v, jx, jy, jz);
+        }
         if constexpr (Store<S>::kDev) { a.x += p.rho0; a.y += p.rho0; }   // sum_i w_i rho0 = rho0
         if (pr.ghost) {
             r1 += a.x; r2 += a.y;
@@ -674,11 +709,11 @@ __device__ __forceinline__ void interior_plane(const Phys<typename Store<S>::R> 
 #pragma unroll
                     for (int k = 0; k < Q; ++k) sm.stash[st][k][tid] = v[k];
                 } else if constexpr (REG != COLL_EQ) {
-                    RegMoments<float, REG> mo;
-                    if constexpr (Store<S>::kRel) moments_rel<REG>(v, mo);
+                    RegMoments<PairF32, REG> mo;
+                    if constexpr (kScalar<S, REG>) moments_scalar<REG>(v, mo);
                     else mo.of(v);
 #pragma unroll
-                    for (int k = 0; k < RegMoments<float, REG>::n; ++k) sm.stash[st][k][tid] = mo.m[k];
+                    for (int k = 0; k < RegMoments<PairF32, REG>::n; ++k) sm.stash[st][k][tid] = mo.m[k];
                 }
                 sm.mom[st][0][tid] = jx; sm.mom[st][1][tid] = jy; sm.mom[st][2][tid] = jz;
             }
@@ -718,7 +753,7 @@ __device__ __forceinline__ void halo_combine(const Phys<R> &p, SM &sm, InvRing *
 // site puts its wall density into the ring (a solid halo cell through its
 // first partial, the others zero) and stores zero populations.
 template <int S, int REG, bool WALLZ, bool MASK, int FORCE>
-__global__ void __launch_bounds__(kThreadsF, kBlocks<S, REG>)
+__global__ void __launch_bounds__(kThreadsF, kBlocks<S, REG, WALLZ>)
 k_step_fused(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T *__restrict__ fout,
              Phys<typename Store<S>::R> p, int ntx, int lz, typename Store<S>::R *__restrict__ s_out,
              const unsigned *__restrict__ links, const float2 *__restrict__ wrho)
@@ -817,8 +852,7 @@ k_step_fused(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T 
             } else if (!pr.constant) {
                 float2 hv[Q], a;
                 GatherAll<S, 0>::run(fin, p.N, gather_ref<S>(fin, p, pr, ch), pr, ch, hl, hv);
-                R jx, jy, jz;
-                sums2<float>(hv, a, jx, jy, jz);
+                a = density(hv);
                 if constexpr (Store<S>::kDev) { a.x += p.rho0; a.y += p.rho0; }
                 if (pr.ghost) { r1 += a.x; r2 += a.y; } else { r1 = a.x; r2 = a.y; }
             }
@@ -851,10 +885,9 @@ k_step_fused(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T 
     // interior populations of plane z0+1, in registers until the first iteration
     // Interior populations of plane z+1, in registers from the gathers issued
     // before the previous collision until phase A: decoded (v), or, in the
-    // 16-bit instances that run periodic lattices without a mask (the ones
-    // measured to gain from it), as stored (rv, with the reference densities
+    // 16-bit instances that gain from it (kRawCarry), as stored (rv, with the reference densities
     // rrv), which keeps 19 registers instead of 38 live across the collision.
-    constexpr bool kRaw = sizeof(typename Store<S>::Raw) < sizeof(float2) && !WALLZ && !MASK;
+    constexpr bool kRaw = kRawCarry<S, REG, WALLZ, MASK>;
     float2 v[Q];
     typename Store<S>::Raw rv[Q];
     float2 rrv = make_float2(0.f, 0.f);
@@ -975,6 +1008,8 @@ cudaError_t launch_inst(dim3 grid, cudaStream_t s, const typename Store<S>::T *f
         if (e != cudaSuccess) return e;
         if (cached) attr_set[dev].store(1, std::memory_order_release);
     }
+    // (programmatic stream serialization gains nothing here: 96^3 52.4 -> 51.8 us
+    // per step, but 64^3 18.6 -> 25.6, where the early CTAs double up on busy SMs)
     k_step_fused<S, REG, WALLZ, MASK, FORCE><<<grid, kThreadsF, smem_bytes<S, REG>(), s>>>(fi, fo, p, ntx, lz, s_out, links, wrho);
     return cudaSuccess;
 }
