@@ -1,0 +1,8 @@
+// Instances of the box step for the f16dev storage format.
+#include "lbm_box_impl.cuh"
+
+namespace lbm {
+namespace box {
+template cudaError_t box_t<ST_F16_DEV>(const HostPhys &, const void *, void *, cudaStream_t, void *);
+}  // namespace box
+}  // namespace lbm

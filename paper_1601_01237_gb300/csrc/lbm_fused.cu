@@ -49,6 +49,44 @@ int fused_planes(long long cols, int nz, int sms)
     return cbest * 20 <= c64 * 19 ? best : (nz < kPlanesMax ? nz : kPlanesMax);
 }
 
+namespace box {
+template <int S>
+cudaError_t box_t(const HostPhys &h, const void *fin, void *fout, cudaStream_t s, void *s_out);
+}  // namespace box
+
+bool use_box(const HostPhys &p)
+{
+    if (p.storage != ST_F32 && p.storage != ST_F16_DEV && p.storage != ST_BF16_DEV) return false;
+    if (!fused_supported(p) || (p.ny + 7) / 8 > 65535 || (p.nz + 3) / 4 > 65535) return false;
+    // One layer along y: the marching tiles would repeat it eight times.
+    if (p.ny == 1) return true;
+    // One periodic layer along z: the box step is the faster one while its halo
+    // comes from L2 (us per step, marching / box: 700^2 47 / 29, 2048^2 363 / 356,
+    // 4096^2 1479 / 2328).
+    if (p.nz == 1 && !p.wall_z) return p.N <= 2048LL * 2048;
+    // Elsewhere by cost: a marching CTA takes about 1.85 us per plane while its
+    // SM holds no other (and in proportion beyond), the box step 0.092 ns per cell
+    // of its padded boxes, 1/20000 of that (marching / box: 56^3 19.3 / 16.1, 60^3
+    // 18.5 / 21.1, 8 x 128 x 128 19.3 / 12.8, 300 x 24 x 24 18.6 / 15.9, 2 x 200 x 200
+    // 10.4 / 11.8).
+    const int sms = current_device_sms();
+    const long long cols = (long long)((p.nx + 31) / 32) * ((p.ny + 7) / 8);
+    const int lz = fused_planes(cols, p.nz, sms);
+    const long long ctas = cols * ((p.nz + lz - 1) / lz);
+    const long long padded = (long long)((p.nx + 7) / 8) * ((p.ny + 7) / 8) * ((p.nz + 3) / 4) * 256;
+    return padded * sms < 20000LL * (lz + 2) * (ctas > sms ? ctas : sms);
+}
+
+cudaError_t launch_step_box(const HostPhys &p, const void *f_in, void *f_out, cudaStream_t s, void *s_out)
+{
+    switch (p.storage) {
+    case ST_F32: return box::box_t<ST_F32>(p, f_in, f_out, s, s_out);
+    case ST_F16_DEV: return box::box_t<ST_F16_DEV>(p, f_in, f_out, s, s_out);
+    case ST_BF16_DEV: return box::box_t<ST_BF16_DEV>(p, f_in, f_out, s, s_out);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 cudaError_t launch_step_fused(const HostPhys &p, const void *f_in, void *f_out, cudaStream_t s, cudaEvent_t *ev,
                               void *s_out)
 {

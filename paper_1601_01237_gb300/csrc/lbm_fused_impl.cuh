@@ -1132,7 +1132,8 @@ cudaError_t fused_t(const HostPhys &h, const void *fin, void *fout, cudaStream_t
         k_wall_solid_rho<S><<<(unsigned)((h.n_bsolid + 255) / 256), 256, 0, s>>>(h.solid, make_phys_f<float>(h), h.bsolid,
                                                                              h.n_bsolid, wr);
     }
-    const cudaError_t e = h.forcing == FORCE_GUO
+    const cudaError_t e = use_box(h) ? launch_step_box(h, fin, fout, s, s_out)
+                          : h.forcing == FORCE_GUO
                               ? launch_coll<S, FORCE_GUO>(h, lz, grid, s, fi, fo, p, ntx, (R *)s_out)
                               : launch_coll<S, FORCE_EDM>(h, lz, grid, s, fi, fo, p, ntx, (R *)s_out);
     if (e != cudaSuccess) return e;

@@ -64,6 +64,12 @@ cudaError_t launch_step_split(const HostPhys &p, const void *f_in, void *f_out, 
 cudaError_t launch_step_fused(const HostPhys &p, const void *f_in, void *f_out, cudaStream_t s,
                               cudaEvent_t *ev = nullptr, void *s_out = nullptr);
 bool fused_supported(const HostPhys &p);
+
+// The fused step of small and thin lattices (same contract; under a
+// mirror-model mask the wall densities must have been refreshed).  use_box:
+// whether launch_step_fused takes it.
+cudaError_t launch_step_box(const HostPhys &p, const void *f_in, void *f_out, cudaStream_t s, void *s_out = nullptr);
+bool use_box(const HostPhys &p);
 // Planes per CTA of the fused step for a lattice of cols = ceil(nx/32) *
 // ceil(ny/8) tile columns and nz planes on a device with sms SMs.
 constexpr int kPlanesMax = 64, kPlanesMin = 8;
