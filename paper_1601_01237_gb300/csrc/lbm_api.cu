@@ -22,7 +22,10 @@ struct lbm_lattice {
     int device;
     cudaStream_t stream;
     bool own_stream;
-    void *f[2];          // population copies (storage format)
+    // population copies (storage format); between calls the one that does not
+    // hold the current state is scratch (host fields of an initialisation, the
+    // velocities of output fields and reductions)
+    void *f[2];
     int cur;             // index of the copy holding the current state
     void *rho;           // density scratch of the two-kernel step (2*N reals)
     double *partials;    // reduction partials (device)
@@ -290,18 +293,9 @@ lbm_status lbm_init_fields(lbm_lattice *h, const double *rho1, const double *rho
     const size_t N = (size_t)h->phys.N;
     const double *d1 = rho1, *d2 = rho2, *du = u;
     // The other state copy is free until the first step: it stages host fields
-    // (no allocation) and then holds the rest values of a state at rest.
-    char *spare = (char *)h->f[1];
-    const size_t cap = lbm::state_bytes(h->phys.storage, N);
-    const size_t stage = on_device ? 0 : sizeof(double) * N * (u ? 5 : 2);
-    const size_t rest = 8 * N * lbm::real_bytes(h->phys.storage);
-    void *tmp = nullptr;
+    // (at most 40 of its 76 or more bytes per cell; no allocation).
     if (!on_device) {
-        double *t = (double *)spare;
-        if (stage + rest > cap) {   // not reached by the built formats (at most 104 of 304 B per cell)
-            CK(cudaMallocAsync(&tmp, stage, h->stream), "lbm_init_fields: staging");
-            t = (double *)tmp;
-        }
+        double *t = (double *)h->f[1];
         lbm_status st;
         if ((st = copy_in(h, t, rho1, sizeof(double) * N, 0)) != LBM_OK) return st;
         if ((st = copy_in(h, t + N, rho2, sizeof(double) * N, 0)) != LBM_OK) return st;
@@ -313,9 +307,7 @@ lbm_status lbm_init_fields(lbm_lattice *h, const double *rho1, const double *rho
     h->cur = 0;
     h->steps = 0;
     h->init_at_rest = u == nullptr;
-    void *scratch = tmp ? (void *)spare : (stage + rest <= cap ? (void *)(spare + stage) : nullptr);
-    CK(lbm::launch_init_feq(h->phys, d1, d2, du, h->f[0], scratch, h->stream), "lbm_init_fields: launch");
-    if (tmp) CK(cudaFreeAsync(tmp, h->stream), "lbm_init_fields: free staging");
+    CK(lbm::launch_init_feq(h->phys, d1, d2, du, h->f[0], h->stream), "lbm_init_fields: launch");
     // host inputs: the caller may reuse its buffers on return
     if (!on_device) CK(cudaStreamSynchronize(h->stream), "lbm_init_fields: sync");
     return LBM_OK;
@@ -452,14 +444,14 @@ lbm_status lbm_moments(lbm_lattice *h, int out_f64, void *rho1, void *rho2, void
     const size_t N = (size_t)h->phys.N;
     const size_t es = out_f64 ? 8 : 4;
     if (on_device) {
-        CK(lbm::launch_moments(h->phys, h->f[h->cur], h->rho, out_f64, rho1, rho2, uF, h->stream),
+        CK(lbm::launch_moments(h->phys, h->f[h->cur], h->rho, h->f[h->cur ^ 1], out_f64, rho1, rho2, uF, h->stream),
            "lbm_moments: launch");
         return LBM_OK;
     }
     void *tmp = nullptr;
     CK(cudaMallocAsync(&tmp, es * N * 5, h->stream), "lbm_moments: staging");
     char *t = (char *)tmp;
-    CK(lbm::launch_moments(h->phys, h->f[h->cur], h->rho, out_f64, rho1 ? t : nullptr,
+    CK(lbm::launch_moments(h->phys, h->f[h->cur], h->rho, h->f[h->cur ^ 1], out_f64, rho1 ? t : nullptr,
                            rho2 ? t + es * N : nullptr, uF ? t + 2 * es * N : nullptr, h->stream),
        "lbm_moments: launch");
     if (rho1) CK(cudaMemcpyAsync(rho1, t, es * N, cudaMemcpyDeviceToHost, h->stream), "lbm_moments: copy");
@@ -474,8 +466,8 @@ lbm_status lbm_reduce(lbm_lattice *h, double out[6])
 {
     if (!h || !out) return fail(LBM_EINVAL, "lbm_reduce: NULL argument");
     DeviceGuard g(h->device);
-    const int nb = lbm::reduce_blocks();
-    CK(lbm::launch_reduce(h->phys, h->f[h->cur], h->rho, h->partials, h->stream), "lbm_reduce: launch");
+    const int nb = lbm::reduce_grid(h->phys.N);
+    CK(lbm::launch_reduce(h->phys, h->f[h->cur], h->rho, h->f[h->cur ^ 1], h->partials, h->stream), "lbm_reduce: launch");
     CK(cudaMemcpyAsync(h->partials_h, h->partials, (size_t)nb * 8 * sizeof(double), cudaMemcpyDeviceToHost,
                        h->stream),
        "lbm_reduce: copy");
@@ -498,7 +490,7 @@ namespace {
 
 lbm_status diag_run(lbm_lattice *h, int which, const double *vec3, double a0, double a1, double *sums, int nsums)
 {
-    const int nb = lbm::diag_blocks(), ns = lbm::diag_slots();
+    const int nb = lbm::diag_grid(h->phys.N), ns = lbm::diag_slots();
     CK(lbm::launch_density(h->phys, h->f[h->cur], h->rho, h->stream), "diagnostics: density");
     if (which == 0)
         CK(lbm::launch_pressure(h->phys, h->rho, vec3, a0, a1, h->partials, h->stream), "diagnostics: pressure");

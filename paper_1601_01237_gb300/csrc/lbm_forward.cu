@@ -12,8 +12,8 @@
 //
 // Staircase walls (the inclined walls of Sec. 4.2) are a mask of solid sites
 // (Phys::solid): links into a solid site bounce back, solid sites hold zero
-// populations, and the density pass is followed by k_wall_rho, which gives
-// each solid site the density it presents to Eq. 13.
+// populations, and the density pass is followed by k_wall_rho_list,
+// which gives each solid site next to fluid the density it presents to Eq. 13.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -51,10 +51,17 @@ __device__ __forceinline__ bool decode_cell(const Phys<R> &p, long long cell, Nb
 {
     if (cell >= p.N) return false;
     const long long plane = (long long)p.nx * p.ny;
-    const int z = (int)(cell / plane);
-    const long long rem = cell - (long long)z * plane;
-    const int y = (int)(rem / p.nx);
-    const int x = (int)(rem - (long long)y * p.nx);
+    int x, y, z;
+    if (p.N <= 0x7fffffffLL) {   // (64-bit divisions cost more than the rest of the index arithmetic)
+        const unsigned c = (unsigned)cell, pl = (unsigned)plane, nx = (unsigned)p.nx;
+        const unsigned zu = c / pl, rem = c - zu * pl, yu = rem / nx;
+        x = (int)(rem - yu * nx); y = (int)yu; z = (int)zu;
+    } else {
+        z = (int)(cell / plane);
+        const long long rem = cell - (long long)z * plane;
+        y = (int)(rem / p.nx);
+        x = (int)(rem - (long long)y * p.nx);
+    }
     n.cell = cell;
     n.z = z;
     n.xo[0] = (x == 0 ? p.nx - 1 : x - 1);
@@ -171,7 +178,7 @@ k_density(const typename Store<S>::T *__restrict__ f, typename Store<S>::R *__re
     using R = typename Store<S>::R;
     Nbr n;
     if (!decode_cell(p, (long long)blockIdx.x * kThreads + threadIdx.x, n)) return;
-    if (p.solid && p.solid[n.cell]) return;   // k_wall_rho writes solid sites
+    if (p.solid && p.solid[n.cell]) return;   // k_wall_rho_list writes the solid sites that are read
     R fa[2][Q];
     gather<S>(f, p, n, fa);
 #pragma unroll
@@ -181,36 +188,6 @@ k_density(const typename Store<S>::T *__restrict__ f, typename Store<S>::R *__re
         for (int i = 0; i < Q; ++i) s += fa[a][i];
         rho[(long long)a * p.N + n.cell] = s;
     }
-}
-
-// Density that a solid site of the mask presents to the interaction sum of
-// Eq. 13, written into rho after the density pass: the modified model takes
-// the mean of rho^b over the site's fluid neighbours weighted by w_i (zero
-// normal derivative for fields that vary along the wall normal) plus rho_s^b;
-// the original model takes rho_s^b.  A site with no fluid neighbour is never
-// read by a fluid cell and gets rho_s^b.
-template <class R>
-__global__ void __launch_bounds__(kThreads)
-k_wall_rho(R *__restrict__ rho, PhysF<R> p)
-{
-    Nbr n;
-    if (!decode_cell(p, (long long)blockIdx.x * kThreads + threadIdx.x, n)) return;
-    if (!p.solid[n.cell]) return;
-    R num1 = 0, num2 = 0;
-    int den36 = 0;   // sum of w_i over fluid neighbours, in units of 1/36
-    if (p.wall_mirror) {
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            const long long nb = n.zo[1 + cz(i)] + n.yo[1 + cy(i)] + n.xo[1 + cx(i)];
-            if (__ldg(p.solid + nb)) continue;
-            const R k = R(k36(i));
-            num1 += k * rho[nb];
-            num2 += k * rho[p.N + nb];
-            den36 += k36(i);
-        }
-    }
-    rho[n.cell] = (den36 ? num1 / R(den36) : R(0)) + p.rho_s[0];
-    rho[p.N + n.cell] = (den36 ? num2 / R(den36) : R(0)) + p.rho_s[1];
 }
 
 // Link flags of a mask: bit i of cell x set when x - c_i is a solid site (so
@@ -379,34 +356,42 @@ k_density64(const double *__restrict__ f, double *__restrict__ rho, PhysF<double
     const unsigned lf = p.links ? __ldg(p.links + cell) : 0u;
     const int a = (int)(t & 1u);
     const Nbr32 n = neighbours32(p, cell);
-    if (lf & 1u) return;   // k_wall_rho64 writes the solid sites that are read
+    if (lf & 1u) return;   // k_wall_rho_list writes the solid sites that are read
     double v[Q];
     gather64(f, p, n, lf, a, v);
     rho[(size_t)a * (unsigned)p.N + cell] = density(v);
 }
 
-// k_wall_rho over the solid sites next to fluid, the only ones that are read,
-// one component per lane.
+// Density that a solid site of the mask presents to the interaction sum of
+// Eq. 13, written into rho after the density pass: the modified model takes
+// the mean of rho^b over the site's fluid neighbours weighted by w_i (zero
+// normal derivative for fields that vary along the wall normal) plus rho_s^b;
+// the original model takes rho_s^b.  Over the sites next to fluid, the only ones
+// that are read, one component per lane.
+// PAIRS: rho holds (rho^1, rho^2) per cell instead of one array per component.
+template <class R, bool PAIRS>
 __global__ void __launch_bounds__(kThreads64)
-k_wall_rho64(double *__restrict__ rho, PhysF<double> p, const unsigned *__restrict__ sites, unsigned n_sites)
+k_wall_rho_list(R *__restrict__ rho, PhysF<R> p, const unsigned *__restrict__ sites, unsigned n_sites)
 {
     const unsigned t = blockIdx.x * kThreads64 + threadIdx.x;
     if ((t >> 1) >= n_sites) return;
     const int a = (int)(t & 1u);
     const Nbr32 n = neighbours32(p, sites[t >> 1]);
-    double *r = rho + (size_t)a * (unsigned)p.N;
-    double num = 0;
+    const unsigned lf = __ldg(p.links + n.cell);   // bit opp(i): x + c_i is solid
+    auto r = [&](unsigned c) -> R & { return PAIRS ? rho[2 * (size_t)c + a] : rho[(size_t)a * (unsigned)p.N + c]; };
+    R num = 0;
     int den36 = 0;
     if (p.wall_mirror) {
 #pragma unroll
         for (int i = 1; i < Q; ++i) {
-            const unsigned nb = n.zo[1 + cz(i)] + n.yo[1 + cy(i)] + n.xo[1 + cx(i)];
-            if (__ldg(p.solid + nb)) continue;
-            num += (double)k36(i) * r[nb];
-            den36 += k36(i);
+            // (every neighbour is read, so that the loads are in flight together)
+            const R v = r(n.zo[1 + cz(i)] + n.yo[1 + cy(i)] + n.xo[1 + cx(i)]);
+            const bool fluid = !((lf >> opp(i)) & 1u);
+            num += fluid ? R(k36(i)) * v : R(0);
+            den36 += fluid ? k36(i) : 0;
         }
     }
-    r[n.cell] = (den36 ? num / (double)den36 : 0.0) + p.rho_s[a];
+    r(n.cell) = (den36 ? num / R(den36) : R(0)) + p.rho_s[a];
 }
 
 template <int KIND, int FORCE>
@@ -452,80 +437,60 @@ k_collide64(const double *__restrict__ fin, double *__restrict__ fout, const dou
     collide_cell<LaneF64, KIND, FORCE, false>(c, p, r, inv, jx * inv, jy * inv, jz * inv, So, mom, get, put);
 }
 
-// Rest-state values of one cell, formed once per cell in FP64 and rounded to
-// the arithmetic type: rho^a w for the three weight classes (w = 1/3, 1/18,
-// 1/36) and rho^a itself, at slot (2 q + a) N + c (q = 0, 1, 2, 3).  The
-// initial populations at rest gather these instead of forming 38 FP64
-// products per cell, each repeated by up to seven readers (the FP64 pipe is
-// a small fraction of the FP32 one on this GPU); the values are the same
-// roundings of the same FP64 products.
-template <class R>
-__global__ void __launch_bounds__(kThreads)
-k_rest_values(const double *__restrict__ rho1, const double *__restrict__ rho2, R *__restrict__ out, long long N)
-{
-    const long long c = (long long)blockIdx.x * kThreads + threadIdx.x;
-    if (c >= N) return;
-    const double r[2] = {rho1[c], rho2[c]};
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-        out[(0 + a) * N + c] = (R)(r[a] * wd(0));
-        out[(2 + a) * N + c] = (R)(r[a] * wd(1));
-        out[(4 + a) * N + c] = (R)(r[a] * wd(7));
-        out[(6 + a) * N + c] = (R)r[a];
-    }
-}
-
-// Stored value s_j(y): the population that the gather of step 0 reads as
-// f_j(y + c_j), or, when y + c_j is a wall site, as f_opp(j)(y).  rest: the
-// values of k_rest_values (the state at rest, u == NULL), or NULL.
+// Initial populations f_i(x) = f^eq_i(rho(x), u(x)) of Eq. 3, each written where
+// the first gather of cell x reads it: population i at x - c_i, or in the place
+// of opp(i) at x itself where x - c_i is a wall site.  A cell's polynomials are
+// formed once, opposite directions sharing them, and its densities are read
+// once (a gather form had every cell's polynomials repeated by its 19 readers:
+// 128^3 FP32 with u 1576 us, this one 590 us, at rest 128 / 64 us; bound by its 150 FP64 operations
+// per cell).  At rest the values are the roundings of the FP64 products rho w_i.
 template <int S>
 __global__ void __launch_bounds__(kThreads)
-k_init_feq(const double *__restrict__ rho1, const double *__restrict__ rho2,
-           const double *__restrict__ u, const typename Store<S>::R *__restrict__ rest,
+k_init_feq(const double *__restrict__ rho1, const double *__restrict__ rho2, const double *__restrict__ u,
            typename Store<S>::T *__restrict__ f, PhysF<typename Store<S>::R> p)
 {
     using R = typename Store<S>::R;
     Nbr n;
-    if (!decode_cell(p, (long long)blockIdx.x * kThreads + threadIdx.x, n)) return;
-    const bool here_solid = p.solid && p.solid[n.cell];
-    const long long N = p.N;
+    if (!decode_cell(p, (long long)blockIdx.x * blockDim.x + threadIdx.x, n)) return;
+    const unsigned lf = p.links ? __ldg(p.links + n.cell) : 0u;   // bit i: x - c_i is solid
+    if (lf & 1u) {   // solid sites hold no populations
 #pragma unroll
-    for (int j = 0; j < Q; ++j) {
-        const long long dst = n.zo[1 + cz(j)] + n.yo[1 + cy(j)] + n.xo[1 + cx(j)];
-        const bool wall = (cz(j) == -1 && n.zlo_wall) || (cz(j) == 1 && n.zhi_wall) ||
-                          (j != 0 && p.solid && p.solid[dst]);
-        const long long src = wall ? n.cell : dst;
-        const int k = wall ? opp(j) : j;
-        R v1, v2, e1 = R(1), e2 = R(1);
-        if (rest) {
-            const int q = k == 0 ? 0 : (k < 7 ? 1 : 2);
-            v1 = rest[(2 * q + 0) * N + src];
-            v2 = rest[(2 * q + 1) * N + src];
-            if constexpr (Store<S>::kRel) { e1 = rest[6 * N + src]; e2 = rest[7 * N + src]; }
-        } else {
-            // f^eq of Eq. 3 at (rho^a, u) of the source cell (u == NULL: at rest)
-            double P = 1.0;
-            if (u) {
-                const double ux = u[3 * src], uy = u[3 * src + 1], uz = u[3 * src + 2];
-                const double usq = ux * ux + uy * uy + uz * uz;
-                const double cu = cdot<double>(k, ux, uy, uz);
-                P = 1.0 - 1.5 * usq + cu * (3.0 - 4.5 * usq) + 4.5 * cu * cu * (1.0 + cu);
-            }
-            v1 = (R)(rho1[src] * wd(k) * P);
-            v2 = (R)(rho2[src] * wd(k) * P);
-            if constexpr (Store<S>::kRel) { e1 = (R)rho1[src]; e2 = (R)rho2[src]; }
+        for (int j = 0; j < Q; ++j) {
+            const R e = Store<S>::kRel ? Store<S>::enc(w<R>(j)) : w<R>(j) * p.rho0;
+            Store<S>::store2(f + pair_index(j, n.cell, p.N), R(0), R(0), e, e);
         }
-        if (here_solid) { v1 = v2 = R(0); e1 = e2 = R(1); }
-        if constexpr (Store<S>::kRel) {   // coded relative to the reader's initial density
-            Store<S>::store2(f + pair_index(j, n.cell, p.N), v1, v2, Store<S>::enc(w<R>(j) * e1),
-                             Store<S>::enc(w<R>(j) * e2));
-        } else {
-            Store<S>::store2(f + pair_index(j, n.cell, p.N), v1, v2, w<R>(j) * p.rho0, w<R>(j) * p.rho0);
-        }
+        if constexpr (Store<S>::kRel) state_ref(f, p.ref_off)[n.cell] = make_float2(1.0f, 1.0f);
+        return;
     }
-    if constexpr (Store<S>::kRel)
-        state_ref(f, p.ref_off)[n.cell] = here_solid ? make_float2(1.0f, 1.0f)
-                                                     : make_float2((float)rho1[n.cell], (float)rho2[n.cell]);
+    const double r1 = rho1[n.cell], r2 = rho2[n.cell];
+    // coded relative to the reader's initial density, which is this cell's
+    const R e1 = Store<S>::kRel ? (R)r1 : p.rho0, e2 = Store<S>::kRel ? (R)r2 : p.rho0;
+    auto put = [&](int i, R v1, R v2) {
+        const bool wall = (cz(i) == 1 && n.zlo_wall) || (cz(i) == -1 && n.zhi_wall) || (i != 0 && ((lf >> i) & 1u));
+        const long long at = wall ? pair_index(opp(i), n.cell, p.N)
+                                  : pair_index(i, n.zo[1 - cz(i)] + n.yo[1 - cy(i)] + n.xo[1 - cx(i)], p.N);
+        Store<S>::store2(f + at, v1, v2, Store<S>::enc(w<R>(i) * e1), Store<S>::enc(w<R>(i) * e2));
+    };
+    if constexpr (Store<S>::kRel) state_ref(f, p.ref_off)[n.cell] = make_float2((float)r1, (float)r2);
+    const double a0 = r1 * wd(0), a1 = r1 * wd(1), a2 = r1 * wd(7), b0 = r2 * wd(0), b1 = r2 * wd(1), b2 = r2 * wd(7);
+    if (!u) {
+        const R v0 = (R)a0, v1 = (R)a1, v2 = (R)a2, w0 = (R)b0, w1 = (R)b1, w2 = (R)b2;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) put(i, i == 0 ? v0 : (i < 7 ? v1 : v2), i == 0 ? w0 : (i < 7 ? w1 : w2));
+        return;
+    }
+    const double ux = u[3 * n.cell], uy = u[3 * n.cell + 1], uz = u[3 * n.cell + 2];
+    const double A = 1.0 - 1.5 * (ux * ux + uy * uy + uz * uz);
+    put(0, (R)(a0 * A), (R)(b0 * A));
+    const double sx = 3.0 * ux, sy = 3.0 * uy, sz = 3.0 * uz;
+#pragma unroll
+    for (int i = 1; i < Q; i += 2) {   // f^eq_+- / (rho w) = A + s^2/2 +- s (A + s^2/6), s = 3 c.u
+        const double s = vdot(i, sx, sy, sz), m = s * s;
+        const double E = fma(m, 0.5, A), O = s * fma(m, 1.0 / 6.0, A);
+        const double a = i < 7 ? a1 : a2, b = i < 7 ? b1 : b2;
+        put(i, (R)(a * (E + O)), (R)(b * (E + O)));
+        put(i + 1, (R)(a * (E - O)), (R)(b * (E - O)));
+    }
 }
 
 // Reference densities of a state set from explicit populations (the *_REL
@@ -607,18 +572,29 @@ __device__ __forceinline__ void velocity_uF(const Phys<R> &p, R r1, R r2, R ux, 
     fz = uz + (g1[2] * r1 + g2[2] * r2) * half_inv;
 }
 
+// Output fields and reductions run in two passes: this one gathers every cell
+// once and leaves its densities (as pairs, where the second pass needs them,
+// and the output fields o1, o2) and its velocity u = j / rho (three planes
+// behind each other); the second one adds the force from the densities'
+// stencil.  u lies in the state copy that is free between steps.  (One pass that
+// gathered again beside a density pass took 1.54 ms for the fields at 256^3
+// FP32, these two 0.68 ms against a floor of 0.43; pairs instead of one array
+// per component halve the second pass's 36 stencil loads.)
+template <class R> struct VecOf;
+template <> struct VecOf<float> { using T = float2; };
+template <> struct VecOf<double> { using T = double2; };
+
 template <int S, class O>
 __global__ void __launch_bounds__(kThreads)
-k_moments(const typename Store<S>::T *__restrict__ f, const typename Store<S>::R *__restrict__ rho,
-          O *__restrict__ o1, O *__restrict__ o2, O *__restrict__ ouF, PhysF<typename Store<S>::R> p)
+k_sums(const typename Store<S>::T *__restrict__ f, typename VecOf<typename Store<S>::R>::T *__restrict__ rho,
+       typename Store<S>::R *__restrict__ u, O *__restrict__ o1, O *__restrict__ o2, PhysF<typename Store<S>::R> p)
 {
     using R = typename Store<S>::R;
     Nbr n;
-    if (!decode_cell(p, (long long)blockIdx.x * kThreads + threadIdx.x, n)) return;
+    if (!decode_cell(p, (long long)blockIdx.x * blockDim.x + threadIdx.x, n)) return;
     if (p.solid && p.solid[n.cell]) {   // no fluid at a solid site
         if (o1) o1[n.cell] = (O)0;
         if (o2) o2[n.cell] = (O)0;
-        if (ouF) { ouF[3 * n.cell] = (O)0; ouF[3 * n.cell + 1] = (O)0; ouF[3 * n.cell + 2] = (O)0; }
         return;
     }
     R fa[2][Q];
@@ -627,55 +603,145 @@ k_moments(const typename Store<S>::T *__restrict__ f, const typename Store<S>::R
     local_moments(fa, r1, r2, ux, uy, uz);
     if (o1) o1[n.cell] = (O)r1;
     if (o2) o2[n.cell] = (O)r2;
-    if (ouF) {
-        R Sb[2][3];
-        interaction_sums(rho, p, n, Sb);
-        R fx, fy, fz;
-        velocity_uF(p, r1, r2, ux, uy, uz, Sb, fx, fy, fz);
-        ouF[3 * n.cell] = (O)fx;
-        ouF[3 * n.cell + 1] = (O)fy;
-        ouF[3 * n.cell + 2] = (O)fz;
+    if (rho) {
+        typename VecOf<R>::T v;
+        v.x = r1;
+        v.y = r2;
+        rho[n.cell] = v;
+        u[n.cell] = ux;
+        u[p.N + n.cell] = uy;
+        u[2 * p.N + n.cell] = uz;
     }
+}
+
+// The same in FP64 with one component per lane.
+template <class O>
+__global__ void __launch_bounds__(kThreads64)
+k_sums64(const double *__restrict__ f, double *__restrict__ rho, double *__restrict__ u, O *__restrict__ o1,
+         O *__restrict__ o2, PhysF<double> p)
+{
+    const unsigned t = blockIdx.x * kThreads64 + threadIdx.x, N32 = (unsigned)p.N;
+    const unsigned cell = min(t >> 1, N32 - 1u);
+    const bool store = (t >> 1) < N32;
+    const LaneF64 c{(int)(t & 1u)};
+    O *o = c.a ? o2 : o1;
+    const unsigned lf = p.links ? __ldg(p.links + cell) : 0u;
+    double v[Q];
+    gather64(f, p, neighbours32(p, cell), lf, c.a, v);
+    const double r = density(v);
+    if (o && store) o[cell] = (lf & 1u) ? (O)0 : (O)r;
+    if (!rho) return;
+    double jx, jy, jz;
+    momentum(c, v, jx, jy, jz);
+    const double inv = 1.0 / c.both(r);
+    if (!store || (lf & 1u)) return;
+    rho[2 * (size_t)cell + c.a] = r;
+    if (c.a == 0) {
+        u[cell] = jx * inv;
+        u[(size_t)N32 + cell] = jy * inv;
+    } else {
+        u[2 * (size_t)N32 + cell] = jz * inv;
+    }
+}
+
+// u_F = u + g / 2 of one cell from the first pass (Eqs. 8-9), with the
+// interaction sums of Eqs. 7 and 13 over opposite neighbours as interaction_sums.
+template <class R>
+__device__ __forceinline__ void velocity_of(const typename VecOf<R>::T *__restrict__ rho, const R *__restrict__ u,
+                                            const PhysF<R> &p, const Nbr32 &n, R &r1, R &r2, R &fx, R &fy, R &fz)
+{
+    using V = typename VecOf<R>::T;
+    auto at = [&](int dx, int dy, int dz) {
+        V v;
+        if ((dz == -1 && n.zlo) || (dz == 1 && n.zhi)) {   // a wall site: its mirror cell's and rho_s, or rho_s
+            v.x = p.rho_s[0];
+            v.y = p.rho_s[1];
+            if (p.wall_mirror) {
+                const V m = __ldg(rho + n.zo[1] + n.yo[1 + dy] + n.xo[1 + dx]);
+                v.x += m.x;
+                v.y += m.y;
+            }
+        } else {
+            v = __ldg(rho + n.zo[1 + dz] + n.yo[1 + dy] + n.xo[1 + dx]);
+        }
+        return v;
+    };
+    R Sb[2][3] = {{0, 0, 0}, {0, 0, 0}};
+#pragma unroll
+    for (int i = 1; i < Q; i += 2) {
+        const V a = at(cx(i), cy(i), cz(i)), b = at(-cx(i), -cy(i), -cz(i));
+        const R d1 = w<R>(i) * (a.x - b.x), d2 = w<R>(i) * (a.y - b.y);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if (ca(i, d) == 1) { Sb[0][d] += d1; Sb[1][d] += d2; }
+            else if (ca(i, d) == -1) { Sb[0][d] -= d1; Sb[1][d] -= d2; }
+        }
+    }
+    const V own = rho[n.cell];
+    const size_t N = (size_t)p.N;
+    r1 = own.x;
+    r2 = own.y;
+    velocity_uF(p, r1, r2, u[n.cell], u[N + n.cell], u[2 * N + n.cell], Sb, fx, fy, fz);
+}
+
+// The three components of a cell's u_F lie side by side in the output; a CTA's
+// are put in order in shared memory and stored in whole rows.
+template <class R, class O>
+__global__ void __launch_bounds__(kThreads)
+k_uF(const typename VecOf<R>::T *__restrict__ rho, const R *__restrict__ u, O *__restrict__ ouF, PhysF<R> p)
+{
+    __shared__ O sh[3 * kThreads];
+    const unsigned c0 = blockIdx.x * blockDim.x, N32 = (unsigned)p.N, cell = c0 + threadIdx.x;
+    R fx = 0, fy = 0, fz = 0;
+    if (cell < N32 && !(p.solid && p.solid[cell])) {
+        R r1, r2;
+        velocity_of<R>(rho, u, p, neighbours32(p, cell), r1, r2, fx, fy, fz);
+    }
+    sh[3 * threadIdx.x] = (O)fx;
+    sh[3 * threadIdx.x + 1] = (O)fy;
+    sh[3 * threadIdx.x + 2] = (O)fz;
+    __syncthreads();
+    const unsigned m = 3 * min(blockDim.x, N32 - c0);
+    O *out = ouF + 3 * (size_t)c0;
+    for (unsigned k = threadIdx.x; k < m; k += blockDim.x) out[k] = sh[k];
 }
 
 constexpr int kReduceBlocks = 1216;   // 152 SMs x 8
 
-template <int S>
-__global__ void __launch_bounds__(kThreads, 2)
-k_reduce(const typename Store<S>::T *__restrict__ f, const typename Store<S>::R *__restrict__ rho,
-         double *__restrict__ partials, PhysF<typename Store<S>::R> p)
+template <class R>
+__global__ void __launch_bounds__(kThreads, 4)
+k_reduce(const typename VecOf<R>::T *__restrict__ rho, const R *__restrict__ u, double *__restrict__ partials,
+         PhysF<R> p)
 {
-    using R = typename Store<S>::R;
     double acc[6] = {0, 0, 0, 0, 0, 0};
-    double bad = 0;
-    for (long long c = (long long)blockIdx.x * kThreads + threadIdx.x; c < p.N;
-         c += (long long)gridDim.x * kThreads) {
-        Nbr n;
-        decode_cell(p, c, n);
+    unsigned bad = 0;
+    R top = 0;   // acc[5] in the arithmetic type
+    const unsigned N32 = (unsigned)p.N;
+    for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < N32; c += gridDim.x * kThreads) {
         if (p.solid && p.solid[c]) continue;   // solid sites hold no fluid
-        R fa[2][Q];
-        gather<S>(f, p, n, fa);
-        R r1, r2, ux, uy, uz;
-        local_moments(fa, r1, r2, ux, uy, uz);
-        R Sb[2][3];
-        interaction_sums(rho, p, n, Sb);
-        R fx, fy, fz;
-        velocity_uF(p, r1, r2, ux, uy, uz, Sb, fx, fy, fz);
+        R r1, r2, fx, fy, fz;
+        velocity_of<R>(rho, u, p, neighbours32(p, c), r1, r2, fx, fy, fz);
         const double rho_t = (double)r1 + (double)r2;
-        if (!(r1 > R(0)) || !(r2 > R(0)) || !isfinite((double)r1) || !isfinite((double)r2)) bad += 1;
+        if (!(r1 > R(0)) || !(r2 > R(0)) || !isfinite(r1) || !isfinite(r2)) ++bad;
         acc[0] += (double)r1;
         acc[1] += (double)r2;
         acc[2] += rho_t * (double)fx;
         acc[3] += rho_t * (double)fy;
         acc[4] += rho_t * (double)fz;
         // max |u_F|^2; the host takes the square root of the maximum, which
-        // equals the maximum of the (correctly rounded, monotonic) roots
-        acc[5] = fmax(acc[5], (double)fx * fx + (double)fy * fy + (double)fz * fz);
+        // equals the maximum of the (correctly rounded, monotonic) roots.  The
+        // FP64 square is formed only where the rounded one can exceed the
+        // maximum so far.
+        const R q = fx * fx + fy * fy + fz * fz;
+        if (!(q * R(1.00001) < top) || top < R(1e-30)) {
+            acc[5] = fmax(acc[5], (double)fx * fx + (double)fy * fy + (double)fz * fz);
+            top = (R)acc[5];
+        }
     }
     // fixed-order block reduction (deterministic)
     __shared__ double sh[7][kThreads];
     for (int k = 0; k < 6; ++k) sh[k][threadIdx.x] = acc[k];
-    sh[6][threadIdx.x] = bad;
+    sh[6][threadIdx.x] = (double)bad;
     __syncthreads();
     for (int stride = kThreads / 2; stride > 0; stride >>= 1) {
         if (threadIdx.x < stride) {
@@ -718,6 +784,19 @@ inline unsigned grid_for(long long N) { return (unsigned)((N + kThreads - 1) / k
 inline bool lanes64(const HostPhys &h) { return (long long)Q * h.N < (1LL << 32) && (!h.links || h.bsolid); }
 inline unsigned grid64(long long cells) { return (unsigned)((2 * cells + kThreads64 - 1) / kThreads64); }
 
+// Densities that the solid sites of a mask present to Eq. 13, into rho.
+template <class R, bool PAIRS>
+void wall_pass(const HostPhys &h, R *rho, const PhysF<R> &p, cudaStream_t s)
+{
+    if (h.n_bsolid > 0)
+        k_wall_rho_list<R, PAIRS><<<grid64(h.n_bsolid), kThreads64, 0, s>>>(rho, p, h.bsolid, (unsigned)h.n_bsolid);
+}
+
+// Threads per CTA of the one-thread-per-cell kernels that run once per call:
+// CTAs of 64 spread a small lattice over more SMs (FP64 above all).
+inline int threads_for(long long N) { return N < 152LL * 4 * kThreads ? 64 : kThreads; }
+inline unsigned grid_by(long long N, int threads) { return (unsigned)((N + threads - 1) / threads); }
+
 // Density pass: rho^a of every fluid cell, then (with a mask) the densities
 // the solid sites present to Eq. 13.
 template <int S>
@@ -725,16 +804,13 @@ void density_pass(const HostPhys &h, const typename Store<S>::T *f, typename Sto
 {
     using R = typename Store<S>::R;
     const PhysF<R> p = make_phys<R>(h);
+    bool lanes = false;
     if constexpr (S == ST_F64) {
-        if (lanes64(h)) {
-            k_density64<<<grid64(h.N), kThreads64, 0, s>>>(f, rho, p);
-            if (h.solid && h.n_bsolid > 0)
-                k_wall_rho64<<<grid64(h.n_bsolid), kThreads64, 0, s>>>(rho, p, h.bsolid, (unsigned)h.n_bsolid);
-            return;
-        }
+        lanes = lanes64(h);
+        if (lanes) k_density64<<<grid64(h.N), kThreads64, 0, s>>>(f, rho, p);
     }
-    k_density<S><<<grid_for(h.N), kThreads, 0, s>>>(f, rho, p);
-    if (h.solid) k_wall_rho<R><<<grid_for(h.N), kThreads, 0, s>>>(rho, p);
+    if (!lanes) k_density<S><<<grid_for(h.N), kThreads, 0, s>>>(f, rho, p);
+    if (h.solid) wall_pass<R, false>(h, rho, p, s);
 }
 
 template <int S>
@@ -779,19 +855,10 @@ cudaError_t step_split_t(const HostPhys &h, const void *fin, void *fout, void *r
 }
 
 template <int S>
-cudaError_t init_t(const HostPhys &h, const double *r1, const double *r2, const double *u, void *f,
-                   void *scratch, cudaStream_t s)
+cudaError_t init_t(const HostPhys &h, const double *r1, const double *r2, const double *u, void *f, cudaStream_t s)
 {
-    using T = typename Store<S>::T;
-    using R = typename Store<S>::R;
-    // the eight rest values per cell fit in the other state copy
-    static_assert(8 * sizeof(R) <= 2 * Q * sizeof(T), "rest values exceed a state copy");
-    R *rest = nullptr;
-    if (!u && scratch) {
-        rest = (R *)scratch;
-        k_rest_values<R><<<grid_for(h.N), kThreads, 0, s>>>(r1, r2, rest, h.N);
-    }
-    k_init_feq<S><<<grid_for(h.N), kThreads, 0, s>>>(r1, r2, u, rest, (T *)f, make_phys<R>(h));
+    const int t = threads_for(h.N);
+    k_init_feq<S><<<grid_by(h.N, t), t, 0, s>>>(r1, r2, u, (typename Store<S>::T *)f, make_phys<typename Store<S>::R>(h));
     return cudaGetLastError();
 }
 
@@ -814,32 +881,51 @@ cudaError_t getpop_t(const HostPhys &h, const void *f, double *dst, cudaStream_t
     return cudaGetLastError();
 }
 
-template <int S>
-cudaError_t moments_t(const HostPhys &h, const void *f, void *rho, int out_f64, void *o1, void *o2,
-                      void *ouF, cudaStream_t s)
+// First pass of the output fields and reductions; with rho also the densities of
+// the solid sites.
+template <int S, class O>
+void sums_pass(const HostPhys &h, const void *f, typename Store<S>::R *rho, typename Store<S>::R *u, O *o1, O *o2,
+               cudaStream_t s)
 {
-    using T = typename Store<S>::T;
     using R = typename Store<S>::R;
     const PhysF<R> p = make_phys<R>(h);
-    const unsigned g = grid_for(h.N);
-    if (ouF) density_pass<S>(h, (const T *)f, (R *)rho, s);
-    if (out_f64)
-        k_moments<S, double><<<g, kThreads, 0, s>>>((const T *)f, (const R *)rho, (double *)o1,
-                                                    (double *)o2, (double *)ouF, p);
-    else
-        k_moments<S, float><<<g, kThreads, 0, s>>>((const T *)f, (const R *)rho, (float *)o1,
-                                                   (float *)o2, (float *)ouF, p);
+    bool lanes = false;
+    if constexpr (S == ST_F64) {
+        lanes = lanes64(h);
+        if (lanes) k_sums64<O><<<grid64(h.N), kThreads64, 0, s>>>((const double *)f, rho, u, o1, o2, p);
+    }
+    if (!lanes) {
+        const int t = threads_for(h.N);
+        k_sums<S, O><<<grid_by(h.N, t), t, 0, s>>>((const typename Store<S>::T *)f, (typename VecOf<R>::T *)rho, u, o1, o2, p);
+    }
+    if (rho && h.solid) wall_pass<R, true>(h, rho, p, s);
+}
+
+template <int S, class O>
+void fields_t(const HostPhys &h, const void *f, void *rho, void *u, O *o1, O *o2, O *ouF, cudaStream_t s)
+{
+    using R = typename Store<S>::R;
+    sums_pass<S, O>(h, f, ouF ? (R *)rho : nullptr, (R *)u, o1, o2, s);
+    if (!ouF) return;
+    const int t = threads_for(h.N);
+    k_uF<R, O><<<grid_by(h.N, t), t, 0, s>>>((const typename VecOf<R>::T *)rho, (const R *)u, ouF, make_phys<R>(h));
+}
+
+template <int S>
+cudaError_t moments_t(const HostPhys &h, const void *f, void *rho, void *u, int out_f64, void *o1, void *o2,
+                      void *ouF, cudaStream_t s)
+{
+    if (out_f64) fields_t<S, double>(h, f, rho, u, (double *)o1, (double *)o2, (double *)ouF, s);
+    else fields_t<S, float>(h, f, rho, u, (float *)o1, (float *)o2, (float *)ouF, s);
     return cudaGetLastError();
 }
 
 template <int S>
-cudaError_t reduce_t(const HostPhys &h, const void *f, void *rho, double *partials, cudaStream_t s)
+cudaError_t reduce_t(const HostPhys &h, const void *f, void *rho, void *u, double *partials, cudaStream_t s)
 {
-    using T = typename Store<S>::T;
     using R = typename Store<S>::R;
-    const PhysF<R> p = make_phys<R>(h);
-    density_pass<S>(h, (const T *)f, (R *)rho, s);
-    k_reduce<S><<<kReduceBlocks, kThreads, 0, s>>>((const T *)f, (const R *)rho, partials, p);
+    sums_pass<S, R>(h, f, (R *)rho, (R *)u, nullptr, nullptr, s);
+    k_reduce<R><<<reduce_grid(h.N), kThreads, 0, s>>>((const typename VecOf<R>::T *)rho, (const R *)u, partials, make_phys<R>(h));
     return cudaGetLastError();
 }
 
@@ -860,15 +946,15 @@ cudaError_t launch_step_split(const HostPhys &p, const void *f_in, void *f_out, 
 }
 
 cudaError_t launch_init_feq(const HostPhys &p, const double *r1, const double *r2, const double *u,
-                            void *f, void *scratch, cudaStream_t s)
+                            void *f, cudaStream_t s)
 {
     switch (p.storage) {
-    case ST_F64: return init_t<ST_F64>(p, r1, r2, u, f, scratch, s);
-    case ST_F32: return init_t<ST_F32>(p, r1, r2, u, f, scratch, s);
-    case ST_F16_DEV: return init_t<ST_F16_DEV>(p, r1, r2, u, f, scratch, s);
-    case ST_BF16_DEV: return init_t<ST_BF16_DEV>(p, r1, r2, u, f, scratch, s);
-    case ST_F16_REL: return init_t<ST_F16_REL>(p, r1, r2, u, f, scratch, s);
-    case ST_BF16_REL: return init_t<ST_BF16_REL>(p, r1, r2, u, f, scratch, s);
+    case ST_F64: return init_t<ST_F64>(p, r1, r2, u, f, s);
+    case ST_F32: return init_t<ST_F32>(p, r1, r2, u, f, s);
+    case ST_F16_DEV: return init_t<ST_F16_DEV>(p, r1, r2, u, f, s);
+    case ST_BF16_DEV: return init_t<ST_BF16_DEV>(p, r1, r2, u, f, s);
+    case ST_F16_REL: return init_t<ST_F16_REL>(p, r1, r2, u, f, s);
+    case ST_BF16_REL: return init_t<ST_BF16_REL>(p, r1, r2, u, f, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -899,21 +985,22 @@ cudaError_t launch_get_populations(const HostPhys &p, const void *f, double *dst
     }
 }
 
-cudaError_t launch_moments(const HostPhys &p, const void *f, void *rho, int out_f64, void *o1, void *o2,
+cudaError_t launch_moments(const HostPhys &p, const void *f, void *rho, void *u, int out_f64, void *o1, void *o2,
                            void *ouF, cudaStream_t s)
 {
     switch (p.storage) {
-    case ST_F64: return moments_t<ST_F64>(p, f, rho, out_f64, o1, o2, ouF, s);
-    case ST_F32: return moments_t<ST_F32>(p, f, rho, out_f64, o1, o2, ouF, s);
-    case ST_F16_DEV: return moments_t<ST_F16_DEV>(p, f, rho, out_f64, o1, o2, ouF, s);
-    case ST_BF16_DEV: return moments_t<ST_BF16_DEV>(p, f, rho, out_f64, o1, o2, ouF, s);
-    case ST_F16_REL: return moments_t<ST_F16_REL>(p, f, rho, out_f64, o1, o2, ouF, s);
-    case ST_BF16_REL: return moments_t<ST_BF16_REL>(p, f, rho, out_f64, o1, o2, ouF, s);
+    case ST_F64: return moments_t<ST_F64>(p, f, rho, u, out_f64, o1, o2, ouF, s);
+    case ST_F32: return moments_t<ST_F32>(p, f, rho, u, out_f64, o1, o2, ouF, s);
+    case ST_F16_DEV: return moments_t<ST_F16_DEV>(p, f, rho, u, out_f64, o1, o2, ouF, s);
+    case ST_BF16_DEV: return moments_t<ST_BF16_DEV>(p, f, rho, u, out_f64, o1, o2, ouF, s);
+    case ST_F16_REL: return moments_t<ST_F16_REL>(p, f, rho, u, out_f64, o1, o2, ouF, s);
+    case ST_BF16_REL: return moments_t<ST_BF16_REL>(p, f, rho, u, out_f64, o1, o2, ouF, s);
     default: return cudaErrorInvalidValue;
     }
 }
 
 int reduce_blocks() { return kReduceBlocks; }
+int reduce_grid(long long N) { return (int)(N < (long long)kReduceBlocks * kThreads ? (N + kThreads - 1) / kThreads : kReduceBlocks); }
 
 cudaError_t launch_mask_setup(const HostPhys &h, const unsigned char *solid, float *wall_rho, unsigned *bfluid,
                               unsigned *bsolid, unsigned long long *counts, cudaStream_t s)
@@ -943,15 +1030,15 @@ cudaError_t launch_density(const HostPhys &h, const void *f, void *rho, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t launch_reduce(const HostPhys &p, const void *f, void *rho, double *partials, cudaStream_t s)
+cudaError_t launch_reduce(const HostPhys &p, const void *f, void *rho, void *u, double *partials, cudaStream_t s)
 {
     switch (p.storage) {
-    case ST_F64: return reduce_t<ST_F64>(p, f, rho, partials, s);
-    case ST_F32: return reduce_t<ST_F32>(p, f, rho, partials, s);
-    case ST_F16_DEV: return reduce_t<ST_F16_DEV>(p, f, rho, partials, s);
-    case ST_BF16_DEV: return reduce_t<ST_BF16_DEV>(p, f, rho, partials, s);
-    case ST_F16_REL: return reduce_t<ST_F16_REL>(p, f, rho, partials, s);
-    case ST_BF16_REL: return reduce_t<ST_BF16_REL>(p, f, rho, partials, s);
+    case ST_F64: return reduce_t<ST_F64>(p, f, rho, u, partials, s);
+    case ST_F32: return reduce_t<ST_F32>(p, f, rho, u, partials, s);
+    case ST_F16_DEV: return reduce_t<ST_F16_DEV>(p, f, rho, u, partials, s);
+    case ST_BF16_DEV: return reduce_t<ST_BF16_DEV>(p, f, rho, u, partials, s);
+    case ST_F16_REL: return reduce_t<ST_F16_REL>(p, f, rho, u, partials, s);
+    case ST_BF16_REL: return reduce_t<ST_BF16_REL>(p, f, rho, u, partials, s);
     default: return cudaErrorInvalidValue;
     }
 }

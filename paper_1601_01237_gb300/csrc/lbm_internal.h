@@ -84,22 +84,21 @@ cudaError_t launch_mask_setup(const HostPhys &h, const unsigned char *solid, flo
 
 // State set-up: populations from (rho1, rho2, u) via f^eq (u may be NULL),
 // or from explicit populations f[a][i][cell] in library order (doubles).
-// scratch (may be NULL): a second state copy, overwritten by the rest values
-// of a state at rest (u == NULL).
 cudaError_t launch_init_feq(const HostPhys &p, const double *rho1, const double *rho2,
-                            const double *u, void *f, void *scratch, cudaStream_t s);
+                            const double *u, void *f, cudaStream_t s);
 cudaError_t launch_set_populations(const HostPhys &p, const double *src, void *f, cudaStream_t s);
 cudaError_t launch_get_populations(const HostPhys &p, const void *f, double *dst, cudaStream_t s);
 
 // Output fields (rho1, rho2, u_F), each pointer optional; out_f64 selects the
-// element type.  Uses rho (scratch) for the density pass.
-cudaError_t launch_moments(const HostPhys &p, const void *f, void *rho, int out_f64,
+// element type.  rho (2*N reals) and u (3*N reals) are scratch.
+cudaError_t launch_moments(const HostPhys &p, const void *f, void *rho, void *u, int out_f64,
                            void *rho1, void *rho2, void *uF, cudaStream_t s);
 
-// FP64 reduction partials: nblocks x 8 doubles
-// (mass1, mass2, px, py, pz, max|uF|, bad-density count, unused).
-int reduce_blocks();
-cudaError_t launch_reduce(const HostPhys &p, const void *f, void *rho, double *partials,
+// FP64 reduction partials: reduce_grid(N) x 8 doubles
+// (mass1, mass2, px, py, pz, max|uF|^2, bad-density count, unused).
+int reduce_blocks();                // at most
+int reduce_grid(long long N);       // of a lattice of N cells
+cudaError_t launch_reduce(const HostPhys &p, const void *f, void *rho, void *u, double *partials,
                           cudaStream_t s);
 
 // Two-kernel step whose density scratch is the library's static device array
@@ -127,9 +126,10 @@ cudaError_t launch_adjoint_rho0(const HostPhys &p, const void *lam, const void *
 // density pass only (rho = sum_i f_i, pull-gathered) into rho
 cudaError_t launch_density(const HostPhys &p, const void *f, void *rho, cudaStream_t s);
 
-// FP64 diagnostics over the density fields in rho (diag_blocks() x
+// FP64 diagnostics over the density fields in rho (diag_grid(N) x
 // diag_slots() partial doubles).
-int diag_blocks();
+int diag_blocks();                  // at most
+int diag_grid(long long N);         // of a lattice of N cells
 int diag_slots();
 cudaError_t launch_pressure(const HostPhys &h, const void *rho, const double center[3], double r_in, double r_out,
                             double *partials, cudaStream_t s);
