@@ -350,6 +350,35 @@ bool build_graph(lbm_lattice *h)
     return ok;
 }
 
+// n >= 2 steps in moment space: the two moment states live in the population
+// copy that does not hold the state, and the last step writes the populations
+// back into the copy that does.  ev (optional, n + 2 events): recorded before
+// the first launch and after each of the n + 1.
+cudaError_t moment_run(lbm_lattice *h, long n, size_t bytes, cudaEvent_t *ev = nullptr)
+{
+    char *m[2] = {(char *)h->f[h->cur ^ 1], (char *)h->f[h->cur ^ 1] + (bytes + 255) / 256 * 256};
+    if (ev) cudaEventRecord(*ev++, h->stream);
+    cudaError_t e = lbm::launch_moment_in(h->phys, h->f[h->cur], m[0], h->stream);
+    if (ev) cudaEventRecord(*ev++, h->stream);
+    for (long t = 1; t < n && e == cudaSuccess; ++t) {
+        e = lbm::launch_moment_step(h->phys, m[(t & 1) ^ 1], m[t & 1], h->stream);
+        if (ev) cudaEventRecord(*ev++, h->stream);
+    }
+    if (e == cudaSuccess) e = lbm::launch_moment_out(h->phys, m[(n & 1) ^ 1], h->f[h->cur], h->stream);
+    if (ev) cudaEventRecord(*ev, h->stream);
+    if (e == cudaSuccess) h->steps += n;
+    return e;
+}
+
+// Bytes of a moment state if the lattice's next n steps run in moment space (two
+// of them fit the free population copy), else 0.
+size_t moment_run_bytes(const lbm_lattice *h, long n)
+{
+    if (!h->use_fused || n < 2) return 0;
+    const size_t b = lbm::moment_bytes(h->phys);
+    return 2 * ((b + 255) / 256 * 256) <= lbm::state_bytes(h->phys.storage, h->phys.N) ? b : 0;
+}
+
 }  // namespace
 
 lbm_status lbm_step(lbm_lattice *h, long n_steps)
@@ -357,6 +386,10 @@ lbm_status lbm_step(lbm_lattice *h, long n_steps)
     if (!h) return fail(LBM_EINVAL, "lbm_step: NULL handle");
     if (n_steps < 0) return fail(LBM_EINVAL, "lbm_step: n_steps = %ld < 0", n_steps);
     DeviceGuard g(h->device);
+    if (const size_t mb = moment_run_bytes(h, n_steps)) {
+        const cudaError_t e = moment_run(h, n_steps, mb);
+        return e == cudaSuccess ? LBM_OK : cuda_fail(e, "lbm_step: launch");
+    }
     long t = 0;
     auto plain = [&](long upto) -> lbm_status {
         for (; t < upto; ++t) {
@@ -392,15 +425,20 @@ lbm_status lbm_step_timed(lbm_lattice *h, long n_steps, double kernel_ms[4], lon
         return fail(LBM_EINVAL, "lbm_step_timed: NULL argument");
     if (n_steps <= 0) return fail(LBM_EINVAL, "lbm_step_timed: n_steps = %ld must be > 0", n_steps);
     DeviceGuard g(h->device);
-    const int kinds = h->use_fused ? 1 : 2;
-    const size_t nev = (size_t)n_steps * (kinds + 1);
+    const size_t mb = moment_run_bytes(h, n_steps);
+    const int kinds = mb ? 3 : (h->use_fused ? 1 : 2);
+    const size_t nev = mb ? (size_t)n_steps + 2 : (size_t)n_steps * (kinds + 1);
     std::vector<cudaEvent_t> ev(nev, nullptr);
     lbm_status st = LBM_OK;
     for (size_t k = 0; k < nev && st == LBM_OK; ++k) {
         cudaError_t e = cudaEventCreate(&ev[k]);
         if (e != cudaSuccess) st = cuda_fail(e, "lbm_step_timed: event");
     }
-    for (long t = 0; t < n_steps && st == LBM_OK; ++t) {
+    if (mb && st == LBM_OK) {
+        const cudaError_t e = moment_run(h, n_steps, mb, ev.data());
+        if (e != cudaSuccess) st = cuda_fail(e, "lbm_step_timed: launch");
+    }
+    for (long t = 0; t < n_steps && !mb && st == LBM_OK; ++t) {
         cudaEvent_t *evt = &ev[(size_t)t * (kinds + 1)];
         cudaError_t e;
         if (h->use_fused)
@@ -419,7 +457,16 @@ lbm_status lbm_step_timed(lbm_lattice *h, long n_steps, double kernel_ms[4], lon
         static const char *kFused[1] = {"k_step_fused"};
         static const char *kSplit[2] = {"k_density", "k_collide"};
         for (int k = 0; k < 4; ++k) { kernel_ms[k] = 0; launches[k] = 0; names[k] = nullptr; }
-        for (long t = 0; t < n_steps && st == LBM_OK; ++t)
+        static const char *kMoment[3] = {"k_step_moment", "k_moment_in", "k_moment_out"};
+        for (long t = 0; mb && t <= n_steps && st == LBM_OK; ++t) {
+            const int k = t == 0 ? 1 : (t == n_steps ? 2 : 0);
+            float ms = 0;
+            cudaError_t e = cudaEventElapsedTime(&ms, ev[(size_t)t], ev[(size_t)t + 1]);
+            if (e != cudaSuccess) { st = cuda_fail(e, "lbm_step_timed: elapsed"); break; }
+            kernel_ms[k] += ms;
+            launches[k] += 1;
+        }
+        for (long t = 0; t < n_steps && !mb && st == LBM_OK; ++t)
             for (int k = 0; k < kinds; ++k) {
                 float ms = 0;
                 cudaError_t e = cudaEventElapsedTime(&ms, ev[(size_t)t * (kinds + 1) + k],
@@ -428,7 +475,7 @@ lbm_status lbm_step_timed(lbm_lattice *h, long n_steps, double kernel_ms[4], lon
                 kernel_ms[k] += ms;
                 launches[k] += 1;
             }
-        for (int k = 0; k < kinds; ++k) names[k] = h->use_fused ? kFused[k] : kSplit[k];
+        for (int k = 0; k < kinds; ++k) names[k] = mb ? kMoment[k] : (h->use_fused ? kFused[k] : kSplit[k]);
         *n_kinds = kinds;
     }
     for (cudaEvent_t e : ev)
@@ -733,12 +780,11 @@ lbm_status lbm_record(lbm_lattice *h, long n_steps, int ckpt_every)
         CK(cudaMalloc((void **)&h->ws_part, sizeof(double) * 4 * lbm::adjoint_blocks(h->phys.storage)), "lbm_record: partials");
     }
     h->rec_at_rest = h->init_at_rest && h->steps == 0;
-    for (long t = 0; t < n_steps; ++t) {
-        if (t % ckpt_every == 0)
-            CK(cudaMemcpyAsync((char *)h->ckpt + sb * (size_t)(t / ckpt_every), h->f[h->cur], sb,
-                               cudaMemcpyDeviceToDevice, h->stream),
-               "lbm_record: checkpoint");
-        lbm_status st = lbm_step(h, 1);
+    for (long t = 0; t < n_steps; t += ckpt_every) {
+        CK(cudaMemcpyAsync((char *)h->ckpt + sb * (size_t)(t / ckpt_every), h->f[h->cur], sb,
+                           cudaMemcpyDeviceToDevice, h->stream),
+           "lbm_record: checkpoint");
+        lbm_status st = lbm_step(h, std::min<long>(ckpt_every, n_steps - t));
         if (st != LBM_OK) return st;
     }
     CK(cudaStreamSynchronize(h->stream), "lbm_record: sync");

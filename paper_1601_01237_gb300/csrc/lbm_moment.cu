@@ -1,0 +1,480 @@
+// Runs of steps in moment space (FP32 populations, exact-difference forcing).
+//
+// Under the regularized operator a step reads its 38 populations only to form
+// the densities, the mixture momentum and (for tau != 1) the second moments
+// of each component, and the post-collision populations are a polynomial in
+// them and in the densities' gradient; at tau = 1 that holds for every
+// operator.  So between the first and the last step of a call nothing else
+// has to travel through memory: a run of n steps is
+//   k_moment_in    populations -> moments m(t) of the gathered populations,
+//   k_step_moment  m(t) -> m(t + 1), n - 1 times,
+//   k_moment_out   m(t + n - 1) -> populations after its collision,
+// with 5 values per cell at tau = 1 (rho^1, rho^2, u; 40 bytes per cell and step
+// instead of 304) and 17 regularized (with sum c c f of both components; 136
+// bytes).  Every value is held and every sum taken in FP32, as in the
+// population steps; the state at the end of the call is the population state.
+// us per step in calls of 10 (512^3), 20 (256^3) and 100 steps, population steps and
+// these: tau = 1 512^3 6723 / 3100, 256^3 842 / 402, 128^3 119 / 66, 96^3 52 / 36,
+// regularized 256^3 883 / 624, 384 x 512 x 512 with walls 5900 / 3770.
+#include <cuda_runtime.h>
+
+#include <atomic>
+
+#include "collide.cuh"
+#include "d3q19.cuh"
+#include "lbm_internal.h"
+
+namespace lbm {
+
+namespace {
+
+// Moment state of N cells: pairs rho, (ux, uy), uz, and NP pairs of second
+// moments (xx, yy, zz, xy, xz, yz), one array behind the other.
+template <int KIND>
+struct MomentState {
+    static constexpr int NP = RegMoments<PairF32, KIND>::n;
+    static_assert(KIND == COLL_EQ || KIND == COLL_REG, "operators that act on moments alone");
+    float2 *rho, *uxy, *P;
+    float *uz;
+    __host__ __device__ MomentState(void *base, long long N)
+    {
+        rho = (float2 *)base;
+        uxy = rho + N;
+        P = uxy + N;                 // P[k N + cell]
+        uz = (float *)(P + (long long)NP * N);
+    }
+};
+template <int KIND>
+constexpr size_t moment_floats() { return 5 + 2 * (size_t)RegMoments<PairF32, KIND>::n; }
+
+struct Nb3 {
+    unsigned cell, xo[3], yo[3], zo[3];
+    bool zlo, zhi;
+};
+
+__device__ __forceinline__ Nb3 nb3(const Phys<float> &p, unsigned cell)
+{
+    const unsigned nx = (unsigned)p.nx, ny = (unsigned)p.ny, nz = (unsigned)p.nz, plane = nx * ny;
+    const unsigned z = cell / plane, rem = cell - z * plane, y = rem / nx, x = rem - y * nx;
+    Nb3 n;
+    n.cell = cell;
+    n.xo[0] = x == 0 ? nx - 1 : x - 1;
+    n.xo[1] = x;
+    n.xo[2] = x == nx - 1 ? 0 : x + 1;
+    n.yo[0] = (y == 0 ? ny - 1 : y - 1) * nx;
+    n.yo[1] = y * nx;
+    n.yo[2] = (y == ny - 1 ? 0 : y + 1) * nx;
+    n.zo[0] = (z == 0 ? nz - 1 : z - 1) * plane;
+    n.zo[1] = z * plane;
+    n.zo[2] = (z == nz - 1 ? 0 : z + 1) * plane;
+    n.zlo = p.wall_z && z == 0;
+    n.zhi = p.wall_z && z == nz - 1;
+    return n;
+}
+
+constexpr int kThreadsM = 256;
+
+// One thread per cell, bound by the 152 bytes it gathers.
+template <int KIND>
+__global__ void __launch_bounds__(kThreadsM)
+k_moment_in(const float *__restrict__ f, MomentState<KIND> m, Phys<float> p)
+{
+    const unsigned cell = blockIdx.x * kThreadsM + threadIdx.x, N32 = (unsigned)p.N;
+    if (cell >= N32) return;
+    const Nb3 n = nb3(p, cell);
+    float2 v[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const bool wall = (cz(i) == 1 && n.zlo) || (cz(i) == -1 && n.zhi);
+        const unsigned src = n.zo[1 - cz(i)] + n.yo[1 - cy(i)] + n.xo[1 - cx(i)];
+        v[i] = ld_pair_f32(f + 2 * (size_t)(wall ? (unsigned)opp(i) * N32 + cell : (unsigned)i * N32 + src));
+    }
+    const float2 r = density(v);
+    float jx, jy, jz;
+    momentum(PairF32(), v, jx, jy, jz);
+    const float inv = 1.0f / (r.x + r.y);
+    m.rho[cell] = r;
+    m.uxy[cell] = make_float2(jx * inv, jy * inv);
+    m.uz[cell] = jz * inv;
+    RegMoments<PairF32, KIND> mo;
+    mo.of(v);
+#pragma unroll
+    for (int k = 0; k < MomentState<KIND>::NP; ++k) m.P[(size_t)k * N32 + cell] = mo.m[k];
+}
+
+// One thread per cell, bound by the 152 bytes it stores.
+template <int KIND>
+__global__ void __launch_bounds__(kThreadsM)
+k_moment_out(MomentState<KIND> m, float *__restrict__ f, Phys<float> p)
+{
+    const unsigned cell = blockIdx.x * kThreadsM + threadIdx.x, N32 = (unsigned)p.N;
+    if (cell >= N32) return;
+    const Nb3 n = nb3(p, cell);
+    const float2 rs = make_float2(p.rho_s[0], p.rho_s[1]);
+    const float2 *__restrict__ rho = m.rho;
+    auto at = [&](int dx, int dy, int dz) {
+        if ((dz == -1 && n.zlo) || (dz == 1 && n.zhi))
+            return p.wall_mirror ? vadd(__ldg(rho + n.zo[1] + n.yo[1 + dy] + n.xo[1 + dx]), rs) : rs;
+        return __ldg(rho + n.zo[1 + dz] + n.yo[1 + dy] + n.xo[1 + dx]);
+    };
+    float2 S[3];
+    interaction<PairF32>([&](int i) { return vsub(at(cx(i), cy(i), cz(i)), at(-cx(i), -cy(i), -cz(i))); }, S);
+    const float2 So[3] = {vswap(S[0]), vswap(S[1]), vswap(S[2])};
+    const float2 r = m.rho[cell], uxy = m.uxy[cell];
+    RegMoments<PairF32, KIND> mo;
+#pragma unroll
+    for (int k = 0; k < MomentState<KIND>::NP; ++k) mo.m[k] = m.P[(size_t)k * N32 + cell];
+    auto get = [](int) { return make_float2(0.f, 0.f); };
+    auto put = [&](int i, float2 v) { *reinterpret_cast<float2 *>(f + 2 * (size_t)((unsigned)i * N32 + cell)) = v; };
+    collide_cell<PairF32, KIND, FORCE_EDM, false>(PairF32(), p, r, 0.f, uxy.x, uxy.y, m.uz[cell], So, mo, get, put);
+}
+
+// ---------------------------------------------------------------------------
+// m(t) -> m(t + 1).  A CTA owns 30 x 14 columns and marches along z over lz
+// planes; its 32 x 16 threads are those columns and the ring around them, one
+// thread per column.  Per plane p:
+//   a. each thread completes the interaction sums of its cell from the density
+//      planes p - 1, p, p + 1 (each plane is read once from shared memory and
+//      adds to the sums of the three planes that see it), collides the cell and
+//      leaves the 16 pairs of its post-collision populations that move in x or
+//      y in shared memory;
+//   -- barrier --
+//   b. each thread picks up the 16 pairs that stream into its column, from the
+//      plane's own direction group (c_z = 0), into plane p + 1 (c_z = +1) and into
+//      plane p - 1 (c_z = -1), as sums and differences of opposite sources, adds
+//      them to the moments of those planes and stores the moments of plane
+//      p - 1, which are then complete;
+//   -- barrier --
+// The next plane's moments and the density plane after it are loaded one
+// iteration ahead.  The ring's collisions are computed by every neighbouring
+// CTA too (512 collisions for 420 cells), and a CTA computes one plane more at
+// each end of its chunk; densities reach one cell further, loaded by 100 of
+// the threads.
+constexpr int kEX = 32, kEY = 16, kThreadsS = kEX * kEY;   // threads: tile and ring
+constexpr int kOX = kEX - 2, kOY = kEY - 2;                // tile
+constexpr int kRX = kEX + 2, kRY = kEY + 2;                // densities
+constexpr int kRim = 2 * kRX + 2 * kEY;                    // cells of the density plane beyond the threads' own
+constexpr int kPad = 40;                                   // a neighbour's offset is at most 33
+constexpr int kMove = 16;
+static_assert(kRim <= kThreadsS && kPad >= kEX + 1, "");
+
+struct MomentSmem {
+    float2 f[kMove][kPad + kThreadsS + kPad];   // moving populations of the current plane
+    float2 rho[2][kRY][kRX];                    // density planes p + 1 and p + 2
+};
+
+// The direction with given components.
+__host__ __device__ constexpr int dir_of(int x, int y, int z)
+{
+    for (int i = 0; i < Q; ++i)
+        if (cx(i) == x && cy(i) == y && cz(i) == z) return i;
+    return -1;
+}
+
+constexpr int kUp = dir_of(0, 0, 1), kDown = dir_of(0, 0, -1);
+static_assert(kUp == 5 && kDown == 6, "");
+// Place of a moving direction in MomentSmem::f (put() below has the same rule).
+// A template, so that it is a constant: the search is not folded at run time
+// (the kernel took 1744 us per step at 256^3 with it, 382 without).
+template <int X, int Y, int Z>
+struct MoveSlot {
+    static constexpr int i = dir_of(X, Y, Z), value = i < kUp ? i - 1 : i - 3;
+    static_assert(X != 0 || Y != 0, "moves in x or y");
+};
+
+// Moments of a plane's cells as they collect: density and second moments as
+// pairs, momentum of the mixture.
+template <int KIND>
+struct Collect {
+    static constexpr int NP = RegMoments<PairF32, KIND>::n;
+    float2 rho, P[NP > 0 ? NP : 1];
+    float jx, jy, jz;
+    __device__ __forceinline__ void zero()
+    {
+        rho = make_float2(0.f, 0.f);
+        jx = jy = jz = 0.f;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) P[k] = make_float2(0.f, 0.f);
+    }
+    // the five populations of a group c_z = Z = +-1: the one that stays in its
+    // column, and those from the columns at -x, +x, -y, +y (moving the other way)
+    template <int Z>
+    __device__ __forceinline__ void add_group(float2 n0, float2 xp, float2 xm, float2 yp, float2 ym)
+    {
+        const float2 ex = vadd(xp, xm), dx = vsub(xp, xm), ey = vadd(yp, ym), dy = vsub(yp, ym);
+        const float2 s = vadd(n0, vadd(ex, ey));
+        rho = vadd(rho, s);
+        jx += dx.x + dx.y;
+        jy += dy.x + dy.y;
+        if (Z > 0) jz += s.x + s.y;
+        else jz -= s.x + s.y;
+        if constexpr (NP > 0) {
+            P[0] = vadd(P[0], ex);
+            P[1] = vadd(P[1], ey);
+            P[2] = vadd(P[2], s);
+            P[4] = Z > 0 ? vadd(P[4], dx) : vsub(P[4], dx);
+            P[5] = Z > 0 ? vadd(P[5], dy) : vsub(P[5], dy);
+        }
+    }
+};
+
+template <int KIND, bool WALLZ>
+__global__ void __launch_bounds__(kThreadsS, KIND == COLL_EQ ? 2 : 1)
+k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, int ntx, int lz)
+{
+    constexpr int NP = MomentState<KIND>::NP;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    MomentSmem &sm = *reinterpret_cast<MomentSmem *>(smem_raw);
+    const int tid = threadIdx.x, ex = tid % kEX, ey = tid / kEX, at = kPad + tid;
+    const int nx = p.nx, ny = p.ny, nz = p.nz;
+    const unsigned plane = (unsigned)nx * (unsigned)ny, N32 = (unsigned)p.N;
+    const int x0 = (int)(blockIdx.x % (unsigned)ntx) * kOX, y0 = (int)(blockIdx.x / (unsigned)ntx) * kOY;
+    const int z0 = (int)blockIdx.y * lz, z1 = min(z0 + lz, nz);
+    const bool stores = ex >= 1 && ex <= kOX && ey >= 1 && ey <= kOY && x0 + ex - 1 < nx && y0 + ey - 1 < ny;
+    auto column = [&](int x, int y) {   // periodic in x and y
+        x %= nx; if (x < 0) x += nx;
+        y %= ny; if (y < 0) y += ny;
+        return (unsigned)y * (unsigned)nx + (unsigned)x;
+    };
+    const unsigned col = column(x0 + ex - 1, y0 + ey - 1);
+    // the rim cell of the density plane that this thread also loads
+    int rx = 0, ry = 0;
+    if (tid < kRX) { rx = tid; ry = 0; }
+    else if (tid < 2 * kRX) { rx = tid - kRX; ry = kRY - 1; }
+    else { const int k = tid - 2 * kRX; rx = (k & 1) ? kRX - 1 : 0; ry = 1 + (k >> 1); }
+    const bool rim = tid < kRim;
+    const unsigned rcol = rim ? column(x0 + rx - 2, y0 + ry - 2) : 0u;
+    // offset of plane q: periodic, or the mirror plane of a wall site
+    auto offset = [&](int q) {
+        if (WALLZ) q = q < 0 ? 0 : (q >= nz ? nz - 1 : q);
+        else { q %= nz; if (q < 0) q += nz; }
+        return (unsigned)q * plane;
+    };
+    const float2 rs = make_float2(p.rho_s[0], p.rho_s[1]);
+    auto present = [&](int q, float2 r) {   // what plane q presents to Eq. 13
+        if (WALLZ && (q < 0 || q >= nz)) return p.wall_mirror ? vadd(r, rs) : rs;
+        return r;
+    };
+    // density plane z0 - 2 into its slot, z0 - 1 into registers
+    const int first = z0 - 1;   // first plane that collides
+    float2 r_next, h_next = make_float2(0.f, 0.f);
+    {
+        const unsigned o = offset(first - 1);
+        sm.rho[(first - 1) & 1][ey + 1][ex + 1] = present(first - 1, in.rho[o + col]);
+        if (rim) sm.rho[(first - 1) & 1][ry][rx] = present(first - 1, in.rho[o + rcol]);
+        const unsigned o1 = offset(first);
+        r_next = in.rho[o1 + col];
+        if (rim) h_next = in.rho[o1 + rcol];
+    }
+    float2 uxy = make_float2(0.f, 0.f);
+    float uz = 0.f;
+    RegMoments<PairF32, KIND> mo;
+    float2 S[3], lo[3], r_own = make_float2(0.f, 0.f);   // sums of plane p so far, and what plane p adds to p + 1's
+#pragma unroll
+    for (int d = 0; d < 3; ++d) S[d] = lo[d] = make_float2(0.f, 0.f);
+    Collect<KIND> c0, c1;   // planes p - 1 and p
+    c0.zero();
+    c1.zero();
+    const float2 w1 = PairF32::dup(w<float>(1)), w2 = PairF32::dup(w<float>(7));
+    __syncthreads();
+    // p = first - 2, first - 1: only the density planes first - 1 and first come in
+    for (int q = first - 2; q <= z1; ++q) {
+        // ---- a. plane q + 1's densities are in place: they complete plane q's
+        //      sums and start plane q + 1's and q + 2's
+        const bool collides = q >= first && !(WALLZ && (q < 0 || q >= nz));
+        // (density plane q + 2 into its slot; its last readers passed two barriers ago)
+        sm.rho[(q + 2) & 1][ey + 1][ex + 1] = present(q + 2, r_next);
+        if (rim) sm.rho[(q + 2) & 1][ry][rx] = present(q + 2, h_next);
+        // loads for the next iteration
+        const float2 uxy_c = uxy;
+        const float uz_c = uz;
+        const RegMoments<PairF32, KIND> mo_c = mo;
+        if (q < z1) {
+            const unsigned o3 = offset(q + 3), o1 = offset(q + 1);
+            r_next = in.rho[o3 + col];
+            if (rim) h_next = in.rho[o3 + rcol];
+            uxy = in.uxy[o1 + col];
+            uz = in.uz[o1 + col];
+#pragma unroll
+            for (int k = 0; k < NP; ++k) mo.m[k] = in.P[(size_t)k * N32 + o1 + col];
+        }
+        float2 So[3], rc;
+        {
+            const float2(*R)[kRX] = &sm.rho[(q + 1) & 1][ey];   // rows ey, ey + 1, ey + 2: y - 1, y, y + 1
+            const float2 xp = R[1][ex + 2], xm = R[1][ex], yp = R[2][ex + 1], ym = R[0][ex + 1];
+            rc = R[1][ex + 1];
+            const float2 dx = vsub(xp, xm), dy = vsub(yp, ym);
+            const float2 a = vsub(R[2][ex + 2], R[0][ex]), b = vsub(R[0][ex + 2], R[2][ex]);   // (1,1), (1,-1)
+            const float2 Z = vfma(w1, rc, vmul(w2, vadd(vadd(xp, xm), vadd(yp, ym))));
+            const float2 lx = vmul(w2, dx), ly = vmul(w2, dy);
+            // plane q: this plane lies above it
+            So[0] = vswap(vadd(S[0], lx));
+            So[1] = vswap(vadd(S[1], ly));
+            So[2] = vswap(vadd(S[2], Z));
+            // plane q + 1: its own plane
+            S[0] = vadd(lo[0], vfma(w1, dx, vmul(w2, vadd(a, b))));
+            S[1] = vadd(lo[1], vfma(w1, dy, vmul(w2, vsub(a, b))));
+            S[2] = lo[2];
+            // plane q + 2: this plane lies below it
+            lo[0] = lx;
+            lo[1] = ly;
+            lo[2] = vsub(make_float2(0.f, 0.f), Z);
+        }
+        const float2 r = r_own;   // density of plane q at this column
+        r_own = rc;
+        float2 f0, fu, fd;        // populations that stay in the column: c_z = 0, +1, -1
+        if (collides) {
+            auto get = [](int) { return make_float2(0.f, 0.f); };
+            auto put = [&](int i, float2 v) {
+                if (i == 0) f0 = v;
+                else if (i == kUp) fu = v;
+                else if (i == kDown) fd = v;
+                else sm.f[i < kUp ? i - 1 : i - 3][at] = v;
+            };
+            collide_cell<PairF32, KIND, FORCE_EDM, false>(PairF32(), p, r, 0.f, uxy_c.x, uxy_c.y, uz_c, So, mo_c, get, put);
+        }
+        __syncthreads();
+        // ---- b. what streams into this column
+        Collect<KIND> c2;         // plane q + 1
+        c2.zero();
+        if (collides) {
+            // the population (X, Y, Z) out of column - (X, Y), and the cell's own
+#define LBM_FROM(X, Y, Z) sm.f[MoveSlot<X, Y, Z>::value][at - (X) - (Y) * kEX]
+#define LBM_OWN(X, Y, Z) sm.f[MoveSlot<X, Y, Z>::value][at]
+            {   // c_z = 0
+                const float2 xp = LBM_FROM(1, 0, 0), xm = LBM_FROM(-1, 0, 0), yp = LBM_FROM(0, 1, 0), ym = LBM_FROM(0, -1, 0);
+                const float2 a = LBM_FROM(1, 1, 0), b = LBM_FROM(-1, -1, 0), c = LBM_FROM(1, -1, 0), d = LBM_FROM(-1, 1, 0);
+                const float2 ab = vadd(a, b), cd = vadd(c, d), da = vsub(a, b), dc = vsub(c, d);
+                const float2 ex2 = vadd(xp, xm), ey2 = vadd(yp, ym), dg = vadd(ab, cd);
+                const float2 jx = vadd(vsub(xp, xm), vadd(da, dc)), jy = vadd(vsub(yp, ym), vsub(da, dc));
+                c1.rho = vadd(c1.rho, vadd(f0, vadd(vadd(ex2, ey2), dg)));
+                c1.jx += jx.x + jx.y;
+                c1.jy += jy.x + jy.y;
+                if constexpr (NP > 0) {
+                    c1.P[0] = vadd(c1.P[0], vadd(ex2, dg));
+                    c1.P[1] = vadd(c1.P[1], vadd(ey2, dg));
+                    c1.P[3] = vsub(ab, cd);
+                }
+            }
+            c2.template add_group<1>(fu, LBM_FROM(1, 0, 1), LBM_FROM(-1, 0, 1), LBM_FROM(0, 1, 1), LBM_FROM(0, -1, 1));
+            c0.template add_group<-1>(fd, LBM_FROM(1, 0, -1), LBM_FROM(-1, 0, -1), LBM_FROM(0, 1, -1), LBM_FROM(0, -1, -1));
+            if (WALLZ) {   // half-way bounce-back: the cell's own populations come back reversed
+                if (q == 0)
+                    c1.template add_group<1>(fd, LBM_OWN(-1, 0, -1), LBM_OWN(1, 0, -1), LBM_OWN(0, -1, -1), LBM_OWN(0, 1, -1));
+                if (q == nz - 1)
+                    c1.template add_group<-1>(fu, LBM_OWN(-1, 0, 1), LBM_OWN(1, 0, 1), LBM_OWN(0, -1, 1), LBM_OWN(0, 1, 1));
+            }
+#undef LBM_FROM
+#undef LBM_OWN
+        }
+        if (q > z0 && stores) {   // plane q - 1 is complete
+            const unsigned cell = (unsigned)(q - 1) * plane + col;
+            const float inv = 1.0f / (c0.rho.x + c0.rho.y);
+            out.rho[cell] = c0.rho;
+            out.uxy[cell] = make_float2(c0.jx * inv, c0.jy * inv);
+            out.uz[cell] = c0.jz * inv;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) out.P[(size_t)k * N32 + cell] = c0.P[k];
+        }
+        c0 = c1;
+        c1 = c2;
+        __syncthreads();
+    }
+}
+
+Phys<float> make_phys_m(const HostPhys &h)
+{
+    Phys<float> p;
+    p.nx = h.nx; p.ny = h.ny; p.nz = h.nz; p.N = h.N;
+    p.wall_z = h.wall_z;
+    p.wall_mirror = h.wall_mirror;
+    p.omega[0] = (float)(1.0 / h.tau[0]);
+    p.omega[1] = (float)(1.0 / h.tau[1]);
+    p.G12 = (float)h.G12; p.G21 = (float)h.G21;
+    for (int d = 0; d < 3; ++d) p.gext[d] = (float)h.gext[d];
+    p.rho_s[0] = (float)h.rho_s[0]; p.rho_s[1] = (float)h.rho_s[1];
+    p.rho0 = 0.f;
+    return p;
+}
+
+// Planes per CTA: equal chunks, the fewest waves x (planes + 4) (the collisions
+// beyond the two ends of a chunk and the density planes before it).
+int moment_planes(long long cols, int nz, long long slots)
+{
+    int best = nz;
+    long long cbest = -1;
+    for (int nch = (nz + 127) / 128; nch <= nz; ++nch) {
+        const int lz = (nz + nch - 1) / nch;
+        if (lz < 4 && nch > 1) break;
+        const long long ctas = cols * ((nz + lz - 1) / lz), c = ((ctas + slots - 1) / slots) * (lz + 4);
+        if (cbest < 0 || c < cbest) { cbest = c; best = lz; }
+    }
+    return best;
+}
+
+constexpr int kMaxAttrDevices = 64;
+
+template <int KIND, bool WALLZ>
+cudaError_t launch_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
+{
+    static std::atomic<int> attr_set[kMaxAttrDevices];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool cached = dev >= 0 && dev < kMaxAttrDevices;
+    if (!cached || !attr_set[dev].load(std::memory_order_acquire)) {
+        e = cudaFuncSetAttribute((const void *)k_step_moment<KIND, WALLZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(MomentSmem));
+        if (e != cudaSuccess) return e;
+        if (cached) attr_set[dev].store(1, std::memory_order_release);
+    }
+    const int ntx = (h.nx + kOX - 1) / kOX, nty = (h.ny + kOY - 1) / kOY;
+    const long long cols = (long long)ntx * nty;
+    const int lz = moment_planes(cols, h.nz, (KIND == COLL_EQ ? 2LL : 1LL) * current_device_sms());
+    k_step_moment<KIND, WALLZ><<<dim3((unsigned)cols, (unsigned)((h.nz + lz - 1) / lz)), kThreadsS, sizeof(MomentSmem), s>>>(
+        MomentState<KIND>(const_cast<void *>(in), h.N), MomentState<KIND>(out, h.N), make_phys_m(h), ntx, lz);
+    return cudaGetLastError();
+}
+
+bool tau_one(const HostPhys &h) { return (float)(1.0 / h.tau[0]) == 1.0f && (float)(1.0 / h.tau[1]) == 1.0f; }
+
+inline unsigned grid_m(long long N) { return (unsigned)((N + kThreadsM - 1) / kThreadsM); }
+
+}  // namespace
+
+size_t moment_bytes(const HostPhys &h)
+{
+    if (h.storage != ST_F32 || h.forcing != FORCE_EDM || h.links || !fused_supported(h) || use_box(h)) return 0;
+    const long long cols = (long long)((h.nx + kOX - 1) / kOX) * ((h.ny + kOY - 1) / kOY);
+    if (cols >= (1LL << 31) || h.nz > 4 * 65535) return 0;   // grid limits
+    const size_t N = (size_t)h.N;
+    if (tau_one(h)) return sizeof(float) * moment_floats<COLL_EQ>() * N;
+    if (h.collision == LBM_REGULARIZED) return sizeof(float) * moment_floats<COLL_REG>() * N;
+    return 0;
+}
+
+cudaError_t launch_moment_in(const HostPhys &h, const void *f, void *m, cudaStream_t s)
+{
+    if (tau_one(h))
+        k_moment_in<COLL_EQ><<<grid_m(h.N), kThreadsM, 0, s>>>((const float *)f, MomentState<COLL_EQ>(m, h.N), make_phys_m(h));
+    else
+        k_moment_in<COLL_REG><<<grid_m(h.N), kThreadsM, 0, s>>>((const float *)f, MomentState<COLL_REG>(m, h.N), make_phys_m(h));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_moment_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
+{
+    if (tau_one(h)) return h.wall_z ? launch_step<COLL_EQ, true>(h, in, out, s) : launch_step<COLL_EQ, false>(h, in, out, s);
+    return h.wall_z ? launch_step<COLL_REG, true>(h, in, out, s) : launch_step<COLL_REG, false>(h, in, out, s);
+}
+
+cudaError_t launch_moment_out(const HostPhys &h, const void *m, void *f, cudaStream_t s)
+{
+    if (tau_one(h))
+        k_moment_out<COLL_EQ><<<grid_m(h.N), kThreadsM, 0, s>>>(MomentState<COLL_EQ>(const_cast<void *>(m), h.N), (float *)f, make_phys_m(h));
+    else
+        k_moment_out<COLL_REG><<<grid_m(h.N), kThreadsM, 0, s>>>(MomentState<COLL_REG>(const_cast<void *>(m), h.N), (float *)f, make_phys_m(h));
+    return cudaGetLastError();
+}
+
+}  // namespace lbm

@@ -1,7 +1,7 @@
 """The step's kernels by collision kind, geometry, forcing and format against
-the FP64 oracle: the marching kernel (lattices large enough for it) with its
-moment and tau = 1 instances, the box kernel of small and thin lattices, and
-the half-cell FP64 kernels."""
+the FP64 oracle: the marching kernel (lattices large enough for it, a call per
+step), runs in moment space (the same lattices, several steps per call), the
+box kernel of small and thin lattices, and the half-cell FP64 kernels."""
 import numpy as np
 import pytest
 
@@ -11,9 +11,10 @@ from paper_1601_01237_gb300 import workloads as wl
 pytestmark = pytest.mark.gpu
 
 # box kernel: one cell, one box, remainders along every axis, one layer along
-# y or z, columns; marching kernel: tile and chunk remainders
+# y or z, columns; marching kernel and moment runs: tile and chunk remainders,
+# fewer planes than a chunk's overlap
 SMALL = [(1, 1, 1), (1, 9, 17), (1, 1, 40), (9, 1, 17), (4, 8, 8), (7, 9, 11), (13, 2, 3), (2, 5, 70)]
-MARCH = [(61, 65, 70)]
+MARCH = [(61, 65, 70), (2, 200, 200), (3, 47, 900)]
 KINDS = [("bgk", (1.0, 1.0)), ("regularized", (0.7, 1.2)), ("regularized3", (0.8, 0.9)), ("bgk", (1.0, 0.8))]
 GEOMETRY = ["periodic", "mirror", "potential", "mask_mirror", "mask_potential"]
 # four steps of about 20 dependent roundings per population, relative to the
@@ -35,7 +36,7 @@ def _geometry(kind, shape):
     return kw, solid
 
 
-def _compare(shape, geometry, collision, tau, forcing, storage, steps, tol, **extra):
+def _compare(shape, geometry, collision, tau, forcing, storage, steps, tol, calls=None, **extra):
     perm = direction_map()
     geo, solid = _geometry(geometry, shape)
     r1, r2, u = wl.random_state(shape, seed=7, rho_lo=0.3, rho_hi=0.7, u_max=0.03)
@@ -43,7 +44,10 @@ def _compare(shape, geometry, collision, tau, forcing, storage, steps, tol, **ex
         u[solid != 0] = 0.0
     kw = dict(tau=tau, G12=-1.2, G21=-1.1, g_ext=(1e-4, -2e-4, 5e-5), collision=collision, forcing=forcing, **geo)
     _, f = oracle_run(shape, r1, r2, u, steps, solid=solid, **kw)
-    lat = gpu_run(shape, r1, r2, u, steps, storage=storage, solid=solid, **kw, **extra)
+    lat = gpu_run(shape, r1, r2, u, 0, storage=storage, solid=solid, **kw, **extra)
+    for n in calls or [steps]:
+        lat.step(n)
+    assert lat.step_count() == steps
     g = lat.get_populations()
     lat.close()
     ref = f[:, perm]
@@ -66,7 +70,18 @@ def test_small_and_thin_against_oracle(gpu_lib, geometry, collision, tau, forcin
 @pytest.mark.parametrize("geometry", ["periodic", "mirror", "mask_mirror"])
 @pytest.mark.parametrize("shape", MARCH)
 def test_marching_against_oracle(gpu_lib, shape, geometry, collision, tau, forcing):
-    _compare(shape, geometry, collision, tau, forcing, "f32", 4, lambda ref: TOL["f32"] * np.abs(ref).max())
+    _compare(shape, geometry, collision, tau, forcing, "f32", 4, lambda ref: TOL["f32"] * np.abs(ref).max(),
+             calls=[1, 1, 1, 1])
+
+
+@pytest.mark.parametrize("collision,tau", KINDS)
+@pytest.mark.parametrize("geometry,shape", [(g, s) for g in ("periodic", "mirror", "potential") for s in MARCH] +
+                         [("mirror", (1, 150, 300)), ("potential", (1, 150, 300))])
+@pytest.mark.parametrize("calls", [[4], [2, 1, 3], [5]])
+def test_runs_of_steps_against_oracle(gpu_lib, geometry, shape, collision, tau, calls):
+    n = sum(calls)
+    _compare(shape, geometry, collision, tau, "edm", "f32", n, lambda ref: n / 4 * TOL["f32"] * np.abs(ref).max(),
+             calls=calls)
 
 
 @pytest.mark.parametrize("storage,eps", [("f16_dev", 2.0 ** -11), ("bf16_dev", 2.0 ** -8)])
