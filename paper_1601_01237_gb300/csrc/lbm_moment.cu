@@ -14,8 +14,8 @@
 // bytes).  Every value is held and every sum taken in FP32, as in the
 // population steps; the state at the end of the call is the population state.
 // us per step in calls of 10 (512^3), 20 (256^3) and 100 steps, population steps and
-// these: tau = 1 512^3 6723 / 3100, 256^3 842 / 402, 128^3 119 / 66, 96^3 52 / 36,
-// regularized 256^3 883 / 624, 384 x 512 x 512 with walls 5900 / 3770.
+// these: tau = 1 512^3 6723 / 2800, 256^3 842 / 374, 128^3 119 / 57, 96^3 52 / 35,
+// regularized 256^3 883 / 594, 384 x 512 x 512 with walls 5900 / 3190.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -130,8 +130,8 @@ k_moment_out(MomentState<KIND> m, float *__restrict__ f, Phys<float> p)
 }
 
 // ---------------------------------------------------------------------------
-// m(t) -> m(t + 1).  A CTA owns 30 x 14 columns and marches along z over lz
-// planes; its 32 x 16 threads are those columns and the ring around them, one
+// m(t) -> m(t + 1).  A CTA owns 30 x (EY - 2) columns and marches along z over
+// lz planes; its 32 x EY threads are those columns and the ring around them, one
 // thread per column.  Per plane p:
 //   a. each thread completes the interaction sums of its cell from the density
 //      planes p - 1, p, p + 1 (each plane is read once from shared memory and
@@ -144,23 +144,41 @@ k_moment_out(MomentState<KIND> m, float *__restrict__ f, Phys<float> p)
 //      plane p - 1 (c_z = -1), as sums and differences of opposite sources, adds
 //      them to the moments of those planes and stores the moments of plane
 //      p - 1, which are then complete;
-//   -- barrier --
+//   -- barrier, unless the next plane's pairs go to another copy --
 // The next plane's moments and the density plane after it are loaded one
 // iteration ahead.  The ring's collisions are computed by every neighbouring
-// CTA too (512 collisions for 420 cells), and a CTA computes one plane more at
-// each end of its chunk; densities reach one cell further, loaded by 100 of
-// the threads.
-constexpr int kEX = 32, kEY = 16, kThreadsS = kEX * kEY;   // threads: tile and ring
-constexpr int kOX = kEX - 2, kOY = kEY - 2;                // tile
-constexpr int kRX = kEX + 2, kRY = kEY + 2;                // densities
-constexpr int kRim = 2 * kRX + 2 * kEY;                    // cells of the density plane beyond the threads' own
-constexpr int kPad = 40;                                   // a neighbour's offset is at most 33
+// CTA too (512 collisions for 420 cells in tiles of 16 rows), and a CTA computes one plane more at
+// each end of its chunk; densities reach one cell further, loaded by 68 + 2 EY
+// of the threads.
+constexpr int kEX = 32, kOX = kEX - 2, kRX = kEX + 2;   // along x: threads, tile, densities
+constexpr int kPad = 40;                                // a neighbour's offset is at most 33
 constexpr int kMove = 16;
-static_assert(kRim <= kThreadsS && kPad >= kEX + 1, "");
+static_assert(kPad >= kEX + 1, "");
+// Tiles of EY thread rows.  NB = 2 copies of the moving populations leave one
+// barrier per plane instead of two, where shared memory holds them.  ns: measured
+// time per plane of an SM full of such CTAs, which is 69 to 77 ns per row at tau = 1
+// and 110 to 114 ns regularized whatever the tile, so that the tile with the fewest
+// rows of work (rings, ragged edges and the last wave counted) is taken:
+// us per step at tau = 1, tiles 12 / 16 / 24: 512^3 2802 / 2759 / 2892, 256^3 374 /
+// 386 / 386, 128^3 66 / 66 / 57, 96^3 35 / 37 / 35; regularized 12 / 16: 256^3 594 /
+// 608, 131 x 150 x 173 129 / 135, 384 x 512 x 512 with walls 3335 / 3182.  (One tile
+// of 16 rows and two barriers: 2810, 392, 68, 37; 599, 134, 3473.  Regularized tiles
+// of 18 or more rows spill: 1028 us at 256^3.)
+template <int KIND, int EY_>
+struct Tile {
+    static constexpr int EY = EY_, ctas = KIND == COLL_EQ && EY <= 16 ? 2 : 1, NB = KIND == COLL_EQ && EY == 16 ? 1 : 2;
+    static constexpr int ns = KIND == COLL_EQ ? (EY == 12 ? 1656 : (EY == 16 ? 2345 : 1860)) : (EY == 12 ? 1320 : 1830);
+    static constexpr int threads = kEX * EY, OY = EY - 2, RY = EY + 2;
+    static constexpr int rim = 2 * kRX + 2 * EY;   // cells of a density plane beyond the threads' own
+    static_assert(rim <= threads, "");
+};
 
+template <class T>
 struct MomentSmem {
-    float2 f[kMove][kPad + kThreadsS + kPad];   // moving populations of the current plane
-    float2 rho[2][kRY][kRX];                    // density planes p + 1 and p + 2
+    float2 lead[kPad];                    // (threads of the ring read past the ends; what they collect is not stored)
+    float2 f[T::NB][kMove][T::threads];   // moving populations of a plane
+    float2 tail[kPad];
+    float2 rho[2][T::RY][kRX];            // density planes p + 1 and p + 2
 };
 
 // The direction with given components.
@@ -218,14 +236,16 @@ struct Collect {
     }
 };
 
-template <int KIND, bool WALLZ>
-__global__ void __launch_bounds__(kThreadsS, KIND == COLL_EQ ? 2 : 1)
+template <int KIND, int EY, bool WALLZ>
+__global__ void __launch_bounds__(Tile<KIND, EY>::threads, Tile<KIND, EY>::ctas)
 k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, int ntx, int lz)
 {
     constexpr int NP = MomentState<KIND>::NP;
+    using T = Tile<KIND, EY>;
+    constexpr int kOY = T::OY, kRY = T::RY, kRim = T::rim, kThreadsS = T::threads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    MomentSmem &sm = *reinterpret_cast<MomentSmem *>(smem_raw);
-    const int tid = threadIdx.x, ex = tid % kEX, ey = tid / kEX, at = kPad + tid;
+    MomentSmem<T> &sm = *reinterpret_cast<MomentSmem<T> *>(smem_raw);
+    const int tid = threadIdx.x, ex = tid % kEX, ey = tid / kEX;
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const unsigned plane = (unsigned)nx * (unsigned)ny, N32 = (unsigned)p.N;
     const int x0 = (int)(blockIdx.x % (unsigned)ntx) * kOX, y0 = (int)(blockIdx.x / (unsigned)ntx) * kOY;
@@ -320,6 +340,7 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
             lo[1] = ly;
             lo[2] = vsub(make_float2(0.f, 0.f), Z);
         }
+        float2 *const F = &sm.f[T::NB == 2 ? (q & 1) : 0][0][tid];
         const float2 r = r_own;   // density of plane q at this column
         r_own = rc;
         float2 f0, fu, fd;        // populations that stay in the column: c_z = 0, +1, -1
@@ -329,7 +350,7 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
                 if (i == 0) f0 = v;
                 else if (i == kUp) fu = v;
                 else if (i == kDown) fd = v;
-                else sm.f[i < kUp ? i - 1 : i - 3][at] = v;
+                else F[(i < kUp ? i - 1 : i - 3) * kThreadsS] = v;
             };
             collide_cell<PairF32, KIND, FORCE_EDM, false>(PairF32(), p, r, 0.f, uxy_c.x, uxy_c.y, uz_c, So, mo_c, get, put);
         }
@@ -339,8 +360,8 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
         c2.zero();
         if (collides) {
             // the population (X, Y, Z) out of column - (X, Y), and the cell's own
-#define LBM_FROM(X, Y, Z) sm.f[MoveSlot<X, Y, Z>::value][at - (X) - (Y) * kEX]
-#define LBM_OWN(X, Y, Z) sm.f[MoveSlot<X, Y, Z>::value][at]
+#define LBM_FROM(X, Y, Z) F[MoveSlot<X, Y, Z>::value * kThreadsS - (X) - (Y) * kEX]
+#define LBM_OWN(X, Y, Z) F[MoveSlot<X, Y, Z>::value * kThreadsS]
             {   // c_z = 0
                 const float2 xp = LBM_FROM(1, 0, 0), xm = LBM_FROM(-1, 0, 0), yp = LBM_FROM(0, 1, 0), ym = LBM_FROM(0, -1, 0);
                 const float2 a = LBM_FROM(1, 1, 0), b = LBM_FROM(-1, -1, 0), c = LBM_FROM(1, -1, 0), d = LBM_FROM(-1, 1, 0);
@@ -378,7 +399,7 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
         }
         c0 = c1;
         c1 = c2;
-        __syncthreads();
+        if (T::NB == 1) __syncthreads();   // (two copies: a copy's readers passed the next plane's barrier)
     }
 }
 
@@ -398,42 +419,69 @@ Phys<float> make_phys_m(const HostPhys &h)
 }
 
 // Planes per CTA: equal chunks, the fewest waves x (planes + 4) (the collisions
-// beyond the two ends of a chunk and the density planes before it).
-int moment_planes(long long cols, int nz, long long slots)
+// beyond the two ends of a chunk and the density planes before it); cost: that
+// number.
+int moment_planes(long long cols, int nz, long long slots, long long *cost)
 {
     int best = nz;
-    long long cbest = -1;
+    *cost = -1;
     for (int nch = (nz + 127) / 128; nch <= nz; ++nch) {
         const int lz = (nz + nch - 1) / nch;
         if (lz < 4 && nch > 1) break;
         const long long ctas = cols * ((nz + lz - 1) / lz), c = ((ctas + slots - 1) / slots) * (lz + 4);
-        if (cbest < 0 || c < cbest) { cbest = c; best = lz; }
+        if (*cost < 0 || c < *cost) { *cost = c; best = lz; }
     }
     return best;
 }
 
+struct Plan {
+    int ntx, lz;
+    long long cols, ns;   // tile columns, estimated time
+};
+template <int KIND, int EY>
+Plan plan_of(const HostPhys &h)
+{
+    using T = Tile<KIND, EY>;
+    Plan q;
+    q.ntx = (h.nx + kOX - 1) / kOX;
+    q.cols = (long long)q.ntx * ((h.ny + T::OY - 1) / T::OY);
+    q.lz = moment_planes(q.cols, h.nz, (long long)T::ctas * current_device_sms(), &q.ns);
+    q.ns *= T::ns;
+    return q;
+}
+
 constexpr int kMaxAttrDevices = 64;
 
-template <int KIND, bool WALLZ>
-cudaError_t launch_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
+template <int KIND, int EY, bool WALLZ>
+cudaError_t launch_tile(const HostPhys &h, const Plan &q, const void *in, void *out, cudaStream_t s)
 {
+    using T = Tile<KIND, EY>;
     static std::atomic<int> attr_set[kMaxAttrDevices];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const bool cached = dev >= 0 && dev < kMaxAttrDevices;
     if (!cached || !attr_set[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute((const void *)k_step_moment<KIND, WALLZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(MomentSmem));
+        e = cudaFuncSetAttribute((const void *)k_step_moment<KIND, EY, WALLZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(MomentSmem<T>));
         if (e != cudaSuccess) return e;
         if (cached) attr_set[dev].store(1, std::memory_order_release);
     }
-    const int ntx = (h.nx + kOX - 1) / kOX, nty = (h.ny + kOY - 1) / kOY;
-    const long long cols = (long long)ntx * nty;
-    const int lz = moment_planes(cols, h.nz, (KIND == COLL_EQ ? 2LL : 1LL) * current_device_sms());
-    k_step_moment<KIND, WALLZ><<<dim3((unsigned)cols, (unsigned)((h.nz + lz - 1) / lz)), kThreadsS, sizeof(MomentSmem), s>>>(
-        MomentState<KIND>(const_cast<void *>(in), h.N), MomentState<KIND>(out, h.N), make_phys_m(h), ntx, lz);
+    const dim3 grid((unsigned)q.cols, (unsigned)((h.nz + q.lz - 1) / q.lz));
+    k_step_moment<KIND, EY, WALLZ><<<grid, T::threads, sizeof(MomentSmem<T>), s>>>(
+        MomentState<KIND>(const_cast<void *>(in), h.N), MomentState<KIND>(out, h.N), make_phys_m(h), q.ntx, q.lz);
     return cudaGetLastError();
+}
+
+template <int KIND, bool WALLZ>
+cudaError_t launch_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
+{
+    const Plan a = plan_of<KIND, 12>(h), b = plan_of<KIND, 16>(h);
+    if constexpr (KIND == COLL_EQ) {
+        const Plan c = plan_of<KIND, 24>(h);
+        if (c.ns < a.ns && c.ns < b.ns) return launch_tile<KIND, 24, WALLZ>(h, c, in, out, s);
+    }
+    return a.ns < b.ns ? launch_tile<KIND, 12, WALLZ>(h, a, in, out, s) : launch_tile<KIND, 16, WALLZ>(h, b, in, out, s);
 }
 
 bool tau_one(const HostPhys &h) { return (float)(1.0 / h.tau[0]) == 1.0f && (float)(1.0 / h.tau[1]) == 1.0f; }
@@ -445,7 +493,7 @@ inline unsigned grid_m(long long N) { return (unsigned)((N + kThreadsM - 1) / kT
 size_t moment_bytes(const HostPhys &h)
 {
     if (h.storage != ST_F32 || h.forcing != FORCE_EDM || h.links || !fused_supported(h) || use_box(h)) return 0;
-    const long long cols = (long long)((h.nx + kOX - 1) / kOX) * ((h.ny + kOY - 1) / kOY);
+    const long long cols = (long long)((h.nx + kOX - 1) / kOX) * ((h.ny + Tile<COLL_REG, 12>::OY - 1) / Tile<COLL_REG, 12>::OY);
     if (cols >= (1LL << 31) || h.nz > 4 * 65535) return 0;   // grid limits
     const size_t N = (size_t)h.N;
     if (tau_one(h)) return sizeof(float) * moment_floats<COLL_EQ>() * N;

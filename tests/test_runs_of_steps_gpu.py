@@ -1,0 +1,40 @@
+"""Runs of steps in moment space against the FP64 oracle: every tile of the step
+kernel, with its remainders along all axes."""
+import numpy as np
+import pytest
+
+from _helpers import direction_map, gpu_run, oracle_run
+from paper_1601_01237_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+# 20 dependent roundings per step and population, relative to the largest one
+EPS = 20 * 6.0e-8
+# tiles of 12, 16 and 24 rows at tau = 1, of 12, 16 and 16 regularized
+TILES = [(27, 58, 147), (8, 285, 153), (10, 254, 99)]
+KINDS = [("bgk", (1.0, 1.0)), ("regularized", (0.7, 1.2))]
+
+
+def _compare(shape, collision, tau, calls, solid=None, **geo):
+    r1, r2, u = wl.random_state(shape, seed=11, rho_lo=0.3, rho_hi=0.7, u_max=0.03)
+    if solid is not None:
+        u[solid != 0] = 0.0
+    kw = dict(tau=tau, G12=-1.2, G21=-1.1, g_ext=(1e-4, -2e-4, 5e-5), collision=collision, **geo)
+    _, f = oracle_run(shape, r1, r2, u, sum(calls), solid=solid, **kw)
+    lat = gpu_run(shape, r1, r2, u, 0, solid=solid, **kw)
+    for n in calls:
+        lat.step(n)
+    g = lat.get_populations()
+    lat.close()
+    ref = f[:, direction_map()]
+    if solid is not None:
+        ref = np.where(solid[None, None] != 0, 0.0, ref)
+    assert np.abs(g - ref).max() < sum(calls) * EPS * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("geometry", ["periodic", "mirror"])
+@pytest.mark.parametrize("collision,tau", KINDS)
+@pytest.mark.parametrize("shape", TILES)
+def test_tiles(gpu_lib, shape, collision, tau, geometry):
+    geo = {} if geometry == "periodic" else dict(rho_s=(0.02, 0.05), wall_model=geometry, periodic=(1, 1, 0))
+    _compare(shape, collision, tau, [3], **geo)
