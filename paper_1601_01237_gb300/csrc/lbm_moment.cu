@@ -15,7 +15,8 @@
 // population steps; the state at the end of the call is the population state.
 // us per step in calls of 10 (512^3), 20 (256^3) and 100 steps, population steps and
 // these: tau = 1 512^3 6723 / 2800, 256^3 842 / 374, 128^3 119 / 57, 96^3 52 / 35,
-// regularized 256^3 883 / 594, 384 x 512 x 512 with walls 5900 / 3190.
+// regularized 256^3 883 / 594, 384 x 512 x 512 with walls 5900 / 3190,
+// tau = 1 under a mask 256^3 1020 / 410.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -42,6 +43,14 @@ struct MomentState {
         uxy = rho + N;
         P = uxy + N;                 // P[k N + cell]
         uz = (float *)(P + (long long)NP * N);
+    }
+    __device__ __forceinline__ void put_solid(unsigned cell, float2 r, unsigned N32) const
+    {
+        rho[cell] = r;
+        uxy[cell] = make_float2(0.f, 0.f);
+        uz[cell] = 0.f;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) P[(size_t)k * N32 + cell] = make_float2(0.f, 0.f);
     }
 };
 template <int KIND>
@@ -75,17 +84,25 @@ __device__ __forceinline__ Nb3 nb3(const Phys<float> &p, unsigned cell)
 constexpr int kThreadsM = 256;
 
 // One thread per cell, bound by the 152 bytes it gathers.
+// links (nullptr without a mask): every cell's link word (bit 0: the cell is
+// solid; bit i: x - c_i is solid, so that link bounces back).  A solid site
+// holds the density that it presents to Eq. 13 and no motion.
 template <int KIND>
 __global__ void __launch_bounds__(kThreadsM)
-k_moment_in(const float *__restrict__ f, MomentState<KIND> m, Phys<float> p)
+k_moment_in(const float *__restrict__ f, MomentState<KIND> m, Phys<float> p, const unsigned *__restrict__ links)
 {
     const unsigned cell = blockIdx.x * kThreadsM + threadIdx.x, N32 = (unsigned)p.N;
     if (cell >= N32) return;
     const Nb3 n = nb3(p, cell);
+    const unsigned lw = links ? __ldg(links + cell) : 0u;
+    if (lw & 1u) {
+        m.put_solid(cell, make_float2(p.rho_s[0], p.rho_s[1]), N32);
+        return;
+    }
     float2 v[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        const bool wall = (cz(i) == 1 && n.zlo) || (cz(i) == -1 && n.zhi);
+        const bool wall = (cz(i) == 1 && n.zlo) || (cz(i) == -1 && n.zhi) || ((lw >> i) & 1u);
         const unsigned src = n.zo[1 - cz(i)] + n.yo[1 - cy(i)] + n.xo[1 - cx(i)];
         v[i] = ld_pair_f32(f + 2 * (size_t)(wall ? (unsigned)opp(i) * N32 + cell : (unsigned)i * N32 + src));
     }
@@ -105,11 +122,17 @@ k_moment_in(const float *__restrict__ f, MomentState<KIND> m, Phys<float> p)
 // One thread per cell, bound by the 152 bytes it stores.
 template <int KIND>
 __global__ void __launch_bounds__(kThreadsM)
-k_moment_out(MomentState<KIND> m, float *__restrict__ f, Phys<float> p)
+k_moment_out(MomentState<KIND> m, float *__restrict__ f, Phys<float> p, const unsigned *__restrict__ links)
 {
     const unsigned cell = blockIdx.x * kThreadsM + threadIdx.x, N32 = (unsigned)p.N;
     if (cell >= N32) return;
     const Nb3 n = nb3(p, cell);
+    if (links && (__ldg(links + cell) & 1u)) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            *reinterpret_cast<float2 *>(f + 2 * (size_t)((unsigned)i * N32 + cell)) = make_float2(0.f, 0.f);
+        return;
+    }
     const float2 rs = make_float2(p.rho_s[0], p.rho_s[1]);
     const float2 *__restrict__ rho = m.rho;
     auto at = [&](int dx, int dy, int dz) {
@@ -127,6 +150,30 @@ k_moment_out(MomentState<KIND> m, float *__restrict__ f, Phys<float> p)
     auto get = [](int) { return make_float2(0.f, 0.f); };
     auto put = [&](int i, float2 v) { *reinterpret_cast<float2 *>(f + 2 * (size_t)((unsigned)i * N32 + cell)) = v; };
     collide_cell<PairF32, KIND, FORCE_EDM, false>(PairF32(), p, r, 0.f, uxy.x, uxy.y, m.uz[cell], So, mo, get, put);
+}
+
+// Wall densities of the mirror model under a mask, after each new moment state:
+// each solid site with a fluid neighbour takes the w_i-weighted mean of its fluid
+// neighbours' densities plus rho_s (Eq. 13).  One thread per site: the sites are a
+// surface, so launch and one gather's latency bound it.
+__global__ void __launch_bounds__(kThreadsM)
+k_moment_walls(float2 *__restrict__ rho, Phys<float> p, const unsigned *__restrict__ links,
+               const unsigned *__restrict__ sites, long long n_sites)
+{
+    const long long t = (long long)blockIdx.x * kThreadsM + threadIdx.x;
+    if (t >= n_sites) return;
+    const Nb3 n = nb3(p, sites[t]);
+    const unsigned lw = __ldg(links + n.cell);   // bit i: x - c_i is solid
+    float2 num = make_float2(0.f, 0.f);
+    int den36 = 0;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+        if ((lw >> i) & 1u) continue;
+        num = vfma(PairF32::dup((float)k36(i)), rho[n.zo[1 - cz(i)] + n.yo[1 - cy(i)] + n.xo[1 - cx(i)]], num);
+        den36 += k36(i);
+    }
+    const float d = (float)den36;
+    rho[n.cell] = den36 ? make_float2(num.x / d + p.rho_s[0], num.y / d + p.rho_s[1]) : make_float2(p.rho_s[0], p.rho_s[1]);
 }
 
 // ---------------------------------------------------------------------------
@@ -150,6 +197,10 @@ k_moment_out(MomentState<KIND> m, float *__restrict__ f, Phys<float> p)
 // CTA too (512 collisions for 420 cells in tiles of 16 rows), and a CTA computes one plane more at
 // each end of its chunk; densities reach one cell further, loaded by 68 + 2 EY
 // of the threads.
+// MASK: a solid site lets nothing out, so that what streams from it is zero, and a
+// cell with a link into a solid site (a bit of its link word) adds its own
+// populations of these links, reversed, to its plane; the solid sites' densities
+// stand in the moment state (k_moment_walls), and the gradient needs no case.
 constexpr int kEX = 32, kOX = kEX - 2, kRX = kEX + 2;   // along x: threads, tile, densities
 constexpr int kPad = 40;                                // a neighbour's offset is at most 33
 constexpr int kMove = 16;
@@ -214,6 +265,23 @@ struct Collect {
 #pragma unroll
         for (int k = 0; k < NP; ++k) P[k] = make_float2(0.f, 0.f);
     }
+    // the eight populations of c_z = 0 that move, along +x, -x, +y, -y and the
+    // diagonals (+,+), (-,-), (+,-), (-,+)
+    __device__ __forceinline__ void add_plane(float2 xp, float2 xm, float2 yp, float2 ym, float2 a, float2 b, float2 c,
+                                              float2 d)
+    {
+        const float2 ab = vadd(a, b), cd = vadd(c, d), da = vsub(a, b), dc = vsub(c, d);
+        const float2 ex = vadd(xp, xm), ey = vadd(yp, ym), dg = vadd(ab, cd);
+        const float2 mx = vadd(vsub(xp, xm), vadd(da, dc)), my = vadd(vsub(yp, ym), vsub(da, dc));
+        rho = vadd(rho, vadd(vadd(ex, ey), dg));
+        jx += mx.x + mx.y;
+        jy += my.x + my.y;
+        if constexpr (NP > 0) {
+            P[0] = vadd(P[0], vadd(ex, dg));
+            P[1] = vadd(P[1], vadd(ey, dg));
+            P[3] = vadd(P[3], vsub(ab, cd));
+        }
+    }
     // the five populations of a group c_z = Z = +-1: the one that stays in its
     // column, and those from the columns at -x, +x, -y, +y (moving the other way)
     template <int Z>
@@ -236,10 +304,12 @@ struct Collect {
     }
 };
 
-template <int KIND, int EY, bool WALLZ>
+template <int KIND, int EY, bool WALLZ, bool MASK>
 __global__ void __launch_bounds__(Tile<KIND, EY>::threads, Tile<KIND, EY>::ctas)
-k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, int ntx, int lz)
+k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, int ntx, int lz,
+              const unsigned *__restrict__ links)
 {
+    static_assert(!(MASK && WALLZ), "a solid mask needs a lattice periodic along z");
     constexpr int NP = MomentState<KIND>::NP;
     using T = Tile<KIND, EY>;
     constexpr int kOY = T::OY, kRY = T::RY, kRim = T::rim, kThreadsS = T::threads;
@@ -288,6 +358,7 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
     }
     float2 uxy = make_float2(0.f, 0.f);
     float uz = 0.f;
+    unsigned lw = 0, lw_p = 0;   // link words of the column at plane q + 1, q - 1
     RegMoments<PairF32, KIND> mo;
     float2 S[3], lo[3], r_own = make_float2(0.f, 0.f);   // sums of plane p so far, and what plane p adds to p + 1's
 #pragma unroll
@@ -308,6 +379,7 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
         // loads for the next iteration
         const float2 uxy_c = uxy;
         const float uz_c = uz;
+        const unsigned lw_c = lw;
         const RegMoments<PairF32, KIND> mo_c = mo;
         if (q < z1) {
             const unsigned o3 = offset(q + 3), o1 = offset(q + 1);
@@ -315,6 +387,7 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
             if (rim) h_next = in.rho[o3 + rcol];
             uxy = in.uxy[o1 + col];
             uz = in.uz[o1 + col];
+            if (MASK) lw = __ldg(links + o1 + col);
 #pragma unroll
             for (int k = 0; k < NP; ++k) mo.m[k] = in.P[(size_t)k * N32 + o1 + col];
         }
@@ -352,7 +425,13 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
                 else if (i == kDown) fd = v;
                 else F[(i < kUp ? i - 1 : i - 3) * kThreadsS] = v;
             };
-            collide_cell<PairF32, KIND, FORCE_EDM, false>(PairF32(), p, r, 0.f, uxy_c.x, uxy_c.y, uz_c, So, mo_c, get, put);
+            if (MASK && (lw_c & 1u)) {   // nothing leaves a solid site
+#pragma unroll
+                for (int i = 0; i < Q; ++i) put(i, make_float2(0.f, 0.f));
+            } else {
+                collide_cell<PairF32, KIND, FORCE_EDM, false>(PairF32(), p, r, 0.f, uxy_c.x, uxy_c.y, uz_c, So, mo_c, get,
+                                                              put);
+            }
         }
         __syncthreads();
         // ---- b. what streams into this column
@@ -365,17 +444,8 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
             {   // c_z = 0
                 const float2 xp = LBM_FROM(1, 0, 0), xm = LBM_FROM(-1, 0, 0), yp = LBM_FROM(0, 1, 0), ym = LBM_FROM(0, -1, 0);
                 const float2 a = LBM_FROM(1, 1, 0), b = LBM_FROM(-1, -1, 0), c = LBM_FROM(1, -1, 0), d = LBM_FROM(-1, 1, 0);
-                const float2 ab = vadd(a, b), cd = vadd(c, d), da = vsub(a, b), dc = vsub(c, d);
-                const float2 ex2 = vadd(xp, xm), ey2 = vadd(yp, ym), dg = vadd(ab, cd);
-                const float2 jx = vadd(vsub(xp, xm), vadd(da, dc)), jy = vadd(vsub(yp, ym), vsub(da, dc));
-                c1.rho = vadd(c1.rho, vadd(f0, vadd(vadd(ex2, ey2), dg)));
-                c1.jx += jx.x + jx.y;
-                c1.jy += jy.x + jy.y;
-                if constexpr (NP > 0) {
-                    c1.P[0] = vadd(c1.P[0], vadd(ex2, dg));
-                    c1.P[1] = vadd(c1.P[1], vadd(ey2, dg));
-                    c1.P[3] = vsub(ab, cd);
-                }
+                c1.rho = vadd(c1.rho, f0);
+                c1.add_plane(xp, xm, yp, ym, a, b, c, d);
             }
             c2.template add_group<1>(fu, LBM_FROM(1, 0, 1), LBM_FROM(-1, 0, 1), LBM_FROM(0, 1, 1), LBM_FROM(0, -1, 1));
             c0.template add_group<-1>(fd, LBM_FROM(1, 0, -1), LBM_FROM(-1, 0, -1), LBM_FROM(0, 1, -1), LBM_FROM(0, -1, -1));
@@ -385,18 +455,36 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
                 if (q == nz - 1)
                     c1.template add_group<-1>(fu, LBM_OWN(-1, 0, 1), LBM_OWN(1, 0, 1), LBM_OWN(0, -1, 1), LBM_OWN(0, 1, 1));
             }
+            if (MASK && lw_c > 1u) {   // links into solid sites
+#define LBM_BACK(X, Y, Z) (((lw_c >> dir_of(X, Y, Z)) & 1u) ? LBM_OWN(-(X), -(Y), -(Z)) : make_float2(0.f, 0.f))
+                {   // c_z = 0
+                    const float2 xp = LBM_BACK(1, 0, 0), xm = LBM_BACK(-1, 0, 0), yp = LBM_BACK(0, 1, 0), ym = LBM_BACK(0, -1, 0);
+                    const float2 a = LBM_BACK(1, 1, 0), b = LBM_BACK(-1, -1, 0), c = LBM_BACK(1, -1, 0), d = LBM_BACK(-1, 1, 0);
+                    c1.add_plane(xp, xm, yp, ym, a, b, c, d);
+                }
+                c1.template add_group<1>(((lw_c >> kUp) & 1u) ? fd : make_float2(0.f, 0.f), LBM_BACK(1, 0, 1), LBM_BACK(-1, 0, 1),
+                                         LBM_BACK(0, 1, 1), LBM_BACK(0, -1, 1));
+                c1.template add_group<-1>(((lw_c >> kDown) & 1u) ? fu : make_float2(0.f, 0.f), LBM_BACK(1, 0, -1),
+                                          LBM_BACK(-1, 0, -1), LBM_BACK(0, 1, -1), LBM_BACK(0, -1, -1));
+#undef LBM_BACK
+            }
 #undef LBM_FROM
 #undef LBM_OWN
         }
         if (q > z0 && stores) {   // plane q - 1 is complete
             const unsigned cell = (unsigned)(q - 1) * plane + col;
-            const float inv = 1.0f / (c0.rho.x + c0.rho.y);
-            out.rho[cell] = c0.rho;
-            out.uxy[cell] = make_float2(c0.jx * inv, c0.jy * inv);
-            out.uz[cell] = c0.jz * inv;
+            if (MASK && (lw_p & 1u)) {
+                out.put_solid(cell, rs, N32);
+            } else {
+                const float inv = 1.0f / (c0.rho.x + c0.rho.y);
+                out.rho[cell] = c0.rho;
+                out.uxy[cell] = make_float2(c0.jx * inv, c0.jy * inv);
+                out.uz[cell] = c0.jz * inv;
 #pragma unroll
-            for (int k = 0; k < NP; ++k) out.P[(size_t)k * N32 + cell] = c0.P[k];
+                for (int k = 0; k < NP; ++k) out.P[(size_t)k * N32 + cell] = c0.P[k];
+            }
         }
+        lw_p = lw_c;
         c0 = c1;
         c1 = c2;
         if (T::NB == 1) __syncthreads();   // (two copies: a copy's readers passed the next plane's barrier)
@@ -452,7 +540,7 @@ Plan plan_of(const HostPhys &h)
 
 constexpr int kMaxAttrDevices = 64;
 
-template <int KIND, int EY, bool WALLZ>
+template <int KIND, int EY, bool WALLZ, bool MASK>
 cudaError_t launch_tile(const HostPhys &h, const Plan &q, const void *in, void *out, cudaStream_t s)
 {
     using T = Tile<KIND, EY>;
@@ -462,26 +550,26 @@ cudaError_t launch_tile(const HostPhys &h, const Plan &q, const void *in, void *
     if (e != cudaSuccess) return e;
     const bool cached = dev >= 0 && dev < kMaxAttrDevices;
     if (!cached || !attr_set[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute((const void *)k_step_moment<KIND, EY, WALLZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute((const void *)k_step_moment<KIND, EY, WALLZ, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(MomentSmem<T>));
         if (e != cudaSuccess) return e;
         if (cached) attr_set[dev].store(1, std::memory_order_release);
     }
     const dim3 grid((unsigned)q.cols, (unsigned)((h.nz + q.lz - 1) / q.lz));
-    k_step_moment<KIND, EY, WALLZ><<<grid, T::threads, sizeof(MomentSmem<T>), s>>>(
-        MomentState<KIND>(const_cast<void *>(in), h.N), MomentState<KIND>(out, h.N), make_phys_m(h), q.ntx, q.lz);
+    k_step_moment<KIND, EY, WALLZ, MASK><<<grid, T::threads, sizeof(MomentSmem<T>), s>>>(
+        MomentState<KIND>(const_cast<void *>(in), h.N), MomentState<KIND>(out, h.N), make_phys_m(h), q.ntx, q.lz, h.links);
     return cudaGetLastError();
 }
 
-template <int KIND, bool WALLZ>
+template <int KIND, bool WALLZ, bool MASK>
 cudaError_t launch_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
 {
     const Plan a = plan_of<KIND, 12>(h), b = plan_of<KIND, 16>(h);
     if constexpr (KIND == COLL_EQ) {
         const Plan c = plan_of<KIND, 24>(h);
-        if (c.ns < a.ns && c.ns < b.ns) return launch_tile<KIND, 24, WALLZ>(h, c, in, out, s);
+        if (c.ns < a.ns && c.ns < b.ns) return launch_tile<KIND, 24, WALLZ, MASK>(h, c, in, out, s);
     }
-    return a.ns < b.ns ? launch_tile<KIND, 12, WALLZ>(h, a, in, out, s) : launch_tile<KIND, 16, WALLZ>(h, b, in, out, s);
+    return a.ns < b.ns ? launch_tile<KIND, 12, WALLZ, MASK>(h, a, in, out, s) : launch_tile<KIND, 16, WALLZ, MASK>(h, b, in, out, s);
 }
 
 bool tau_one(const HostPhys &h) { return (float)(1.0 / h.tau[0]) == 1.0f && (float)(1.0 / h.tau[1]) == 1.0f; }
@@ -492,7 +580,7 @@ inline unsigned grid_m(long long N) { return (unsigned)((N + kThreadsM - 1) / kT
 
 size_t moment_bytes(const HostPhys &h)
 {
-    if (h.storage != ST_F32 || h.forcing != FORCE_EDM || h.links || !fused_supported(h) || use_box(h)) return 0;
+    if (h.storage != ST_F32 || h.forcing != FORCE_EDM || !fused_supported(h) || use_box(h)) return 0;
     const long long cols = (long long)((h.nx + kOX - 1) / kOX) * ((h.ny + Tile<COLL_REG, 12>::OY - 1) / Tile<COLL_REG, 12>::OY);
     if (cols >= (1LL << 31) || h.nz > 4 * 65535) return 0;   // grid limits
     const size_t N = (size_t)h.N;
@@ -501,28 +589,56 @@ size_t moment_bytes(const HostPhys &h)
     return 0;
 }
 
+namespace {
+
+template <int KIND>
+cudaError_t moment_walls(const HostPhys &h, void *m, cudaStream_t s)
+{
+    if (h.links && h.wall_mirror && h.n_bsolid > 0)
+        k_moment_walls<<<grid_m(h.n_bsolid), kThreadsM, 0, s>>>(MomentState<KIND>(m, h.N).rho, make_phys_m(h), h.links,
+                                                                h.bsolid, h.n_bsolid);
+    return cudaGetLastError();
+}
+
+template <int KIND>
+cudaError_t moment_in_t(const HostPhys &h, const void *f, void *m, cudaStream_t s)
+{
+    k_moment_in<KIND><<<grid_m(h.N), kThreadsM, 0, s>>>((const float *)f, MomentState<KIND>(m, h.N), make_phys_m(h), h.links);
+    return moment_walls<KIND>(h, m, s);
+}
+
+template <int KIND>
+cudaError_t moment_step_t(const HostPhys &h, const void *in, void *out, cudaStream_t s)
+{
+    const cudaError_t e = h.wall_z ? launch_step<KIND, true, false>(h, in, out, s)
+                          : h.links ? launch_step<KIND, false, true>(h, in, out, s)
+                                    : launch_step<KIND, false, false>(h, in, out, s);
+    return e == cudaSuccess ? moment_walls<KIND>(h, out, s) : e;
+}
+
+template <int KIND>
+cudaError_t moment_out_t(const HostPhys &h, const void *m, void *f, cudaStream_t s)
+{
+    k_moment_out<KIND><<<grid_m(h.N), kThreadsM, 0, s>>>(MomentState<KIND>(const_cast<void *>(m), h.N), (float *)f,
+                                                         make_phys_m(h), h.links);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_moment_in(const HostPhys &h, const void *f, void *m, cudaStream_t s)
 {
-    if (tau_one(h))
-        k_moment_in<COLL_EQ><<<grid_m(h.N), kThreadsM, 0, s>>>((const float *)f, MomentState<COLL_EQ>(m, h.N), make_phys_m(h));
-    else
-        k_moment_in<COLL_REG><<<grid_m(h.N), kThreadsM, 0, s>>>((const float *)f, MomentState<COLL_REG>(m, h.N), make_phys_m(h));
-    return cudaGetLastError();
+    return tau_one(h) ? moment_in_t<COLL_EQ>(h, f, m, s) : moment_in_t<COLL_REG>(h, f, m, s);
 }
 
 cudaError_t launch_moment_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
 {
-    if (tau_one(h)) return h.wall_z ? launch_step<COLL_EQ, true>(h, in, out, s) : launch_step<COLL_EQ, false>(h, in, out, s);
-    return h.wall_z ? launch_step<COLL_REG, true>(h, in, out, s) : launch_step<COLL_REG, false>(h, in, out, s);
+    return tau_one(h) ? moment_step_t<COLL_EQ>(h, in, out, s) : moment_step_t<COLL_REG>(h, in, out, s);
 }
 
 cudaError_t launch_moment_out(const HostPhys &h, const void *m, void *f, cudaStream_t s)
 {
-    if (tau_one(h))
-        k_moment_out<COLL_EQ><<<grid_m(h.N), kThreadsM, 0, s>>>(MomentState<COLL_EQ>(const_cast<void *>(m), h.N), (float *)f, make_phys_m(h));
-    else
-        k_moment_out<COLL_REG><<<grid_m(h.N), kThreadsM, 0, s>>>(MomentState<COLL_REG>(const_cast<void *>(m), h.N), (float *)f, make_phys_m(h));
-    return cudaGetLastError();
+    return tau_one(h) ? moment_out_t<COLL_EQ>(h, m, f, s) : moment_out_t<COLL_REG>(h, m, f, s);
 }
 
 }  // namespace lbm

@@ -38,3 +38,18 @@ def _compare(shape, collision, tau, calls, solid=None, **geo):
 def test_tiles(gpu_lib, shape, collision, tau, geometry):
     geo = {} if geometry == "periodic" else dict(rho_s=(0.02, 0.05), wall_model=geometry, periodic=(1, 1, 0))
     _compare(shape, collision, tau, [3], **geo)
+
+
+def _scattered(shape):
+    """One site in twelve solid, and a slab across the lattice."""
+    solid = (np.random.default_rng(5).random(shape) < 1 / 12).astype(np.uint8)
+    z, x = np.arange(shape[0])[:, None, None], np.arange(shape[2])[None, None, :]
+    solid[np.broadcast_to((z + x // 2) % max(shape[0], 9) < 3, shape)] = 1
+    return solid
+
+
+@pytest.mark.parametrize("model", ["mirror", "potential"])
+@pytest.mark.parametrize("collision,tau", KINDS)
+@pytest.mark.parametrize("shape,calls", [(s, [4]) for s in TILES] + [((61, 65, 70), [2, 1, 3]), ((2, 200, 200), [3])])
+def test_masks(gpu_lib, shape, collision, tau, model, calls):
+    _compare(shape, collision, tau, calls, solid=_scattered(shape), rho_s=(0.02, 0.05), wall_model=model)
