@@ -141,8 +141,13 @@ lbm_status lbm_init_fields(lbm_lattice *h, const double *rho1, const double *rho
                            const double *u, int on_device);
 
 /* Advance n_steps >= 0 full time steps (moments, interaction force, collision
- * with forcing, streaming; Sec. 2 and Eq. 1 or Eq. 10).  Asynchronous on the
- * lattice's stream.  Errors: LBM_EINVAL (n_steps < 0), LBM_ECUDA. */
+ * with forcing, streaming; Sec. 2 and Eq. 1 or Eq. 10).  Between the first and
+ * the last step of a call the FP32 arithmetic may act on moments instead of
+ * stored populations (tau = 1 and the regularized operator), so the states of
+ * calls that split a run differently agree to rounding: of FP32, or of the 16-bit
+ * formats, which round what they store once per call then and not at every step.
+ * Asynchronous on the lattice's stream.  Errors: LBM_EINVAL (n_steps < 0),
+ * LBM_ECUDA. */
 lbm_status lbm_step(lbm_lattice *h, long n_steps);
 
 /* lbm_step with per-kernel timing: advances n_steps > 0 steps exactly as
@@ -252,7 +257,8 @@ lbm_status lbm_sync(lbm_lattice *h);
  * ceil(n_steps / ckpt_every) states), and reserves the working memory of the
  * reverse pass (adjoint fields of 2 x 19 values per cell, one checkpoint
  * segment of states and of their densities); both are held until the next
- * lbm_record or lbm_destroy, so that lbm_adjoint allocates nothing.
+ * lbm_record of another shape, lbm_set_solid or lbm_destroy, so that lbm_adjoint
+ * allocates nothing.
  * Synchronizes.  Errors: LBM_EINVAL, LBM_ENOMEM, LBM_ECUDA. */
 lbm_status lbm_record(lbm_lattice *h, long n_steps, int ckpt_every);
 

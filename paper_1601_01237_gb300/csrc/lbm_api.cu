@@ -357,12 +357,17 @@ bool build_graph(lbm_lattice *h)
 }
 
 // n >= 2 steps in moment space: the two moment states live in the population
-// copy that does not hold the state, and the last step writes the populations
-// back into the copy that does.  ev (optional, n + 2 events): recorded before
-// the first launch and after each of the n + 1.
+// copy that does not hold the state or, where two do not fit (16-bit formats), one
+// in each copy (the populations have been read by then), and the last step writes
+// the populations back over the moments that it does not read.  ev (optional,
+// n + 2 events): recorded before the first launch and after each of the n + 1.
 cudaError_t moment_run(lbm_lattice *h, long n, size_t bytes, cudaEvent_t *ev = nullptr)
 {
-    char *m[2] = {(char *)h->f[h->cur ^ 1], (char *)h->f[h->cur ^ 1] + (bytes + 255) / 256 * 256};
+    const size_t stride = (bytes + 255) / 256 * 256;
+    const bool one_copy = 2 * stride <= lbm::state_bytes(h->phys.storage, h->phys.N);
+    char *m[2] = {(char *)h->f[h->cur ^ 1], one_copy ? (char *)h->f[h->cur ^ 1] + stride : (char *)h->f[h->cur]};
+    const int last = (n & 1) ? 0 : 1;   // the state that the last step reads
+    const int dst = !one_copy && last == 1 ? h->cur ^ 1 : h->cur;
     if (ev) cudaEventRecord(*ev++, h->stream);
     cudaError_t e = lbm::launch_moment_in(h->phys, h->f[h->cur], m[0], h->stream);
     if (ev) cudaEventRecord(*ev++, h->stream);
@@ -370,19 +375,22 @@ cudaError_t moment_run(lbm_lattice *h, long n, size_t bytes, cudaEvent_t *ev = n
         e = lbm::launch_moment_step(h->phys, m[(t & 1) ^ 1], m[t & 1], h->stream);
         if (ev) cudaEventRecord(*ev++, h->stream);
     }
-    if (e == cudaSuccess) e = lbm::launch_moment_out(h->phys, m[(n & 1) ^ 1], h->f[h->cur], h->stream);
+    if (e == cudaSuccess) e = lbm::launch_moment_out(h->phys, m[last], h->f[dst], h->stream);
     if (ev) cudaEventRecord(*ev, h->stream);
-    if (e == cudaSuccess) h->steps += n;
+    if (e == cudaSuccess) {
+        h->cur = dst;
+        h->steps += n;
+    }
     return e;
 }
 
-// Bytes of a moment state if the lattice's next n steps run in moment space (two
-// of them fit the free population copy), else 0.
+// Bytes of a moment state if the lattice's next n steps run in moment space (a
+// population copy holds one), else 0.
 size_t moment_run_bytes(const lbm_lattice *h, long n)
 {
-    if (!h->use_fused || n < 2) return 0;
-    const size_t b = lbm::moment_bytes(h->phys);
-    return 2 * ((b + 255) / 256 * 256) <= lbm::state_bytes(h->phys.storage, h->phys.N) ? b : 0;
+    if (!h->use_fused) return 0;
+    const size_t b = lbm::moment_bytes(h->phys, n);
+    return b <= lbm::state_bytes(h->phys.storage, h->phys.N) ? b : 0;
 }
 
 }  // namespace
@@ -791,12 +799,17 @@ lbm_status lbm_record(lbm_lattice *h, long n_steps, int ckpt_every)
         h->ws_every = (long)E;
     }
     h->rec_at_rest = h->init_at_rest && h->steps == 0;
+    const bool rounds = h->phys.storage != lbm::ST_F32 && h->phys.storage != lbm::ST_F64;
     for (long t = 0; t < n_steps; t += ckpt_every) {
         CK(cudaMemcpyAsync((char *)h->ckpt + sb * (size_t)(t / ckpt_every), h->f[h->cur], sb,
                            cudaMemcpyDeviceToDevice, h->stream),
            "lbm_record: checkpoint");
-        lbm_status st = lbm_step(h, std::min<long>(ckpt_every, n_steps - t));
-        if (st != LBM_OK) return st;
+        // in 16 bits step by step: the reverse pass recomputes the same rounded states
+        const long n = std::min<long>(ckpt_every, n_steps - t), each = rounds ? 1 : n;
+        for (long k = 0; k < n; k += each) {
+            const lbm_status st = lbm_step(h, each);
+            if (st != LBM_OK) return st;
+        }
     }
     CK(cudaStreamSynchronize(h->stream), "lbm_record: sync");
     h->rec_steps = n_steps;

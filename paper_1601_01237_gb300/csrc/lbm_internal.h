@@ -71,9 +71,9 @@ bool fused_supported(const HostPhys &p);
 cudaError_t launch_step_box(const HostPhys &p, const void *f_in, void *f_out, cudaStream_t s, void *s_out = nullptr);
 bool use_box(const HostPhys &p);
 // Runs of n >= 2 steps in moment space (lbm_moment.cu): the bytes of one moment
-// state of the lattice, 0 where it does not step that way; populations to
+// state of the lattice, 0 where its next n steps do not run that way; populations to
 // moments, a step on moments, and the last step from moments to populations.
-size_t moment_bytes(const HostPhys &h);
+size_t moment_bytes(const HostPhys &h, long n);
 cudaError_t launch_moment_in(const HostPhys &h, const void *f, void *m, cudaStream_t s);
 cudaError_t launch_moment_step(const HostPhys &h, const void *m_in, void *m_out, cudaStream_t s);
 cudaError_t launch_moment_out(const HostPhys &h, const void *m, void *f, cudaStream_t s);

@@ -1,4 +1,4 @@
-// Runs of steps in moment space (FP32 populations, exact-difference forcing).
+// Runs of steps in moment space (FP32 arithmetic, exact-difference forcing).
 //
 // Under the regularized operator a step reads its 38 populations only to form
 // the densities, the mixture momentum and (for tau != 1) the second moments
@@ -16,7 +16,7 @@
 // us per step in calls of 10 (512^3), 20 (256^3) and 100 steps, population steps and
 // these: tau = 1 512^3 6723 / 2800, 256^3 842 / 374, 128^3 119 / 57, 96^3 52 / 35,
 // regularized 256^3 883 / 594, 384 x 512 x 512 with walls 5900 / 3190,
-// tau = 1 under a mask 256^3 1020 / 410.
+// tau = 1 under a mask 256^3 1020 / 405.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -83,13 +83,13 @@ __device__ __forceinline__ Nb3 nb3(const Phys<float> &p, unsigned cell)
 
 constexpr int kThreadsM = 256;
 
-// One thread per cell, bound by the 152 bytes it gathers.
+// One thread per cell, bound by the bytes it gathers (152 in FP32, 76 in 16 bits).
 // links (nullptr without a mask): every cell's link word (bit 0: the cell is
 // solid; bit i: x - c_i is solid, so that link bounces back).  A solid site
 // holds the density that it presents to Eq. 13 and no motion.
-template <int KIND>
+template <int S, int KIND>
 __global__ void __launch_bounds__(kThreadsM)
-k_moment_in(const float *__restrict__ f, MomentState<KIND> m, Phys<float> p, const unsigned *__restrict__ links)
+k_moment_in(const typename Store<S>::T *__restrict__ f, MomentState<KIND> m, Phys<float> p, const unsigned *__restrict__ links)
 {
     const unsigned cell = blockIdx.x * kThreadsM + threadIdx.x, N32 = (unsigned)p.N;
     if (cell >= N32) return;
@@ -99,14 +99,18 @@ k_moment_in(const float *__restrict__ f, MomentState<KIND> m, Phys<float> p, con
         m.put_solid(cell, make_float2(p.rho_s[0], p.rho_s[1]), N32);
         return;
     }
-    float2 v[Q];
+    float2 v[Q], ref = make_float2(0.f, 0.f);
+    if constexpr (Store<S>::kRel) ref = state_ref(f, p.ref_off)[cell];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const bool wall = (cz(i) == 1 && n.zlo) || (cz(i) == -1 && n.zhi) || ((lw >> i) & 1u);
         const unsigned src = n.zo[1 - cz(i)] + n.yo[1 - cy(i)] + n.xo[1 - cx(i)];
-        v[i] = ld_pair_f32(f + 2 * (size_t)(wall ? (unsigned)opp(i) * N32 + cell : (unsigned)i * N32 + src));
+        const typename Store<S>::T *q = f + 2 * (size_t)(wall ? (unsigned)opp(i) * N32 + cell : (unsigned)i * N32 + src);
+        if constexpr (Store<S>::kDev) Store<S>::load2_d(q, v[i].x, v[i].y);   // (deviations have the momentum of the populations)
+        else Store<S>::load2(q, w<float>(i) * ref.x, w<float>(i) * ref.y, v[i].x, v[i].y);
     }
-    const float2 r = density(v);
+    float2 r = density(v);
+    if constexpr (Store<S>::kDev) r = vadd(r, PairF32::dup(p.rho0));
     float jx, jy, jz;
     momentum(PairF32(), v, jx, jy, jz);
     const float inv = 1.0f / (r.x + r.y);
@@ -116,21 +120,33 @@ k_moment_in(const float *__restrict__ f, MomentState<KIND> m, Phys<float> p, con
     RegMoments<PairF32, KIND> mo;
     mo.of(v);
 #pragma unroll
-    for (int k = 0; k < MomentState<KIND>::NP; ++k) m.P[(size_t)k * N32 + cell] = mo.m[k];
+    for (int k = 0; k < MomentState<KIND>::NP; ++k) {
+        if constexpr (Store<S>::kDev) {
+            if (k < 3) mo.m[k] = vadd(mo.m[k], PairF32::dup(p.rho0 * (1.0f / 3.0f)));
+        }
+        m.P[(size_t)k * N32 + cell] = mo.m[k];
+    }
 }
 
-// One thread per cell, bound by the 152 bytes it stores.
-template <int KIND>
+// One thread per cell, bound by the bytes it stores.  The relative formats code a
+// population by the density of the cell that reads it next (x + c_i, or x itself
+// across a wall) and keep the cell's own.
+template <int FMT, int KIND>
 __global__ void __launch_bounds__(kThreadsM)
-k_moment_out(MomentState<KIND> m, float *__restrict__ f, Phys<float> p, const unsigned *__restrict__ links)
+k_moment_out(MomentState<KIND> m, typename Store<FMT>::T *__restrict__ f, Phys<float> p, const unsigned *__restrict__ links)
 {
     const unsigned cell = blockIdx.x * kThreadsM + threadIdx.x, N32 = (unsigned)p.N;
     if (cell >= N32) return;
     const Nb3 n = nb3(p, cell);
-    if (links && (__ldg(links + cell) & 1u)) {
+    const unsigned lw = links ? __ldg(links + cell) : 0u;
+    const float base = Store<FMT>::kRel ? 1.0f : p.rho0;   // (a solid site's codes are those of the population steps)
+    if (lw & 1u) {
 #pragma unroll
-        for (int i = 0; i < Q; ++i)
-            *reinterpret_cast<float2 *>(f + 2 * (size_t)((unsigned)i * N32 + cell)) = make_float2(0.f, 0.f);
+        for (int i = 0; i < Q; ++i) {
+            const float e = Store<FMT>::enc(w<float>(i) * base);
+            Store<FMT>::store2(f + 2 * (size_t)((unsigned)i * N32 + cell), 0.f, 0.f, e, e);
+        }
+        if constexpr (Store<FMT>::kRel) state_ref(f, p.ref_off)[cell] = make_float2(1.0f, 1.0f);
         return;
     }
     const float2 rs = make_float2(p.rho_s[0], p.rho_s[1]);
@@ -148,14 +164,32 @@ k_moment_out(MomentState<KIND> m, float *__restrict__ f, Phys<float> p, const un
 #pragma unroll
     for (int k = 0; k < MomentState<KIND>::NP; ++k) mo.m[k] = m.P[(size_t)k * N32 + cell];
     auto get = [](int) { return make_float2(0.f, 0.f); };
-    auto put = [&](int i, float2 v) { *reinterpret_cast<float2 *>(f + 2 * (size_t)((unsigned)i * N32 + cell)) = v; };
-    collide_cell<PairF32, KIND, FORCE_EDM, false>(PairF32(), p, r, 0.f, uxy.x, uxy.y, m.uz[cell], So, mo, get, put);
+    if constexpr (Store<FMT>::kRel) state_ref(f, p.ref_off)[cell] = r;
+    auto put = [&](int i, float2 v) {
+        typename Store<FMT>::T *q = f + 2 * (size_t)((unsigned)i * N32 + cell);
+        if constexpr (Store<FMT>::kDev) {
+            Store<FMT>::store2_d(q, v.x, v.y);
+        } else if constexpr (Store<FMT>::kRel) {
+            const bool wall = (cz(i) == -1 && n.zlo) || (cz(i) == 1 && n.zhi) || ((lw >> opp(i)) & 1u);
+            const float2 e = wall || i == 0 ? r : __ldg(rho + n.zo[1 + cz(i)] + n.yo[1 + cy(i)] + n.xo[1 + cx(i)]);
+            Store<FMT>::store2(q, v.x, v.y, Store<FMT>::enc(w<float>(i) * e.x), Store<FMT>::enc(w<float>(i) * e.y));
+        } else {
+            Store<FMT>::store2(q, v.x, v.y, 0.f, 0.f);
+        }
+    };
+    if constexpr (Store<FMT>::kDev) {   // collide_cell takes the second moments of the deviations
+#pragma unroll
+        for (int k = 0; k < 3 && k < MomentState<KIND>::NP; ++k)
+            mo.m[k] = vsub(mo.m[k], PairF32::dup(p.rho0 * (1.0f / 3.0f)));
+    }
+    collide_cell<PairF32, KIND, FORCE_EDM, Store<FMT>::kDev>(PairF32(), p, r, 0.f, uxy.x, uxy.y, m.uz[cell], So, mo, get, put);
 }
 
 // Wall densities of the mirror model under a mask, after each new moment state:
 // each solid site with a fluid neighbour takes the w_i-weighted mean of its fluid
 // neighbours' densities plus rho_s (Eq. 13).  One thread per site: the sites are a
-// surface, so launch and one gather's latency bound it.
+// surface, so launch and one gather's latency bound it (8.5 us beside the 396 of a
+// 256^3 step with an inclined slab).
 __global__ void __launch_bounds__(kThreadsM)
 k_moment_walls(float2 *__restrict__ rho, Phys<float> p, const unsigned *__restrict__ links,
                const unsigned *__restrict__ sites, long long n_sites)
@@ -502,7 +536,8 @@ Phys<float> make_phys_m(const HostPhys &h)
     p.G12 = (float)h.G12; p.G21 = (float)h.G21;
     for (int d = 0; d < 3; ++d) p.gext[d] = (float)h.gext[d];
     p.rho_s[0] = (float)h.rho_s[0]; p.rho_s[1] = (float)h.rho_s[1];
-    p.rho0 = 0.f;
+    p.rho0 = (float)h.rho0;
+    p.ref_off = h.ref_off;
     return p;
 }
 
@@ -578,9 +613,15 @@ inline unsigned grid_m(long long N) { return (unsigned)((N + kThreadsM - 1) / kT
 
 }  // namespace
 
-size_t moment_bytes(const HostPhys &h)
+size_t moment_bytes(const HostPhys &h, long n)
 {
-    if (h.storage != ST_F32 || h.forcing != FORCE_EDM || !fused_supported(h) || use_box(h)) return 0;
+    // Two steps of a relative format lose to the cost of coding the state (regularized,
+    // 256^3: 1892 us step by step, 2096 in moment space; three 2836, 2683); the others
+    // gain from two on (two steps, FP16 deviations regularized 256^3 1370, 1345, 61 x
+    // 65 x 70 70, 40; FP32 1768, 1657, 65, 42).
+    const bool rel = h.storage == ST_F16_REL || h.storage == ST_BF16_REL;
+    if (n < (rel && !tau_one(h) ? 3 : 2)) return 0;
+    if (h.storage == ST_F64 || h.forcing != FORCE_EDM || !fused_supported(h) || use_box(h)) return 0;
     const long long cols = (long long)((h.nx + kOX - 1) / kOX) * ((h.ny + Tile<COLL_REG, 12>::OY - 1) / Tile<COLL_REG, 12>::OY);
     if (cols >= (1LL << 31) || h.nz > 4 * 65535) return 0;   // grid limits
     const size_t N = (size_t)h.N;
@@ -600,10 +641,11 @@ cudaError_t moment_walls(const HostPhys &h, void *m, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <int KIND>
+template <int S, int KIND>
 cudaError_t moment_in_t(const HostPhys &h, const void *f, void *m, cudaStream_t s)
 {
-    k_moment_in<KIND><<<grid_m(h.N), kThreadsM, 0, s>>>((const float *)f, MomentState<KIND>(m, h.N), make_phys_m(h), h.links);
+    k_moment_in<S, KIND><<<grid_m(h.N), kThreadsM, 0, s>>>((const typename Store<S>::T *)f, MomentState<KIND>(m, h.N),
+                                                           make_phys_m(h), h.links);
     return moment_walls<KIND>(h, m, s);
 }
 
@@ -616,19 +658,38 @@ cudaError_t moment_step_t(const HostPhys &h, const void *in, void *out, cudaStre
     return e == cudaSuccess ? moment_walls<KIND>(h, out, s) : e;
 }
 
-template <int KIND>
+template <int S, int KIND>
 cudaError_t moment_out_t(const HostPhys &h, const void *m, void *f, cudaStream_t s)
 {
-    k_moment_out<KIND><<<grid_m(h.N), kThreadsM, 0, s>>>(MomentState<KIND>(const_cast<void *>(m), h.N), (float *)f,
-                                                         make_phys_m(h), h.links);
+    k_moment_out<S, KIND><<<grid_m(h.N), kThreadsM, 0, s>>>(MomentState<KIND>(const_cast<void *>(m), h.N),
+                                                            (typename Store<S>::T *)f, make_phys_m(h), h.links);
     return cudaGetLastError();
+}
+
+template <int S>
+cudaError_t in_s(const HostPhys &h, const void *f, void *m, cudaStream_t s)
+{
+    return tau_one(h) ? moment_in_t<S, COLL_EQ>(h, f, m, s) : moment_in_t<S, COLL_REG>(h, f, m, s);
+}
+
+template <int S>
+cudaError_t out_s(const HostPhys &h, const void *m, void *f, cudaStream_t s)
+{
+    return tau_one(h) ? moment_out_t<S, COLL_EQ>(h, m, f, s) : moment_out_t<S, COLL_REG>(h, m, f, s);
 }
 
 }  // namespace
 
 cudaError_t launch_moment_in(const HostPhys &h, const void *f, void *m, cudaStream_t s)
 {
-    return tau_one(h) ? moment_in_t<COLL_EQ>(h, f, m, s) : moment_in_t<COLL_REG>(h, f, m, s);
+    switch (h.storage) {
+    case ST_F32: return in_s<ST_F32>(h, f, m, s);
+    case ST_F16_DEV: return in_s<ST_F16_DEV>(h, f, m, s);
+    case ST_BF16_DEV: return in_s<ST_BF16_DEV>(h, f, m, s);
+    case ST_F16_REL: return in_s<ST_F16_REL>(h, f, m, s);
+    case ST_BF16_REL: return in_s<ST_BF16_REL>(h, f, m, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_moment_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
@@ -638,7 +699,14 @@ cudaError_t launch_moment_step(const HostPhys &h, const void *in, void *out, cud
 
 cudaError_t launch_moment_out(const HostPhys &h, const void *m, void *f, cudaStream_t s)
 {
-    return tau_one(h) ? moment_out_t<COLL_EQ>(h, m, f, s) : moment_out_t<COLL_REG>(h, m, f, s);
+    switch (h.storage) {
+    case ST_F32: return out_s<ST_F32>(h, m, f, s);
+    case ST_F16_DEV: return out_s<ST_F16_DEV>(h, m, f, s);
+    case ST_BF16_DEV: return out_s<ST_BF16_DEV>(h, m, f, s);
+    case ST_F16_REL: return out_s<ST_F16_REL>(h, m, f, s);
+    case ST_BF16_REL: return out_s<ST_BF16_REL>(h, m, f, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace lbm

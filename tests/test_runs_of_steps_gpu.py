@@ -15,13 +15,13 @@ TILES = [(27, 58, 147), (8, 285, 153), (10, 254, 99)]
 KINDS = [("bgk", (1.0, 1.0)), ("regularized", (0.7, 1.2))]
 
 
-def _compare(shape, collision, tau, calls, solid=None, **geo):
+def _compare(shape, collision, tau, calls, solid=None, storage="f32", tol=None, **geo):
     r1, r2, u = wl.random_state(shape, seed=11, rho_lo=0.3, rho_hi=0.7, u_max=0.03)
     if solid is not None:
         u[solid != 0] = 0.0
     kw = dict(tau=tau, G12=-1.2, G21=-1.1, g_ext=(1e-4, -2e-4, 5e-5), collision=collision, **geo)
     _, f = oracle_run(shape, r1, r2, u, sum(calls), solid=solid, **kw)
-    lat = gpu_run(shape, r1, r2, u, 0, solid=solid, **kw)
+    lat = gpu_run(shape, r1, r2, u, 0, solid=solid, storage=storage, **kw)
     for n in calls:
         lat.step(n)
     g = lat.get_populations()
@@ -29,7 +29,7 @@ def _compare(shape, collision, tau, calls, solid=None, **geo):
     ref = f[:, direction_map()]
     if solid is not None:
         ref = np.where(solid[None, None] != 0, 0.0, ref)
-    assert np.abs(g - ref).max() < sum(calls) * EPS * np.abs(ref).max()
+    assert np.abs(g - ref).max() < (tol or sum(calls) * EPS * np.abs(ref).max())
 
 
 @pytest.mark.parametrize("geometry", ["periodic", "mirror"])
@@ -53,3 +53,29 @@ def _scattered(shape):
 @pytest.mark.parametrize("shape,calls", [(s, [4]) for s in TILES] + [((61, 65, 70), [2, 1, 3]), ((2, 200, 200), [3])])
 def test_masks(gpu_lib, shape, collision, tau, model, calls):
     _compare(shape, collision, tau, calls, solid=_scattered(shape), rho_s=(0.02, 0.05), wall_model=model)
+
+
+@pytest.mark.parametrize("geometry", ["periodic", "mirror", "mask"])
+@pytest.mark.parametrize("collision,tau", KINDS)
+@pytest.mark.parametrize("storage,eps,vmax", [("f16_dev", 2.0 ** -11, 0.4 / 3), ("bf16_dev", 2.0 ** -8, 0.4 / 3),
+                                              ("f16_rel", 2.0 ** -11, 1.0 / 3), ("bf16_rel", 2.0 ** -8, 1.0 / 3)])
+@pytest.mark.parametrize("calls", [[2], [3], [4, 1, 3]])
+def test_16_bit_formats(gpu_lib, storage, eps, vmax, collision, tau, geometry, calls):
+    """A run rounds what it stores (at most vmax) once going in and once coming out:
+    no further off than steps that do so each time, five such roundings a step (the
+    collision mixes the incoming ones with weights that sum to at most about 4)."""
+    shape = (61, 65, 70)
+    geo = dict(periodic={}, mirror=dict(rho_s=(0.02, 0.05), wall_model="mirror", periodic=(1, 1, 0)),
+               mask=dict(rho_s=(0.02, 0.05), wall_model="mirror", solid=_scattered(shape)))[geometry]
+    if storage.endswith("_dev"):
+        geo["rho0_dev"] = 0.5
+    _compare(shape, collision, tau, calls, storage=storage, tol=sum(calls) * 5 * eps * vmax, **geo)
+
+
+@pytest.mark.parametrize("geometry", ["periodic", "mirror"])
+@pytest.mark.parametrize("collision,tau", KINDS)
+@pytest.mark.parametrize("shape", [(1, 9, 17), (1, 40, 1), (9, 1, 17), (5, 3, 2)])
+def test_small_relative_format(gpu_lib, shape, collision, tau, geometry):
+    """The relative formats run in moment space on lattices smaller than a tile too."""
+    geo = {} if geometry == "periodic" else dict(rho_s=(0.02, 0.05), wall_model=geometry, periodic=(1, 1, 0))
+    _compare(shape, collision, tau, [3], storage="f16_rel", tol=3 * 5 * 2.0 ** -11 / 3, **geo)
