@@ -99,15 +99,14 @@ k_moment_in(const typename Store<S>::T *__restrict__ f, MomentState<KIND> m, Phy
         m.put_solid(cell, make_float2(p.rho_s[0], p.rho_s[1]), N32);
         return;
     }
-    float2 v[Q], ref = make_float2(0.f, 0.f);
-    if constexpr (Store<S>::kRel) ref = state_ref(f, p.ref_off)[cell];
+    float2 v[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const bool wall = (cz(i) == 1 && n.zlo) || (cz(i) == -1 && n.zhi) || ((lw >> i) & 1u);
         const unsigned src = n.zo[1 - cz(i)] + n.yo[1 - cy(i)] + n.xo[1 - cx(i)];
         const typename Store<S>::T *q = f + 2 * (size_t)(wall ? (unsigned)opp(i) * N32 + cell : (unsigned)i * N32 + src);
         if constexpr (Store<S>::kDev) Store<S>::load2_d(q, v[i].x, v[i].y);   // (deviations have the momentum of the populations)
-        else Store<S>::load2(q, w<float>(i) * ref.x, w<float>(i) * ref.y, v[i].x, v[i].y);
+        else v[i] = ld_pair_f32(q);
     }
     float2 r = density(v);
     if constexpr (Store<S>::kDev) r = vadd(r, PairF32::dup(p.rho0));
@@ -128,9 +127,7 @@ k_moment_in(const typename Store<S>::T *__restrict__ f, MomentState<KIND> m, Phy
     }
 }
 
-// One thread per cell, bound by the bytes it stores.  The relative formats code a
-// population by the density of the cell that reads it next (x + c_i, or x itself
-// across a wall) and keep the cell's own.
+// One thread per cell, bound by the bytes it stores.
 template <int FMT, int KIND>
 __global__ void __launch_bounds__(kThreadsM)
 k_moment_out(MomentState<KIND> m, typename Store<FMT>::T *__restrict__ f, Phys<float> p, const unsigned *__restrict__ links)
@@ -138,15 +135,12 @@ k_moment_out(MomentState<KIND> m, typename Store<FMT>::T *__restrict__ f, Phys<f
     const unsigned cell = blockIdx.x * kThreadsM + threadIdx.x, N32 = (unsigned)p.N;
     if (cell >= N32) return;
     const Nb3 n = nb3(p, cell);
-    const unsigned lw = links ? __ldg(links + cell) : 0u;
-    const float base = Store<FMT>::kRel ? 1.0f : p.rho0;   // (a solid site's codes are those of the population steps)
-    if (lw & 1u) {
+    if (links && (__ldg(links + cell) & 1u)) {   // nothing in a solid site
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            const float e = Store<FMT>::enc(w<float>(i) * base);
+            const float e = w<float>(i) * p.rho0;
             Store<FMT>::store2(f + 2 * (size_t)((unsigned)i * N32 + cell), 0.f, 0.f, e, e);
         }
-        if constexpr (Store<FMT>::kRel) state_ref(f, p.ref_off)[cell] = make_float2(1.0f, 1.0f);
         return;
     }
     const float2 rs = make_float2(p.rho_s[0], p.rho_s[1]);
@@ -164,18 +158,10 @@ k_moment_out(MomentState<KIND> m, typename Store<FMT>::T *__restrict__ f, Phys<f
 #pragma unroll
     for (int k = 0; k < MomentState<KIND>::NP; ++k) mo.m[k] = m.P[(size_t)k * N32 + cell];
     auto get = [](int) { return make_float2(0.f, 0.f); };
-    if constexpr (Store<FMT>::kRel) state_ref(f, p.ref_off)[cell] = r;
     auto put = [&](int i, float2 v) {
         typename Store<FMT>::T *q = f + 2 * (size_t)((unsigned)i * N32 + cell);
-        if constexpr (Store<FMT>::kDev) {
-            Store<FMT>::store2_d(q, v.x, v.y);
-        } else if constexpr (Store<FMT>::kRel) {
-            const bool wall = (cz(i) == -1 && n.zlo) || (cz(i) == 1 && n.zhi) || ((lw >> opp(i)) & 1u);
-            const float2 e = wall || i == 0 ? r : __ldg(rho + n.zo[1 + cz(i)] + n.yo[1 + cy(i)] + n.xo[1 + cx(i)]);
-            Store<FMT>::store2(q, v.x, v.y, Store<FMT>::enc(w<float>(i) * e.x), Store<FMT>::enc(w<float>(i) * e.y));
-        } else {
-            Store<FMT>::store2(q, v.x, v.y, 0.f, 0.f);
-        }
+        if constexpr (Store<FMT>::kDev) Store<FMT>::store2_d(q, v.x, v.y);
+        else Store<FMT>::store2(q, v.x, v.y, 0.f, 0.f);
     };
     if constexpr (Store<FMT>::kDev) {   // collide_cell takes the second moments of the deviations
 #pragma unroll
@@ -537,7 +523,6 @@ Phys<float> make_phys_m(const HostPhys &h)
     for (int d = 0; d < 3; ++d) p.gext[d] = (float)h.gext[d];
     p.rho_s[0] = (float)h.rho_s[0]; p.rho_s[1] = (float)h.rho_s[1];
     p.rho0 = (float)h.rho0;
-    p.ref_off = h.ref_off;
     return p;
 }
 
@@ -615,13 +600,14 @@ inline unsigned grid_m(long long N) { return (unsigned)((N + kThreadsM - 1) / kT
 
 size_t moment_bytes(const HostPhys &h, long n)
 {
-    // Two steps of a relative format lose to the cost of coding the state (regularized,
-    // 256^3: 1892 us step by step, 2096 in moment space; three 2836, 2683); the others
-    // gain from two on (two steps, FP16 deviations regularized 256^3 1370, 1345, 61 x
-    // 65 x 70 70, 40; FP32 1768, 1657, 65, 42).
-    const bool rel = h.storage == ST_F16_REL || h.storage == ST_BF16_REL;
-    if (n < (rel && !tau_one(h) ? 3 : 2)) return 0;
-    if (h.storage == ST_F64 || h.forcing != FORCE_EDM || !fused_supported(h) || use_box(h)) return 0;
+    // From two steps on all gain (us, two steps one by one and in moment space: FP16
+    // deviations regularized 256^3 1370, 1345, 61 x 65 x 70 70, 40; FP32 1768, 1657,
+    // 65, 42).
+    if (n < 2) return 0;
+    // The relative formats stay step by step: they hand out FP32 reference densities,
+    // which carry every step's rounding to 16 bits.
+    if (h.storage != ST_F32 && h.storage != ST_F16_DEV && h.storage != ST_BF16_DEV) return 0;
+    if (h.forcing != FORCE_EDM || !fused_supported(h) || use_box(h)) return 0;
     const long long cols = (long long)((h.nx + kOX - 1) / kOX) * ((h.ny + Tile<COLL_REG, 12>::OY - 1) / Tile<COLL_REG, 12>::OY);
     if (cols >= (1LL << 31) || h.nz > 4 * 65535) return 0;   // grid limits
     const size_t N = (size_t)h.N;
@@ -686,8 +672,6 @@ cudaError_t launch_moment_in(const HostPhys &h, const void *f, void *m, cudaStre
     case ST_F32: return in_s<ST_F32>(h, f, m, s);
     case ST_F16_DEV: return in_s<ST_F16_DEV>(h, f, m, s);
     case ST_BF16_DEV: return in_s<ST_BF16_DEV>(h, f, m, s);
-    case ST_F16_REL: return in_s<ST_F16_REL>(h, f, m, s);
-    case ST_BF16_REL: return in_s<ST_BF16_REL>(h, f, m, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -703,8 +687,6 @@ cudaError_t launch_moment_out(const HostPhys &h, const void *m, void *f, cudaStr
     case ST_F32: return out_s<ST_F32>(h, m, f, s);
     case ST_F16_DEV: return out_s<ST_F16_DEV>(h, m, f, s);
     case ST_BF16_DEV: return out_s<ST_BF16_DEV>(h, m, f, s);
-    case ST_F16_REL: return out_s<ST_F16_REL>(h, m, f, s);
-    case ST_BF16_REL: return out_s<ST_BF16_REL>(h, m, f, s);
     default: return cudaErrorInvalidValue;
     }
 }
