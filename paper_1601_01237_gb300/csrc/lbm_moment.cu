@@ -1,4 +1,4 @@
-// Runs of steps in moment space (FP32 arithmetic, exact-difference forcing).
+// Runs of steps in moment space (FP32 arithmetic).
 //
 // Under the regularized operator a step reads its 38 populations only to form
 // the densities, the mixture momentum and (for tau != 1) the second moments
@@ -128,7 +128,7 @@ k_moment_in(const typename Store<S>::T *__restrict__ f, MomentState<KIND> m, Phy
 }
 
 // One thread per cell, bound by the bytes it stores.
-template <int FMT, int KIND>
+template <int FMT, int KIND, int FORCE>
 __global__ void __launch_bounds__(kThreadsM)
 k_moment_out(MomentState<KIND> m, typename Store<FMT>::T *__restrict__ f, Phys<float> p, const unsigned *__restrict__ links)
 {
@@ -168,7 +168,7 @@ k_moment_out(MomentState<KIND> m, typename Store<FMT>::T *__restrict__ f, Phys<f
         for (int k = 0; k < 3 && k < MomentState<KIND>::NP; ++k)
             mo.m[k] = vsub(mo.m[k], PairF32::dup(p.rho0 * (1.0f / 3.0f)));
     }
-    collide_cell<PairF32, KIND, FORCE_EDM, Store<FMT>::kDev>(PairF32(), p, r, 0.f, uxy.x, uxy.y, m.uz[cell], So, mo, get, put);
+    collide_cell<PairF32, KIND, FORCE, Store<FMT>::kDev>(PairF32(), p, r, 1.0f / (r.x + r.y), uxy.x, uxy.y, m.uz[cell], So, mo, get, put);
 }
 
 // Wall densities of the mirror model under a mask, after each new moment state:
@@ -324,7 +324,7 @@ struct Collect {
     }
 };
 
-template <int KIND, int EY, bool WALLZ, bool MASK>
+template <int KIND, int FORCE, int EY, bool WALLZ, bool MASK>
 __global__ void __launch_bounds__(Tile<KIND, EY>::threads, Tile<KIND, EY>::ctas)
 k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, int ntx, int lz,
               const unsigned *__restrict__ links)
@@ -449,8 +449,8 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
 #pragma unroll
                 for (int i = 0; i < Q; ++i) put(i, make_float2(0.f, 0.f));
             } else {
-                collide_cell<PairF32, KIND, FORCE_EDM, false>(PairF32(), p, r, 0.f, uxy_c.x, uxy_c.y, uz_c, So, mo_c, get,
-                                                              put);
+                collide_cell<PairF32, KIND, FORCE, false>(PairF32(), p, r, 1.0f / (r.x + r.y), uxy_c.x, uxy_c.y, uz_c, So,
+                                                          mo_c, get, put);
             }
         }
         __syncthreads();
@@ -560,7 +560,7 @@ Plan plan_of(const HostPhys &h)
 
 constexpr int kMaxAttrDevices = 64;
 
-template <int KIND, int EY, bool WALLZ, bool MASK>
+template <int KIND, int FORCE, int EY, bool WALLZ, bool MASK>
 cudaError_t launch_tile(const HostPhys &h, const Plan &q, const void *in, void *out, cudaStream_t s)
 {
     using T = Tile<KIND, EY>;
@@ -570,13 +570,13 @@ cudaError_t launch_tile(const HostPhys &h, const Plan &q, const void *in, void *
     if (e != cudaSuccess) return e;
     const bool cached = dev >= 0 && dev < kMaxAttrDevices;
     if (!cached || !attr_set[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute((const void *)k_step_moment<KIND, EY, WALLZ, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute((const void *)k_step_moment<KIND, FORCE, EY, WALLZ, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(MomentSmem<T>));
         if (e != cudaSuccess) return e;
         if (cached) attr_set[dev].store(1, std::memory_order_release);
     }
     const dim3 grid((unsigned)q.cols, (unsigned)((h.nz + q.lz - 1) / q.lz));
-    k_step_moment<KIND, EY, WALLZ, MASK><<<grid, T::threads, sizeof(MomentSmem<T>), s>>>(
+    k_step_moment<KIND, FORCE, EY, WALLZ, MASK><<<grid, T::threads, sizeof(MomentSmem<T>), s>>>(
         MomentState<KIND>(const_cast<void *>(in), h.N), MomentState<KIND>(out, h.N), make_phys_m(h), q.ntx, q.lz, h.links);
     return cudaGetLastError();
 }
@@ -584,12 +584,17 @@ cudaError_t launch_tile(const HostPhys &h, const Plan &q, const void *in, void *
 template <int KIND, bool WALLZ, bool MASK>
 cudaError_t launch_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
 {
-    const Plan a = plan_of<KIND, 12>(h), b = plan_of<KIND, 16>(h);
+    constexpr int E = FORCE_EDM;
+    const Plan a = plan_of<KIND, 12>(h);
+    // Guo's forcing takes the tile of 12 rows (it needs the registers of it)
+    if (h.forcing == FORCE_GUO) return launch_tile<KIND, FORCE_GUO, 12, WALLZ, MASK>(h, a, in, out, s);
+    const Plan b = plan_of<KIND, 16>(h);
     if constexpr (KIND == COLL_EQ) {
         const Plan c = plan_of<KIND, 24>(h);
-        if (c.ns < a.ns && c.ns < b.ns) return launch_tile<KIND, 24, WALLZ, MASK>(h, c, in, out, s);
+        if (c.ns < a.ns && c.ns < b.ns) return launch_tile<KIND, E, 24, WALLZ, MASK>(h, c, in, out, s);
     }
-    return a.ns < b.ns ? launch_tile<KIND, 12, WALLZ, MASK>(h, a, in, out, s) : launch_tile<KIND, 16, WALLZ, MASK>(h, b, in, out, s);
+    return a.ns < b.ns ? launch_tile<KIND, E, 12, WALLZ, MASK>(h, a, in, out, s)
+                       : launch_tile<KIND, E, 16, WALLZ, MASK>(h, b, in, out, s);
 }
 
 bool tau_one(const HostPhys &h) { return (float)(1.0 / h.tau[0]) == 1.0f && (float)(1.0 / h.tau[1]) == 1.0f; }
@@ -600,14 +605,17 @@ inline unsigned grid_m(long long N) { return (unsigned)((N + kThreadsM - 1) / kT
 
 size_t moment_bytes(const HostPhys &h, long n)
 {
-    // From two steps on all gain (us, two steps one by one and in moment space: FP16
-    // deviations regularized 256^3 1370, 1345, 61 x 65 x 70 70, 40; FP32 1768, 1657,
-    // 65, 42).
-    if (n < 2) return 0;
+    // Short regularized runs of large lattices under Guo's forcing lose to the cost of
+    // the two ends (us at 256^3, step by step / in moment space: FP32 two 1771 / 1790,
+    // three 2654 / 2475, FP16 deviations three 2155 / 2205, ten 7178 / 7009); the others
+    // gain from two on (two steps, exact difference: FP16 deviations 1370 / 1345, FP32
+    // 1768 / 1657).
+    const int least = tau_one(h) || h.forcing != FORCE_GUO ? 2 : (h.storage == ST_F32 ? 3 : 6);
+    if (n < least) return 0;
     // The relative formats stay step by step: they hand out FP32 reference densities,
     // which carry every step's rounding to 16 bits.
     if (h.storage != ST_F32 && h.storage != ST_F16_DEV && h.storage != ST_BF16_DEV) return 0;
-    if (h.forcing != FORCE_EDM || !fused_supported(h) || use_box(h)) return 0;
+    if (!fused_supported(h) || use_box(h)) return 0;
     const long long cols = (long long)((h.nx + kOX - 1) / kOX) * ((h.ny + Tile<COLL_REG, 12>::OY - 1) / Tile<COLL_REG, 12>::OY);
     if (cols >= (1LL << 31) || h.nz > 4 * 65535) return 0;   // grid limits
     const size_t N = (size_t)h.N;
@@ -644,10 +652,10 @@ cudaError_t moment_step_t(const HostPhys &h, const void *in, void *out, cudaStre
     return e == cudaSuccess ? moment_walls<KIND>(h, out, s) : e;
 }
 
-template <int S, int KIND>
+template <int S, int KIND, int FORCE>
 cudaError_t moment_out_t(const HostPhys &h, const void *m, void *f, cudaStream_t s)
 {
-    k_moment_out<S, KIND><<<grid_m(h.N), kThreadsM, 0, s>>>(MomentState<KIND>(const_cast<void *>(m), h.N),
+    k_moment_out<S, KIND, FORCE><<<grid_m(h.N), kThreadsM, 0, s>>>(MomentState<KIND>(const_cast<void *>(m), h.N),
                                                             (typename Store<S>::T *)f, make_phys_m(h), h.links);
     return cudaGetLastError();
 }
@@ -661,7 +669,9 @@ cudaError_t in_s(const HostPhys &h, const void *f, void *m, cudaStream_t s)
 template <int S>
 cudaError_t out_s(const HostPhys &h, const void *m, void *f, cudaStream_t s)
 {
-    return tau_one(h) ? moment_out_t<S, COLL_EQ>(h, m, f, s) : moment_out_t<S, COLL_REG>(h, m, f, s);
+    if (h.forcing == FORCE_GUO)
+        return tau_one(h) ? moment_out_t<S, COLL_EQ, FORCE_GUO>(h, m, f, s) : moment_out_t<S, COLL_REG, FORCE_GUO>(h, m, f, s);
+    return tau_one(h) ? moment_out_t<S, COLL_EQ, FORCE_EDM>(h, m, f, s) : moment_out_t<S, COLL_REG, FORCE_EDM>(h, m, f, s);
 }
 
 }  // namespace

@@ -67,3 +67,16 @@ def test_16_bit_formats(gpu_lib, storage, eps, vmax, collision, tau, geometry, c
     geo = dict(periodic={}, mirror=dict(rho_s=(0.02, 0.05), wall_model="mirror", periodic=(1, 1, 0)),
                mask=dict(rho_s=(0.02, 0.05), wall_model="mirror", solid=_scattered(shape)))[geometry]
     _compare(shape, collision, tau, calls, storage=storage, tol=sum(calls) * 5 * eps * vmax, rho0_dev=0.5, **geo)
+
+
+@pytest.mark.parametrize("geometry", ["periodic", "mirror", "mask"])
+@pytest.mark.parametrize("collision,tau", KINDS)
+@pytest.mark.parametrize("storage", ["f32", "f16_dev"])
+@pytest.mark.parametrize("shape,calls", [(TILES[0], [3]), ((61, 65, 70), [2, 1, 6])])
+def test_guo_forcing(gpu_lib, shape, calls, storage, collision, tau, geometry):
+    geo = dict(periodic={}, mirror=dict(rho_s=(0.02, 0.05), wall_model="mirror", periodic=(1, 1, 0)),
+               mask=dict(rho_s=(0.02, 0.05), wall_model="mirror", solid=_scattered(shape)))[geometry]
+    if storage == "f16_dev":
+        geo["rho0_dev"] = 0.5
+    tol = None if storage == "f32" else sum(calls) * 5 * 2.0 ** -11 / 3
+    _compare(shape, collision, tau, calls, storage=storage, tol=tol, forcing="guo", **geo)
