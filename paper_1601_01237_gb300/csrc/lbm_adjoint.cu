@@ -33,6 +33,12 @@ int adjoint_blocks(int storage)
     return per_sm * current_device_sms();
 }
 
+bool adjoint_eq(const HostPhys &h, int rho_is_sums)
+{
+    return rho_is_sums && h.storage != ST_F64 && h.forcing == FORCE_EDM && (float)(1.0 / h.tau[0]) == 1.0f &&
+           (float)(1.0 / h.tau[1]) == 1.0f;
+}
+
 cudaError_t launch_adjoint_step(const HostPhys &p, const void *f, const void *rho, int rho_is_sums, const void *lam_next,
                                 const void *Dn, void *lam_loc, void *a, void *Dout, double *partials, cudaStream_t s)
 {
@@ -47,9 +53,14 @@ cudaError_t launch_adjoint_step(const HostPhys &p, const void *f, const void *rh
     }
 }
 
-cudaError_t launch_adjoint_seed(const HostPhys &p, const void *g1, const void *g2, int g_f64, void *lam,
-                                cudaStream_t s)
+cudaError_t launch_adjoint_seed(const HostPhys &p, const void *g1, const void *g2, int g_f64, void *lam, void *D,
+                                int rho_is_sums, cudaStream_t s)
 {
+    if (adjoint_eq(p, rho_is_sums)) {
+        if (g_f64) k_adj_seed_eq<<<gridA(p.N), kThreadsA, 0, s>>>((const double *)g1, (const double *)g2, (float *)lam, (float *)D, p.N);
+        else k_adj_seed_eq<<<gridA(p.N), kThreadsA, 0, s>>>((const float *)g1, (const float *)g2, (float *)lam, (float *)D, p.N);
+        return cudaGetLastError();
+    }
     if (p.storage == ST_F64) {
         if (g_f64) k_adj_seed<double, double><<<gridA(p.N), kThreadsA, 0, s>>>((const double *)g1, (const double *)g2, (double *)lam, p.N);
         else k_adj_seed<double, float><<<gridA(p.N), kThreadsA, 0, s>>>((const float *)g1, (const float *)g2, (double *)lam, p.N);
@@ -61,8 +72,9 @@ cudaError_t launch_adjoint_seed(const HostPhys &p, const void *g1, const void *g
 }
 
 cudaError_t launch_adjoint_rho0(const HostPhys &p, const void *lam, const void *D, double *g1, double *g2,
-                                cudaStream_t s)
+                                int rho_is_sums, cudaStream_t s)
 {
+    if (adjoint_eq(p, rho_is_sums)) lam = nullptr;
     if (p.storage == ST_F64)
         k_adj_rho0<double><<<gridA(p.N), kThreadsA, 0, s>>>((const double *)lam, (const double *)D, g1, g2, p.N,
                                                             p.solid);

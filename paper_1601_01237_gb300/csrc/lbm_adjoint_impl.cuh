@@ -22,6 +22,17 @@
 // k_adj_rho0 (dL/drho_0 = sum_i w_i lambda^0_i for an initial state
 // f^eq(rho_0, u = 0)).
 //
+// At tau = 1 in both components (EQ instances) a step keeps nothing of its
+// populations but the densities and the mixture momentum, so that
+//   lambda_loc_i(y) = base_a(y) + c_i . jb(y)
+// with one base per component and one vector jb for both: lambda_loc is then held
+// as these 5 values per cell instead of 38 (jb as 4-vectors [N], behind them
+// base[2][N]), and k_adj_D adds base to D, so that the next reverse step gathers
+//   mu_i(y) = D_a(y + c_i) + c_i . jb(y + c_i).
+// us per reverse step with its replay, 38 values and 5: 96^3 184 / 154, 128^3 472 / 343,
+// masked 96^3 214 / 188; what is left waits on the 19 populations and 19 cached
+// sensitivities that each lane gathers.
+//
 // Kernel templates of the reverse step; adj::adj_step_t is instantiated per
 // storage format in lbm_adjoint_<format>.cu (compiled in parallel), and
 // lbm_adjoint.cu dispatches over the formats.
@@ -101,7 +112,7 @@ __device__ __forceinline__ unsigned at(const Nb &n, int dx, int dy, int dz)
 //   mu_i(y) = lambda^{n+1}_i(y + c_i) = lambda_loc^{n+1}_i(y + c_i) + D^{n+1}_a(y + c_i)
 // (or lambda^{n+1}_opp(i)(y) at a wall), and writes lambda_loc^n_i(y) of its
 // component and a^n_b(y) of the other component b = 1 - a.
-template <int S, int REG, bool SIN, bool MASK, bool WZ, int FORCE>
+template <int S, int REG, bool SIN, bool MASK, bool WZ, int FORCE, bool EQ>
 __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict__ f,
                                          const typename Store<S>::R *__restrict__ rho,
                                          const typename Store<S>::R *__restrict__ lam_next,
@@ -135,7 +146,22 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
     // ---- incoming sensitivities (issued with the population loads, so that
     //      both sets of gathers are in flight together) ----------------------
     R mu[Q];
-    {
+    if constexpr (EQ) {
+        const float4 *jn = reinterpret_cast<const float4 *>(lam_next);
+        const R *D_a = Dn + (size_t)a * (size_t)N;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const bool wall = (cz(i) == -1 && zlo) || (cz(i) == 1 && zhi) ||
+                              (MASK && i != 0 && ((lw >> opp(i)) & 1u));   // y + c_i solid
+            const unsigned cell = wall ? n.cell : at(n, cx(i), cy(i), cz(i));
+            mu[i] = D_a[cell];
+            if (i > 0) {
+                const float4 j = __ldg(jn + cell);
+                const R d = cdot<R>(i, j.x, j.y, j.z);
+                mu[i] += wall ? -d : d;
+            }
+        }
+    } else {
         const R *lam_a = lam_next + (size_t)a * Q * (size_t)N;
         const R *D_a = Dn + (size_t)a * (size_t)N;
 #pragma unroll
@@ -272,21 +298,29 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
         vbv += R(3) * mk;
         if (!REG) {
             const R Pu = R(1) - R(1.5) * usq;
-            Kbar += m * (fa[0] - rq * R(12) * Pu);
-            rbar -= keep * mk * Pu;
-            ubv += R(3) * mk;
+            if constexpr (!EQ) Kbar += m * (fa[0] - rq * R(12) * Pu);
+            if constexpr (!EQ) {
+                rbar -= keep * mk * Pu;
+                ubv += R(3) * mk;
+            }
         } else {
-            Kbar += mk * R(0.125) * (-tr / R(3));
-            const R nb = keep * mk * R(0.125);
-            pb[0] -= nb / R(3);
-            pb[1] -= nb / R(3);
-            pb[2] -= nb / R(3);
+            if constexpr (!EQ) Kbar += mk * R(0.125) * (-tr / R(3));
+            if constexpr (!EQ) {
+                const R nb = keep * mk * R(0.125);
+                pb[0] -= nb / R(3);
+                pb[1] -= nb / R(3);
+                pb[2] -= nb / R(3);
+            }
         }
     }
+    // (EQ: the non-equilibrium populations of Kbar sum to zero, so that it takes mu
+    // relative to the rest direction's: smaller terms, smaller rounding)
+    const R mu0 = EQ ? mu[0] : R(0);
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
         const R ki = R(k36(i));
         const R sg = (mu[i] + mu[i + 1]) * ki, df = (mu[i] - mu[i + 1]) * ki;
+        const R sk = EQ ? sg - R(2) * ki * mu0 : sg;
         const R cv = cdot<R>(i, v0, v1, v2), cv2 = cv * cv;
         const R E = R(1) + R(4.5) * cv2 - R(1.5) * vsq, O = cv * (R(3) + R(4.5) * cv2 - R(4.5) * vsq);
         rbar += E * sg + O * df;
@@ -307,34 +341,40 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
         if (!REG) {
             const R cu = cdot<R>(i, u0, u1, u2), cu2 = cu * cu;
             const R Eu = R(1) + R(4.5) * cu2 - R(1.5) * usq, Ou = cu * (R(3) + R(4.5) * cu2 - R(4.5) * usq);
-            const R Pm = Eu * sg + Ou * df;
-            Kbar += mu[i] * fa[i] + mu[i + 1] * fa[i + 1] - rq * Pm;
-            rbar -= keep * Pm;
-            const R tu = (R(3) + R(13.5) * cu2 - R(4.5) * usq) * df + R(9) * cu * sg;
-            if (cx(i)) ubx += R(cx(i)) * tu;
-            if (cy(i)) uby += R(cy(i)) * tu;
-            if (cz(i)) ubz += R(cz(i)) * tu;
-            ubv += R(3) * sg + R(9) * cu * df;
+            const R Pm = Eu * sk + Ou * df;
+            Kbar += (mu[i] - mu0) * fa[i] + (mu[i + 1] - mu0) * fa[i + 1] - rq * Pm;
+            if constexpr (!EQ) {
+                rbar -= keep * Pm;
+                const R tu = (R(3) + R(13.5) * cu2 - R(4.5) * usq) * df + R(9) * cu * sg;
+                if (cx(i)) ubx += R(cx(i)) * tu;
+                if (cy(i)) uby += R(cy(i)) * tu;
+                if (cz(i)) ubz += R(cz(i)) * tu;
+                ubv += R(3) * sg + R(9) * cu * df;
+            }
         } else {
             const int c0 = cx(i), c1 = cy(i), c2 = cz(i);
             const R ccP = R(c0 * c0) * Pi[0] + R(c1 * c1) * Pi[1] + R(c2 * c2) * Pi[2] + R(2 * c0 * c1) * Pi[3] +
                           R(2 * c0 * c2) * Pi[4] + R(2 * c1 * c2) * Pi[5];
-            Kbar += sg * R(0.125) * (ccP - tr / R(3));
-            const R nb = keep * sg * R(0.125);
-            pb[0] += nb * (R(c0 * c0) - R(1) / R(3));
-            pb[1] += nb * (R(c1 * c1) - R(1) / R(3));
-            pb[2] += nb * (R(c2 * c2) - R(1) / R(3));
-            if (c0 && c1) pb[3] += nb * R(c0 * c1);
-            if (c0 && c2) pb[4] += nb * R(c0 * c2);
-            if (c1 && c2) pb[5] += nb * R(c1 * c2);
+            Kbar += sk * R(0.125) * (ccP - tr / R(3));
+            if constexpr (!EQ) {
+                const R nb = keep * sg * R(0.125);
+                pb[0] += nb * (R(c0 * c0) - R(1) / R(3));
+                pb[1] += nb * (R(c1 * c1) - R(1) / R(3));
+                pb[2] += nb * (R(c2 * c2) - R(1) / R(3));
+                if (c0 && c1) pb[3] += nb * R(c0 * c1);
+                if (c0 && c2) pb[4] += nb * R(c0 * c2);
+                if (c1 && c2) pb[5] += nb * R(c1 * c2);
+            }
             if (REG == 2) {
                 // f*_i +- keep (k_i / 8) sum_a (S_a h3s3(i, a) + D_a h3d(i, a)) for i, opp(i)
                 Kbar += df * R(0.125) * (th.odd(i) / (R(k36(i)) * R(0.125)));
-                const R nd = keep * df * R(0.125);
+                if constexpr (!EQ) {
+                    const R nd = keep * df * R(0.125);
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    if (h3s3(i, q)) sb[q] += nd * R(h3s3(i, q));
-                    if (h3d(i, q)) db[q] += nd * R(h3d(i, q));
+                    for (int q = 0; q < 3; ++q) {
+                        if (h3s3(i, q)) sb[q] += nd * R(h3s3(i, q));
+                        if (h3d(i, q)) db[q] += nd * R(h3d(i, q));
+                    }
                 }
             }
         }
@@ -343,7 +383,9 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
     // dL/dv^a
     const R vbar0 = rq * (vbx - v0 * vbv), vbar1 = rq * (vby - v1 * vbv), vbar2 = rq * (vbz - v2 * vbv);
     R ub0 = vbar0, ub1 = vbar1, ub2 = vbar2;
-    if (!REG) {
+    if (EQ) {
+        // (keep = 0: v = u + g^a is all that depends on u)
+    } else if (!REG) {
         ub0 -= keep * rq * (ubx - u0 * ubv);
         ub1 -= keep * rq * (uby - u1 * ubv);
         ub2 -= keep * rq * (ubz - u2 * ubv);
@@ -411,7 +453,22 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
     const R base = rbar - (U0 * u0 + U1 * u1 + U2 * u2) / rt;
     // dL/dg^a: the velocity shift v = u + g^a (exact difference), or rho^a dL/dF^a (Guo)
     const R gb0 = guo ? ra * Fb0 : vbar0, gb1 = guo ? ra * Fb1 : vbar1, gb2 = guo ? ra * Fb2 : vbar2;
-    if (store && MASK && (lw & 1u)) {
+    if constexpr (EQ) {
+        if (store) {
+            const bool solid = MASK && (lw & 1u);   // no sensitivities (a = 0 keeps it out of D)
+            if (a == 0)
+                reinterpret_cast<float4 *>(lam_loc)[n.cell] =
+                    solid ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(jb0, jb1, jb2, 0.f);
+            lam_loc[(size_t)(4 + a) * (size_t)N + n.cell] = solid ? R(0) : base;
+            aout[((long long)b * 3 + 0) * N + n.cell] = solid ? R(0) : Ga * gb0;
+            aout[((long long)b * 3 + 1) * N + n.cell] = solid ? R(0) : Ga * gb1;
+            aout[((long long)b * 3 + 2) * N + n.cell] = solid ? R(0) : Ga * gb2;
+            if (!solid) {
+                par_g += gb0 * Sb0 + gb1 * Sb1 + gb2 * Sb2;
+                par_t += Kbar * omega * omega;
+            }
+        }
+    } else if (store && MASK && (lw & 1u)) {
         // solid site: no populations, no sensitivities (a = 0 keeps it out of D)
         R *lo = lam_loc + (size_t)a * Q * (size_t)N + n.cell;
 #pragma unroll
@@ -456,7 +513,7 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
 // solid).  The lanes of a solid site still run the arithmetic (on meaningless
 // values), so that both lanes of every pair take part in the shuffles, and
 // store zeros.
-template <int S, int REG, bool SIN, bool MASK, bool WZ, int FORCE>
+template <int S, int REG, bool SIN, bool MASK, bool WZ, int FORCE, bool EQ>
 __global__ void __launch_bounds__(AdjLaunch<typename Store<S>::R>::threads, AdjLaunch<typename Store<S>::R>::blocks)
 k_adj_local(const typename Store<S>::T *__restrict__ f, const typename Store<S>::R *__restrict__ rho,
             const typename Store<S>::R *__restrict__ lam_next, const typename Store<S>::R *__restrict__ Dn,
@@ -496,7 +553,7 @@ k_adj_local(const typename Store<S>::T *__restrict__ f, const typename Store<S>:
         py -= cyr * ny;
         pz += sz + cyr;
         const unsigned lw = MASK ? __ldg(links + n.cell) : 0u;
-        adj_half<S, REG, SIN, MASK, WZ, FORCE>(f, rho, lam_next, Dn, lam_loc, aout, p, n, a, valid, pg, pt, lw);
+        adj_half<S, REG, SIN, MASK, WZ, FORCE, EQ>(f, rho, lam_next, Dn, lam_loc, aout, p, n, a, valid, pg, pt, lw);
     }
     // lanes of component a hold parts of par[a] and par[2 + a]
     __shared__ double sh[4][kThreadsL];
@@ -533,7 +590,7 @@ struct DTile {
 
 template <class R>
 __global__ void __launch_bounds__(kThreadsA, 2)
-k_adj_D(const R *__restrict__ a, R *__restrict__ D, Phys<R> p, int ntx)
+k_adj_D(const R *__restrict__ a, const R *__restrict__ base, R *__restrict__ D, Phys<R> p, int ntx)
 {
     using T = DTile<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -643,8 +700,8 @@ k_adj_D(const R *__restrict__ a, R *__restrict__ D, Phys<R> p, int ntx)
         const int z = z0 + k;
         if (z < nz) {
             const unsigned cell = ((unsigned)z * (unsigned)ny + (unsigned)y) * (unsigned)nx + (unsigned)x;
-            D[cell] = acc[k][0];
-            D[N32 + cell] = acc[k][1];
+            D[cell] = acc[k][0] + (base ? base[cell] : R(0));
+            D[N32 + cell] = acc[k][1] + (base ? base[N32 + cell] : R(0));
         }
     }
 }
@@ -699,7 +756,21 @@ k_adj_seed(const G *__restrict__ g1, const G *__restrict__ g2, R *__restrict__ l
     }
 }
 
-// dL/drho^a_0 = sum_i w_i lambda^0_i = sum_i w_i lambda_loc^0_i + D^0_a (sum_i w_i = 1).
+// The same for the EQ instances: base = v1, v2 (in D, which has no other part at
+// the last step) and jb = 0.
+template <class G>
+__global__ void __launch_bounds__(kThreadsA)
+k_adj_seed_eq(const G *__restrict__ g1, const G *__restrict__ g2, float *__restrict__ lam, float *__restrict__ D, long long N)
+{
+    const long long c = (long long)blockIdx.x * kThreadsA + threadIdx.x;
+    if (c >= N) return;
+    D[c] = g1 ? (float)g1[c] : 0.f;
+    D[N + c] = g2 ? (float)g2[c] : 0.f;
+    reinterpret_cast<float4 *>(lam)[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// dL/drho^a_0 = sum_i w_i lambda^0_i = sum_i w_i lambda_loc^0_i + D^0_a (sum_i w_i = 1;
+// EQ instances, lam null: D has base, and sum_i w_i c_i = 0).
 template <class R>
 __global__ void __launch_bounds__(kThreadsA)
 k_adj_rho0(const R *__restrict__ lam, const R *__restrict__ D, double *__restrict__ g1, double *__restrict__ g2,
@@ -714,7 +785,7 @@ k_adj_rho0(const R *__restrict__ lam, const R *__restrict__ D, double *__restric
     }
     double s1 = 0, s2 = 0;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
+    for (int i = 0; lam && i < Q; ++i) {
         s1 += wd(i) * (double)lam[(long long)i * N + c];
         s2 += wd(i) * (double)lam[(long long)(Q + i) * N + c];
     }
@@ -746,7 +817,7 @@ constexpr int kMaxAttrDevices = 64;
 // Launch of the tiled D pass; its dynamic shared-memory attribute belongs to
 // the device context and is set once per device.
 template <class R>
-cudaError_t launch_adj_D(const HostPhys &h, const R *a, R *D, const Phys<R> &p, cudaStream_t s)
+cudaError_t launch_adj_D(const HostPhys &h, const R *a, const R *base, R *D, const Phys<R> &p, cudaStream_t s)
 {
     using T = DTile<R>;
     const int ntx = (h.nx + kDX - 1) / kDX, nty = (h.ny + kDY - 1) / kDY;
@@ -762,7 +833,7 @@ cudaError_t launch_adj_D(const HostPhys &h, const R *a, R *D, const Phys<R> &p, 
         if (e != cudaSuccess) return e;
         if (cached) attr_set[dev].store(1, std::memory_order_release);
     }
-    k_adj_D<R><<<dim3((unsigned)(ntx * nty), (unsigned)zb), kThreadsA, T::kSmem, s>>>(a, D, p, ntx);
+    k_adj_D<R><<<dim3((unsigned)(ntx * nty), (unsigned)zb), kThreadsA, T::kSmem, s>>>(a, base, D, p, ntx);
     return cudaGetLastError();
 }
 
@@ -777,16 +848,14 @@ cudaError_t adj_step_t(const HostPhys &h, const void *f, const void *rho, int rh
     using T = typename Store<S>::T;
     using R = typename Store<S>::R;
     const Phys<R> p = make_phys_a<R>(h);
+#define LBM_ADJ_I(REG_, SIN_, MASK_, WZ_, FORCE_, EQ_)                                                            \
+    k_adj_local<S, REG_, SIN_, MASK_, WZ_, FORCE_, EQ_><<<nblk, AdjLaunch<R>::threads, 0, s>>>(                   \
+        (const T *)f, (const R *)rho, (const R *)lam_next, (const R *)Dn, (R *)lam_loc, (R *)a, partials, p, h.links)
 #define LBM_ADJ(REG_, SIN_, MASK_, WZ_)                                                                           \
     do {                                                                                                          \
-        if (h.forcing == FORCE_GUO)                                                                               \
-            k_adj_local<S, REG_, SIN_, MASK_, WZ_, FORCE_GUO><<<nblk, AdjLaunch<R>::threads, 0, s>>>(             \
-                (const T *)f, (const R *)rho, (const R *)lam_next, (const R *)Dn, (R *)lam_loc, (R *)a, partials, \
-                p, h.links);                                                                                      \
-        else                                                                                                      \
-            k_adj_local<S, REG_, SIN_, MASK_, WZ_, FORCE_EDM><<<nblk, AdjLaunch<R>::threads, 0, s>>>(             \
-                (const T *)f, (const R *)rho, (const R *)lam_next, (const R *)Dn, (R *)lam_loc, (R *)a, partials, \
-                p, h.links);                                                                                      \
+        if (h.forcing == FORCE_GUO) LBM_ADJ_I(REG_, SIN_, MASK_, WZ_, FORCE_GUO, false);                          \
+        else if (eq) LBM_ADJ_I(REG_, SIN_, MASK_, WZ_, FORCE_EDM, (SIN_ && S != ST_F64));                         \
+        else LBM_ADJ_I(REG_, SIN_, MASK_, WZ_, FORCE_EDM, false);                                                 \
     } while (0)
 #define LBM_ADJ_REG(SIN_, MASK_, WZ_)                  \
     do {                                               \
@@ -796,6 +865,7 @@ cudaError_t adj_step_t(const HostPhys &h, const void *f, const void *rho, int rh
     } while (0)
     const int reg = h.collision == LBM_REGULARIZED ? 1 : (h.collision == LBM_REGULARIZED3 ? 2 : 0);
     const int nblk = adjoint_blocks(h.storage);
+    const bool eq = adjoint_eq(h, rho_is_sums);
     // geometry instances: a mask (periodic z), z walls, or periodic
     if (h.links) {
         if (rho_is_sums) LBM_ADJ_REG(true, true, false);
@@ -809,7 +879,8 @@ cudaError_t adj_step_t(const HostPhys &h, const void *f, const void *rho, int rh
     }
 #undef LBM_ADJ_REG
 #undef LBM_ADJ
-    cudaError_t e = launch_adj_D<R>(h, (const R *)a, (R *)Dout, p, s);
+#undef LBM_ADJ_I
+    cudaError_t e = launch_adj_D<R>(h, (const R *)a, eq ? (const R *)lam_loc + 4 * h.N : nullptr, (R *)Dout, p, s);
     if (e == cudaSuccess && h.links && h.wall_mirror && h.n_bfluid > 0) {
         k_adj_D_wall<R><<<gridA(h.n_bfluid), kThreadsA, 0, s>>>((R *)Dout, h.solid, p, h.bfluid, h.n_bfluid);
         e = cudaGetLastError();

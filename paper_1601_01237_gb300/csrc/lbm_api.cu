@@ -864,7 +864,7 @@ lbm_status lbm_adjoint(lbm_lattice *h, const double *dL_drho1, const double *dL_
         g1 = dL_drho1 ? io1 : nullptr;
         g2 = dL_drho2 ? io2 : nullptr;
     }
-    CKA(lbm::launch_adjoint_seed(h->phys, g1, g2, 1, lam, h->stream), "lbm_adjoint: seed");
+    CKA(lbm::launch_adjoint_seed(h->phys, g1, g2, 1, lam, dbuf, h->use_fused, h->stream), "lbm_adjoint: seed");
     void *d_cur = dbuf, *d_nxt = (char *)dbuf + rb * 2 * N;   // D^N = 0 (cleared above)
     const bool use_fused = h->use_fused;
     // One checkpoint segment of len steps on stream st: recompute its forward
@@ -957,7 +957,7 @@ lbm_status lbm_adjoint(lbm_lattice *h, const double *dL_drho1, const double *dL_
     if (dL_drho1_0 || dL_drho2_0) {
         double *o1 = on_device ? dL_drho1_0 : (dL_drho1_0 ? io1 : nullptr);
         double *o2 = on_device ? dL_drho2_0 : (dL_drho2_0 ? io2 : nullptr);
-        CKA(lbm::launch_adjoint_rho0(h->phys, lam, d_cur, o1, o2, h->stream), "lbm_adjoint: rho0");
+        CKA(lbm::launch_adjoint_rho0(h->phys, lam, d_cur, o1, o2, h->use_fused, h->stream), "lbm_adjoint: rho0");
         if (!on_device) {
             if (dL_drho1_0) CKA(cudaMemcpyAsync(dL_drho1_0, io1, sizeof(double) * N, cudaMemcpyDeviceToHost, h->stream), "lbm_adjoint: copy out");
             if (dL_drho2_0) CKA(cudaMemcpyAsync(dL_drho2_0, io2, sizeof(double) * N, cudaMemcpyDeviceToHost, h->stream), "lbm_adjoint: copy out");

@@ -122,15 +122,20 @@ cudaError_t launch_step_split_noalloc(const HostPhys &p, const void *f_in, void 
 // (adjoint_blocks(storage) x 4 doubles: dG12, dG21, dtau1, dtau2) accumulate.
 // lambda^n = lambda_loc^n + D^n of the population's component.
 int adjoint_blocks(int storage);
+// Whether the reverse step keeps lambda_loc as 5 values per cell (tau = 1, the
+// exact-difference forcing, FP32 arithmetic, replayed sums): these are in the lambda
+// buffer, base_a added to D.
+bool adjoint_eq(const HostPhys &h, int rho_is_sums);
 cudaError_t launch_adjoint_step(const HostPhys &p, const void *f, const void *rho, int rho_is_sums,
                                 const void *lam_next, const void *Dn, void *lam_loc, void *a, void *Dout,
                                 double *partials, cudaStream_t s);
-// lambda_loc^N_i = dL/drho^a of the component of i (g1/g2 may be NULL).
-cudaError_t launch_adjoint_seed(const HostPhys &p, const void *g1, const void *g2, int g_f64, void *lam,
-                                cudaStream_t s);
+// lambda_loc^N_i = dL/drho^a of the component of i (g1/g2 may be NULL); D^N, cleared by
+// the caller, takes it instead where adjoint_eq.
+cudaError_t launch_adjoint_seed(const HostPhys &p, const void *g1, const void *g2, int g_f64, void *lam, void *D,
+                                int rho_is_sums, cudaStream_t s);
 // dL/drho^a_0 = sum_i w_i lambda^0_i for an initial state f^eq(rho_0, u = 0).
 cudaError_t launch_adjoint_rho0(const HostPhys &p, const void *lam, const void *D, double *g1, double *g2,
-                                cudaStream_t s);
+                                int rho_is_sums, cudaStream_t s);
 // density pass only (rho = sum_i f_i, pull-gathered) into rho
 cudaError_t launch_density(const HostPhys &p, const void *f, void *rho, cudaStream_t s);
 

@@ -32,3 +32,28 @@ def test_recordings_in_a_row(gpu_lib, storage):
         fresh.close()
         assert all(np.array_equal(g, w) for g, w in zip(got, want))
     lat.close()
+
+
+@pytest.mark.parametrize("collision", ["bgk", "regularized", "regularized3"])
+@pytest.mark.parametrize("geometry", ["periodic", "mirror", "mask_mirror"])
+def test_reverse_step_of_tau_one(gpu_lib, collision, geometry):
+    """FP32 at tau = 1 against the FP64 reverse pass, which sums the general form: 20
+    dependent roundings a step, relative to the largest value."""
+    shape, steps = (10, 12, 35), 12
+    state = wl.random_state(shape, seed=3, rho_lo=0.4, rho_hi=0.6, u_max=0.0)[:2]
+    kw = dict(G12=-1.2, G21=-1.1, g_ext=(1e-4, -2e-4, 5e-5), collision=collision, rho_s=(0.02, 0.05))
+    solid = None
+    if geometry == "mirror":
+        kw.update(periodic=(1, 1, 0), wall_model="mirror")
+    elif geometry == "mask_mirror":
+        kw.update(wall_model="mirror")
+        solid = np.zeros(shape, np.uint8)
+        solid[:2, :, ::2] = 1
+        solid[5:7, 3:9, 10:20] = 1
+    got = []
+    for storage in ("f32", "f64"):
+        lat = gpu_run(shape, *state, None, 0, storage=storage, solid=solid, **kw)
+        got.append(_gradient(lat, state, steps, 5))
+        lat.close()
+    for g, w in zip(*got):
+        assert np.abs(g - w).max() < steps * 20 * 6.0e-8 * np.abs(w).max()
