@@ -14,8 +14,8 @@
 // bytes).  Every value is held and every sum taken in FP32, as in the
 // population steps; the state at the end of the call is the population state.
 // us per step in calls of 10 (512^3), 20 (256^3) and 100 steps, population steps and
-// these: tau = 1 512^3 6723 / 2800, 256^3 842 / 374, 128^3 119 / 57, 96^3 52 / 35,
-// regularized 256^3 883 / 594, 384 x 512 x 512 with walls 5900 / 3190,
+// these: tau = 1 512^3 6723 / 2650, 256^3 842 / 371, 128^3 119 / 55, 96^3 52 / 33,
+// regularized 256^3 883 / 592, 384 x 512 x 512 with walls 5900 / 3190,
 // tau = 1 under a mask 256^3 1020 / 405.
 #include <cuda_runtime.h>
 
@@ -365,6 +365,8 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
         if (WALLZ && (q < 0 || q >= nz)) return p.wall_mirror ? vadd(r, rs) : rs;
         return r;
     };
+    cudaTriggerProgrammaticLaunchCompletion();   // the next step may be set up
+    cudaGridDependencySynchronize();             // the previous step's moments
     // density plane z0 - 2 into its slot, z0 - 1 into registers
     const int first = z0 - 1;   // first plane that collides
     float2 r_next, h_next = make_float2(0.f, 0.f);
@@ -576,9 +578,22 @@ cudaError_t launch_tile(const HostPhys &h, const Plan &q, const void *in, void *
         if (cached) attr_set[dev].store(1, std::memory_order_release);
     }
     const dim3 grid((unsigned)q.cols, (unsigned)((h.nz + q.lz - 1) / q.lz));
-    k_step_moment<KIND, FORCE, EY, WALLZ, MASK><<<grid, T::threads, sizeof(MomentSmem<T>), s>>>(
-        MomentState<KIND>(const_cast<void *>(in), h.N), MomentState<KIND>(out, h.N), make_phys_m(h), q.ntx, q.lz, h.links);
-    return cudaGetLastError();
+    // Successive steps overlap at their ends (programmatic stream serialization):
+    // a step's CTAs are set up while the last wave of the previous one drains, and
+    // wait for it before their first access (us per step without and with: tau = 1 61 x
+    // 65 x 70 16.4 / 14.0, 100^3 35.0 / 32.9, regularized 20.5 / 17.1, 54.0 / 51.9).
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(T::threads);
+    c.dynamicSmemBytes = sizeof(MomentSmem<T>);
+    c.stream = s;
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k_step_moment<KIND, FORCE, EY, WALLZ, MASK>, MomentState<KIND>(const_cast<void *>(in), h.N),
+                              MomentState<KIND>(out, h.N), make_phys_m(h), q.ntx, q.lz, h.links);
 }
 
 template <int KIND, bool WALLZ, bool MASK>
