@@ -162,9 +162,11 @@ def measured_hbm_peak():
 
 # source files that define each timed kernel (a change to any of them voids
 # the committed DRAM-traffic figure of that kernel)
-KERNEL_SOURCES = {"k_step_fused": ("d3q19.cuh", "lbm_fused_impl.cuh"),
+KERNEL_SOURCES = {"k_step_fused": ("d3q19.cuh", "collide.cuh", "lbm_fused_impl.cuh"),
                   "k_density": ("d3q19.cuh", "lbm_forward.cu"),
-                  "k_collide": ("d3q19.cuh", "lbm_forward.cu")}
+                  "k_collide": ("d3q19.cuh", "lbm_forward.cu"),
+                  **{k: ("d3q19.cuh", "collide.cuh", "lbm_moment.cu")
+                     for k in ("k_step_moment", "k_moment_in", "k_moment_out")}}
 
 
 def kernel_source_hash(kernel):
@@ -194,13 +196,20 @@ def ncu_traffic(kernel, storage, cells):
     return e["dram_bytes_per_cell"] * cells
 
 
-def algorithmic_bytes_per_cell(kernel, storage):
+def algorithmic_bytes_per_cell(kernel, storage, tau_one=True):
     """Minimum HBM bytes per cell of one launch: every population read once
     and written once (2 components x 19 values x s bytes x 2, and for the
     relative 16-bit formats the cell's two FP32 reference densities read and
     written); the density pass of the two-kernel step reads the state and
-    writes 2 densities; the collision pass also reads the 2 densities."""
+    writes 2 densities; the collision pass also reads the 2 densities.  A step
+    in moment space reads and writes 5 FP32 values at tau = 1 and 17 otherwise
+    (regularized), and its first and last launches trade them for a state."""
     b = state_bytes_per_cell(storage)
+    m = 4 * (5 if tau_one else 17)
+    if kernel == "k_step_moment":
+        return 2 * m
+    if kernel in ("k_moment_in", "k_moment_out"):
+        return b + m
     r = 8 if storage == "f64" else 4
     if kernel == "k_density":
         return b + 2 * r
@@ -415,17 +424,19 @@ def run_ours(args, rank, world, local_rank):
     dom = max(kern, key=lambda k: kern[k][0])
     dom_ms, dom_n = kern[dom]
     per_launch_s = dom_ms / dom_n / 1e3
-    alg = algorithmic_bytes_per_cell(dom, storage) * cells
+    tau_one = all(float(t) == 1.0 for t in kw.get("tau", (1.0, 1.0)))
+    alg = algorithmic_bytes_per_cell(dom, storage, tau_one) * cells
     peak, peak_src = measured_hbm_peak()
     achieved = alg / per_launch_s / 1e9
-    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+    # (steps in moment space are bound by shared memory and FP32 issue together)
+    roofline = {"bound": "hbm" if dom != "k_step_moment" else "shared memory and issue", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": ncu_traffic(dom, storage, cells), "kernel": dom,
                 "algorithmic_bytes_per_launch": alg, "launch_ms": per_launch_s * 1e3,
                 "peak_source": peak_src,
                 "kernels": {k: {"ms_per_launch": v[0] / v[1], "launches": v[1],
                                 "share": v[0] / sum(x[0] for x in kern.values())} for k, v in kern.items()}}
-    step_bytes = state_bytes_per_cell(storage) * 2 * cells
-    roofline["step_frac_of_peak"] = step_bytes / (ms_max / args.steps / 1e3) / 1e9 / peak
+    step_bytes = sum(algorithmic_bytes_per_cell(k, storage, tau_one) * cells * v[1] for k, v in kern.items())
+    roofline["step_frac_of_peak"] = step_bytes / (ms_max / 1e3) / 1e9 / peak
 
     # ---- end to end through the public API with host buffers -------------
     e2e = None
@@ -461,8 +472,10 @@ def run_ours(args, rank, world, local_rank):
                        parallelism="replicas" if world > 1 else "single GPU",
                        **({"mask": mask_desc} if mask_desc else {})),
         "roofline": roofline,
-        # (a mask adds the two wall-density kernels of the mirror model per step)
-        "gpu_launches": sum(v[1] for v in kern.values()) * (3 if mask_desc and "k_step_fused" in kern else 1),
+        # (a mask adds the wall-density kernels of the mirror model: two per step, one
+        # after each new moment state)
+        "gpu_launches": sum(v[1] * ((3 if k == "k_step_fused" else 2 if k in ("k_step_moment", "k_moment_in") else 1)
+                                    if mask_desc else 1) for k, v in kern.items()),
         "clocks": clocks,
         "e2e": e2e,
         "mass": [red["mass1"], red["mass2"]],
