@@ -29,8 +29,8 @@
 // as these 5 values per cell instead of 38 (jb as 4-vectors [N], behind them
 // base[2][N]), and k_adj_D adds base to D, so that the next reverse step gathers
 //   mu_i(y) = D_a(y + c_i) + c_i . jb(y + c_i).
-// us per reverse step with its replay, 38 values and 5: 96^3 184 / 154, 128^3 472 / 343,
-// masked 96^3 214 / 188; what is left waits on the 19 populations and 19 cached
+// us per reverse step with its replay, 38 values and 5: 96^3 184 / 150, 128^3 472 / 334,
+// masked 96^3 214 / 176; what is left waits on the 19 populations and 19 cached
 // sensitivities that each lane gathers.
 //
 // Kernel templates of the reverse step; adj::adj_step_t is instantiated per
@@ -145,21 +145,23 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
     }
     // ---- incoming sensitivities (issued with the population loads, so that
     //      both sets of gathers are in flight together) ----------------------
-    R mu[Q];
+    // EQ: relative to the rest direction's mu0.  f* sums to rho and its other
+    // derivatives to zero, so that a constant in mu adds itself to dL/drho and
+    // nothing else: the sums below then round with mu's differences.
+    R mu[Q], mu0 = 0;
     if constexpr (EQ) {
         const float4 *jn = reinterpret_cast<const float4 *>(lam_next);
         const R *D_a = Dn + (size_t)a * (size_t)N;
+        mu0 = D_a[n.cell];
+        mu[0] = 0;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
+        for (int i = 1; i < Q; ++i) {
             const bool wall = (cz(i) == -1 && zlo) || (cz(i) == 1 && zhi) ||
                               (MASK && i != 0 && ((lw >> opp(i)) & 1u));   // y + c_i solid
             const unsigned cell = wall ? n.cell : at(n, cx(i), cy(i), cz(i));
-            mu[i] = D_a[cell];
-            if (i > 0) {
-                const float4 j = __ldg(jn + cell);
-                const R d = cdot<R>(i, j.x, j.y, j.z);
-                mu[i] += wall ? -d : d;
-            }
+            const float4 j = __ldg(jn + cell);
+            const R d = cdot<R>(i, j.x, j.y, j.z);
+            mu[i] = (D_a[cell] - mu0) + (wall ? -d : d);
         }
     } else {
         const R *lam_a = lam_next + (size_t)a * Q * (size_t)N;
@@ -298,13 +300,13 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
         vbv += R(3) * mk;
         if (!REG) {
             const R Pu = R(1) - R(1.5) * usq;
-            if constexpr (!EQ) Kbar += m * (fa[0] - rq * R(12) * Pu);
+            Kbar += m * (fa[0] - rq * R(12) * Pu);
             if constexpr (!EQ) {
                 rbar -= keep * mk * Pu;
                 ubv += R(3) * mk;
             }
         } else {
-            if constexpr (!EQ) Kbar += mk * R(0.125) * (-tr / R(3));
+            Kbar += mk * R(0.125) * (-tr / R(3));
             if constexpr (!EQ) {
                 const R nb = keep * mk * R(0.125);
                 pb[0] -= nb / R(3);
@@ -313,14 +315,10 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
             }
         }
     }
-    // (EQ: the non-equilibrium populations of Kbar sum to zero, so that it takes mu
-    // relative to the rest direction's: smaller terms, smaller rounding)
-    const R mu0 = EQ ? mu[0] : R(0);
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
         const R ki = R(k36(i));
         const R sg = (mu[i] + mu[i + 1]) * ki, df = (mu[i] - mu[i + 1]) * ki;
-        const R sk = EQ ? sg - R(2) * ki * mu0 : sg;
         const R cv = cdot<R>(i, v0, v1, v2), cv2 = cv * cv;
         const R E = R(1) + R(4.5) * cv2 - R(1.5) * vsq, O = cv * (R(3) + R(4.5) * cv2 - R(4.5) * vsq);
         rbar += E * sg + O * df;
@@ -341,8 +339,8 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
         if (!REG) {
             const R cu = cdot<R>(i, u0, u1, u2), cu2 = cu * cu;
             const R Eu = R(1) + R(4.5) * cu2 - R(1.5) * usq, Ou = cu * (R(3) + R(4.5) * cu2 - R(4.5) * usq);
-            const R Pm = Eu * sk + Ou * df;
-            Kbar += (mu[i] - mu0) * fa[i] + (mu[i + 1] - mu0) * fa[i + 1] - rq * Pm;
+            const R Pm = Eu * sg + Ou * df;
+            Kbar += mu[i] * fa[i] + mu[i + 1] * fa[i + 1] - rq * Pm;
             if constexpr (!EQ) {
                 rbar -= keep * Pm;
                 const R tu = (R(3) + R(13.5) * cu2 - R(4.5) * usq) * df + R(9) * cu * sg;
@@ -355,7 +353,7 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
             const int c0 = cx(i), c1 = cy(i), c2 = cz(i);
             const R ccP = R(c0 * c0) * Pi[0] + R(c1 * c1) * Pi[1] + R(c2 * c2) * Pi[2] + R(2 * c0 * c1) * Pi[3] +
                           R(2 * c0 * c2) * Pi[4] + R(2 * c1 * c2) * Pi[5];
-            Kbar += sk * R(0.125) * (ccP - tr / R(3));
+            Kbar += sg * R(0.125) * (ccP - tr / R(3));
             if constexpr (!EQ) {
                 const R nb = keep * sg * R(0.125);
                 pb[0] += nb * (R(c0 * c0) - R(1) / R(3));
@@ -380,6 +378,7 @@ __device__ __forceinline__ void adj_half(const typename Store<S>::T *__restrict_
         }
     }
     rbar /= R(36);
+    if constexpr (EQ) rbar += mu0;
     // dL/dv^a
     const R vbar0 = rq * (vbx - v0 * vbv), vbar1 = rq * (vby - v1 * vbv), vbar2 = rq * (vbz - v2 * vbv);
     R ub0 = vbar0, ub1 = vbar1, ub2 = vbar2;
