@@ -87,16 +87,22 @@ __host__ __device__ constexpr bool odd_dirs_lead_positive()
 }
 static_assert(odd_dirs_lead_positive(), "vdot takes the leading component of odd directions as +1");
 
-// x / 36 and x / 3.  FP32 splits the constant in two: within an ulp of the
-// rounded quotient and unbiased (a product with the rounded 1/36 alone would
-// add that constant's relative error to the mass at every collision); FP64
-// multiplies (its relative error 5e-17 stays below the rounding of the sums).
-__device__ __forceinline__ float2 vdivc(float2 x, double c)
+// x / N (N = 3, 36) with 1 / N in two parts: within an ulp of the quotient and
+// unbiased.  (A product with the rounded reciprocal alone carries that constant's
+// relative error, in FP64 5.55e-17 low, into every collision with the same sign.)
+template <int N>
+__device__ __forceinline__ float2 vdivc(float2 x)
 {
-    const float hi = (float)c, lo = (float)(c - (double)hi);
+    constexpr float hi = (float)(1.0 / N), lo = (float)(1.0 / N - (double)hi);
     return vfma(x, make_float2(hi, hi), vmul(x, make_float2(lo, lo)));
 }
-__device__ __forceinline__ double vdivc(double x, double c) { return x * c; }
+template <int N>
+__device__ __forceinline__ double vdivc(double x)
+{
+    // lo = (1 - N hi) / N; the products of N with the two halves of hi are exact
+    constexpr double hi = 1.0 / N, up = (double)(float)hi, lo = ((1.0 - N * up) - N * (hi - up)) / N;
+    return fma(x, hi, x * lo);
+}
 
 // Collision kinds of the kernels: the three operators, and EQ for tau = 1 in
 // both components, where 1 - 1/tau = 0: all three operators then give
@@ -231,14 +237,24 @@ static_assert(cx(7) == 1 && cy(7) == 1 && cz(11) == 1, "first diagonal of each a
 //   get   get(i): the pre-collision population of direction i (BGK only)
 //   put   put(i, o): receives the post-collision population of direction i
 // DEV: populations in and out are deviations d = f - w_i rho0 of the deviation
-// formats: a constant per unit weight more in each output, -omega rho0 under
-// BGK (keep f = keep d + keep w rho0), -rho0 under the regularized filter,
-// and rho0 T0 on the diagonal of the second moments.
+// formats (and rho0 T0 less on the diagonal of the second moments).
 //
-// f^eq of Eq. 3 is taken in s_i = 3 c_i . v: with A = 1 - 3/2 v^2,
-//   f^eq_i, f^eq_opp = rho w_i (E +- O),  E = A + s^2 / 2,  O = s (A + s^2 / 6),
-// with the density folded into A and the two factors once per weight, seven
-// operations per opposite pair (nine in c_i . v with a product by rho w_i).
+// f^eq of Eq. 3 is taken in s_i = 3 c_i . v: with B = -3/2 v^2 and A = 1 + B,
+//   f^eq_i, f^eq_opp = rho w_i (1 + E +- O),  E = B + s^2 / 2,  O = s (A + s^2 / 6).
+// With q = rho / 36 the parts q k E and q k O are small and q k is added last, so
+// that roundings of a population's size are made once per opposite pair and once per
+// direction (tau = 1 in FP32: once per direction); q, which all directions share, takes
+// its rounding out of the mass again by the rest direction, which has rho - 24 q in the
+// place of 12 q.  One collision's rms error in units of 2^-24 rho (2^-53 in FP64), BGK
+// with tau != 1 / regularized / tau = 1: mass 0.24 / 0.23 / 0.22, momentum 0.08 / 0.08 /
+// 0.06, pressure 0.22 / 0.20 / 0.15; with each direction's polynomial formed at scale 1
+// and multiplied by rho w_i 0.63 / 0.55 / 0.55, 0.11 / 0.08 / 0.08, 0.24 / 0.25 / 0.21;
+// with q A rounded once for all directions 0.90 / 0.83 / 0.68, 0.09 / 0.08 / 0.08, 0.31 /
+// 0.33 / 0.23, and in FP64 with q = rho times the rounded 1/36 a mean of -0.50 per step.
+// Parameter derivatives of 50 steps at 96^3 (six droplets, largest error over largest
+// value): with the last of these 6.5e-8 / 8.2e-8 / 7.6e-8 / 3.3e-8, here 2.0e-8 / 2.2e-8 /
+// 2.2e-8 / 3.1e-8.  us per step, that form and this one: 512^3 3052 / 3044, 256^3 393 /
+// 402, regularized 617 / 631, FP64 1 x 64 x 64 8.8 / 9.2.
 template <class C, int REG, int FORCE, bool DEV, class GET, class PUT>
 __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::R> &p, typename C::V r,
                                              typename C::R inv, typename C::R ux, typename C::R uy, typename C::R uz,
@@ -265,18 +281,26 @@ __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::
     }
     const R usq = ux * ux + uy * uy + uz * uz;
     const U Ux = C::dup(ux), Uy = C::dup(uy), Uz = C::dup(uz);
-    const U Au = C::dup(fma(usq, R(-1.5), R(1)));
+    const U Bu = C::dup(usq * R(-1.5)), Au = C::dup(fma(usq, R(-1.5), R(1)));
     const U three = C::dup(R(3));
     const U Sx = vmul(three, Ux), Sy = vmul(three, Uy), Sz = vmul(three, Uz);   // 3 u
-    const V rq = vdivc(r, 1.0 / 36.0);                                          // rho w_i = rq k_i
-    V vx, vy, vz, A;   // 3 v^a and A(v^a)
+    const V rq = vdivc<36>(r);   // rho w_i = rq k_i
+    V rd = r, dq = rq;           // less rho0 in the deviation formats
+    if constexpr (DEV) {
+        rd = vsub(r, C::dup(p.rho0));
+        dq = vdivc<36>(rd);
+    }
+    V vx, vy, vz, A, B;   // 3 v^a, A(v^a) and B(v^a)
     if constexpr (FORCE == FORCE_EDM) {
         vx = vadd(gx, Ux); vy = vadd(gy, Uy); vz = vadd(gz, Uz);
-        A = vfma(vfma(vx, vx, vfma(vy, vy, vmul(vz, vz))), C::dup(R(-1.5)), one);
+        const V sq = vfma(vx, vx, vfma(vy, vy, vmul(vz, vz)));
+        B = vmul(sq, C::dup(R(-1.5)));
+        A = vfma(sq, C::dup(R(-1.5)), one);
         vx = vmul(vx, three); vy = vmul(vy, three); vz = vmul(vz, three);
     } else {
         vx = Sx; vy = Sy; vz = Sz;
         A = Au;
+        B = Bu;
     }
     // Guo's forcing term k_i ((c.u*)(c.Q) 3 - u*.Q +- c.Q), Q = (3 cf / 36) F,
     // cf = 1 - 1/(2 tau) (BGK) or 1/2
@@ -289,23 +313,25 @@ __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::
     if constexpr (REG == COLL_BGK) {
         // f* = f^eq(v) - keep f^eq(u) + keep f; with Guo's forcing v = u and
         // f^eq(v) - keep f^eq(u) = omega f^eq(u)
-        const V keep = vsub(one, om);
-        const V re = FORCE == FORCE_GUO ? vmul(rq, om) : rq;
+        const V keep = vsub(one, om), oc = vsub(one, keep);   // oc: exactly what keep leaves (1 - omega rounds below 1/2)
+        const V re = FORCE == FORCE_GUO ? vmul(rq, oc) : rq;
         const V ra = vmul(re, A);
         const V h = vmul(re, C::dup(R(0.5))), t = vmul(re, C::dup(R(1.0 / 6.0)));
-        V nh, nt, na;    // -keep rq / 2, -keep rq / 6, -keep rq A(u)
-        V even0 = ra;    // k_i of it is what f* has at s = 0
+        V nh, nt, na;             // -keep rq / 2, -keep rq / 6, -keep rq A(u)
+        V even0 = vmul(re, B);    // E at s = 0
         if constexpr (FORCE == FORCE_EDM) {
-            const V nk = vmul(vsub(om, one), rq);
+            const V nk = vmul(vmul(keep, C::dup(R(-1))), rq);
             nh = vmul(nk, C::dup(R(0.5)));
             nt = vmul(nk, C::dup(R(1.0 / 6.0)));
             na = vmul(nk, Au);
-            even0 = vadd(ra, na);
+            even0 = vfma(nk, Bu, even0);
         } else {
-            even0 = vsub(ra, uQ);
+            even0 = vsub(even0, uQ);
         }
-        if constexpr (DEV) even0 = vfma(om, C::dup(p.rho0 * R(-1.0 / 36.0)), even0);
-        put(0, vfma(even0, C::dup(R(12)), vmul(keep, get(0))));
+        // omega rho - 36 q: 32 q is exact, and what is left after it a ninth of the size
+        const V q = vmul(oc, dq), q2 = vadd(q, q);
+        const V left = vfma(q, C::dup(R(-4)), vfma(oc, rd, vmul(q, C::dup(R(-32)))));
+        put(0, vfma(even0, C::dup(R(12)), vfma(q, C::dup(R(12)), vfma(keep, get(0), left))));
 #pragma unroll
         for (int i = 1; i < Q; i += 2) {
             const V s = vdot(i, vx, vy, vz), m = vmul(s, s);
@@ -319,9 +345,11 @@ __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::
                 P = vfma(cQ, s, P);
                 M = vadd(M, cQ);
             }
-            if (i < 7) { P = vadd(P, P); M = vadd(M, M); }
-            put(i, vfma(keep, get(i), vadd(P, M)));
-            put(i + 1, vfma(keep, get(i + 1), vsub(P, M)));
+            // (keep f + k q has the size of a population, so that two roundings of that size are made)
+            const V a = vfma(keep, get(i), i < 7 ? q2 : q), b = vfma(keep, get(i + 1), i < 7 ? q2 : q);
+            const V x = vadd(P, M), y = vsub(P, M);
+            put(i, i < 7 ? vfma(x, C::dup(R(2)), a) : vadd(a, x));
+            put(i + 1, i < 7 ? vfma(y, C::dup(R(2)), b) : vadd(b, y));
         }
     } else {
         // Pi = sum c c f - rho (T0 I + u u) [+ (u F + F u) / 2], times keep / 8:
@@ -331,9 +359,8 @@ __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::
         const V k8 = vmul(vsub(one, om), C::dup(R(0.125)));
         const V ra = vmul(rq, A);
         const V h = vmul(rq, C::dup(R(0.5))), t6 = vmul(rq, C::dup(R(1.0 / 6.0)));
-        V even0 = ra;   // the part of f* / k_i that all directions share
+        V even0 = vmul(rq, B);   // E at s = 0
         if constexpr (FORCE == FORCE_GUO) even0 = vsub(even0, uQ);
-        if constexpr (DEV) even0 = vsub(even0, C::dup(p.rho0 * R(1.0 / 36.0)));
         V P[6], axis[3], diag[3];   // even0 + f^neq / k_i of the axes and, but for the P_ab term, of the diagonals
         if constexpr (kNeq) {
             const R T0 = R(1) / R(3);
@@ -357,7 +384,7 @@ __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::
             P[3] = off(3, ux, uy, Fx, Fy);
             P[4] = off(4, ux, uz, Fx, Fz);
             P[5] = off(5, uy, uz, Fy, Fz);
-            even0 = vsub(even0, vdivc(vadd(P[0], vadd(P[1], P[2])), 1.0 / 3.0));
+            even0 = vsub(even0, vdivc<3>(vadd(P[0], vadd(P[1], P[2]))));
             axis[0] = vadd(even0, P[0]);
             axis[1] = vadd(even0, P[1]);
             axis[2] = vadd(even0, P[2]);
@@ -371,12 +398,16 @@ __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 const R ub = u[a == 0 ? 1 : 0], uc = u[a == 2 ? 1 : 2];
-                const R eq = R(0.5) * u[a] * (ub * ub + uc * uc), dq = R(1.5) * u[a] * (ub * ub - uc * uc);
-                s3[a] = vmul(k8, vfma(nr, C::dup(eq), vdivc(mom.m[6 + a], 1.0 / 3.0)));
-                d3[a] = vmul(k8, vfma(nr, C::dup(dq), mom.m[9 + a]));
+                const R hs = R(0.5) * u[a] * (ub * ub + uc * uc), hd = R(1.5) * u[a] * (ub * ub - uc * uc);
+                s3[a] = vmul(k8, vfma(nr, C::dup(hs), vdivc<3>(mom.m[6 + a])));
+                d3[a] = vmul(k8, vfma(nr, C::dup(hd), mom.m[9 + a]));
             }
         }
-        put(0, vmul(even0, C::dup(R(12))));
+        constexpr bool kPlain = !kNeq && FORCE == FORCE_EDM;   // f^eq(v) alone
+        const V q2 = vadd(dq, dq), rq2 = vadd(rq, rq);
+        // rho - 24 q is rounded before E joins it: half of its values are ties, which an E
+        // that is never positive at tau = 1 would all turn down
+        put(0, vfma(even0, C::dup(R(12)), vfma(dq, C::dup(R(-24)), rd)));
 #pragma unroll
         for (int i = 1; i < Q; i += 2) {
             V b = even0;
@@ -386,7 +417,25 @@ __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::
                                             : vsub(diag[(i - 7) / 4], P[3 + (i - 7) / 4]);
             }
             const V s = vdot(i, vx, vy, vz), m = vmul(s, s);
-            V e = vfma(m, h, b), o = vmul(s, vfma(m, t6, ra));
+            if constexpr (kPlain && sizeof(R) == 4) {
+                // (q outside the polynomials: constants in the place of the pairs h, t6 and ra, for
+                // which the moment step's tiles of 16 rows have no registers: 512^3 3044 us per step,
+                // with them 3954)
+                const V x = vfma(m, C::dup(R(0.5)), B), y = vmul(s, vfma(m, C::dup(R(1.0 / 6.0)), A));
+                put(i, vfma(i < 7 ? rq2 : rq, vadd(x, y), i < 7 ? q2 : dq));
+                put(i + 1, vfma(i < 7 ? rq2 : rq, vsub(x, y), i < 7 ? q2 : dq));
+                continue;
+            }
+            V e = vfma(m, h, b);
+            if constexpr (sizeof(R) == 8 && FORCE == FORCE_EDM && REG != COLL_REG3) {
+                // (an operation less; a negated factor costs the packed form one)
+                const V O = vfma(m, t6, ra), t = i < 7 ? vadd(s, s) : s;
+                e = i < 7 ? vfma(e, C::dup(R(2)), q2) : vadd(e, dq);
+                put(i, vfma(t, O, e));
+                put(i + 1, vfma(-t, O, e));
+                continue;
+            }
+            V o = vmul(s, vfma(m, t6, ra));
             if constexpr (FORCE == FORCE_GUO) {
                 const V cQ = vdot(i, Qx, Qy, Qz);
                 e = vfma(cQ, s, e);
@@ -404,9 +453,15 @@ __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::
                 }
                 o = t;
             }
-            if (i < 7) { e = vadd(e, e); o = vadd(o, o); }
-            put(i, vadd(e, o));
-            put(i + 1, vsub(e, o));
+            if (i < 7) {   // k_i = 2
+                e = vfma(e, C::dup(R(2)), q2);
+                put(i, vfma(o, C::dup(R(2)), e));
+                put(i + 1, vfma(o, C::dup(R(-2)), e));
+            } else {
+                e = vadd(e, dq);
+                put(i, vadd(e, o));
+                put(i + 1, vsub(e, o));
+            }
         }
     }
 }

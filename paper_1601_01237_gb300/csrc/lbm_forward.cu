@@ -302,7 +302,7 @@ k_collide(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T *__
 //     34^3 lattice on 2 CTAs per busy SM, and a 64^2 one on 16 SMs;
 //   - the densities are formed once, in the density pass, and the collision
 //     reads its own back instead of summing them again;
-//   - the seven-operations-per-pair form of the collision;
+//   - the collision in 3 c.v, six or seven operations per pair;
 //   - warps inside a wall do no arithmetic.
 // Of CTAs of 32, 64 and 128 threads the smallest leaves the least imbalance
 // (34^3 39.5 / 42.7 / 42.7 us per step).  us per step before and now: 1 x 64 x 64
