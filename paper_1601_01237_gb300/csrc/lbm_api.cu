@@ -356,6 +356,13 @@ bool build_graph(lbm_lattice *h)
     return ok;
 }
 
+// Whether two moment states of that many bytes fit one population copy.
+size_t moment_stride(size_t bytes) { return (bytes + 255) / 256 * 256; }
+bool moment_one_copy(const lbm_lattice *h, size_t bytes)
+{
+    return 2 * moment_stride(bytes) <= lbm::state_bytes(h->phys.storage, h->phys.N);
+}
+
 // n >= 2 steps in moment space: the two moment states live in the population
 // copy that does not hold the state or, where two do not fit (16-bit formats), one
 // in each copy (the populations have been read by then), and the last step writes
@@ -363,8 +370,8 @@ bool build_graph(lbm_lattice *h)
 // n + 2 events): recorded before the first launch and after each of the n + 1.
 cudaError_t moment_run(lbm_lattice *h, long n, size_t bytes, cudaEvent_t *ev = nullptr)
 {
-    const size_t stride = (bytes + 255) / 256 * 256;
-    const bool one_copy = 2 * stride <= lbm::state_bytes(h->phys.storage, h->phys.N);
+    const size_t stride = moment_stride(bytes);
+    const bool one_copy = moment_one_copy(h, bytes);
     char *m[2] = {(char *)h->f[h->cur ^ 1], one_copy ? (char *)h->f[h->cur ^ 1] + stride : (char *)h->f[h->cur]};
     const int last = (n & 1) ? 0 : 1;   // the state that the last step reads
     const int dst = !one_copy && last == 1 ? h->cur ^ 1 : h->cur;
@@ -384,13 +391,25 @@ cudaError_t moment_run(lbm_lattice *h, long n, size_t bytes, cudaEvent_t *ev = n
     return e;
 }
 
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return false;
+}
+
 // Bytes of a moment state if the lattice's next n steps run in moment space (a
-// population copy holds one), else 0.
+// population copy holds one), else 0.  A run of even n over both copies leaves its
+// state in the other copy and moments in the one it began with, so that a caller's
+// graph of it could not be replayed; while one is captured such a run goes step by
+// step, which ends in the copy it began with.
 size_t moment_run_bytes(const lbm_lattice *h, long n)
 {
     if (!h->use_fused) return 0;
     const size_t b = lbm::moment_bytes(h->phys, n);
-    return b <= lbm::state_bytes(h->phys.storage, h->phys.N) ? b : 0;
+    if (b == 0 || b > lbm::state_bytes(h->phys.storage, h->phys.N)) return 0;
+    return n % 2 == 0 && !moment_one_copy(h, b) && capturing(h->stream) ? 0 : b;
 }
 
 }  // namespace
