@@ -181,7 +181,8 @@ k_droplet(const R *__restrict__ rho, Geo<R> g, double threshold, Origin og, doub
         }
     }
     acc[0] = (double)count;
-    for (int k = 0; k < 3; ++k) acc[1 + k] = (double)sum[k] - (double)count * og.o[k];
+    // (no cell, no share of the origin: it may be infinite)
+    for (int k = 0; k < 3; ++k) acc[1 + k] = count ? fma(-(double)count, og.o[k], (double)sum[k]) : 0.0;
     acc[6] = (double)film;
     block_reduce_store<7>(acc, partials);
 }
