@@ -11,8 +11,11 @@
 //   k_moment_out   m(t + n - 1) -> populations after its collision,
 // with 5 values per cell at tau = 1 (rho^1, rho^2, u; 40 bytes per cell and step
 // instead of 304) and 17 regularized (with sum c c f of both components; 136
-// bytes).  Every value is held and every sum taken in FP32, as in the
-// population steps; the state at the end of the call is the population state.
+// bytes).  Every value is held and every sum taken in FP32, opposite neighbours and
+// opposite populations subtracted first in x and y and in z, where they come planes
+// apart, taken relative to the column's densities (rms errors of u_z, u_x in runs of 5 to
+// 100 steps over those of population steps: 0.92 to 0.97, 0.89 to 0.94; u_z with plain sums
+// 1.04 to 1.13); the state at the end of the call is the population state.
 // us per step in calls of 10 (512^3), 20 (256^3) and 100 steps, population steps and
 // these: tau = 1 512^3 6723 / 2650, 256^3 842 / 371, 128^3 119 / 55, 96^3 52 / 33,
 // regularized 256^3 883 / 592, 384 x 512 x 512 with walls 5900 / 3190,
@@ -241,6 +244,9 @@ struct Tile {
     static constexpr int ns = KIND == COLL_EQ ? (EY == 12 ? 1656 : (EY == 16 ? 2345 : 1860)) : (EY == 12 ? 1320 : 1830);
     static constexpr int threads = kEX * EY, OY = EY - 2, RY = EY + 2;
     static constexpr int rim = 2 * kRX + 2 * EY;   // cells of a density plane beyond the threads' own
+    // density planes held: 4 leave a column's densities at q - 1, q and q + 1 in place
+    // where the 64 registers of two CTAs of 512 threads do not hold them
+    static constexpr int NR = KIND == COLL_EQ && EY == 16 ? 4 : 2;
     static_assert(rim <= threads, "");
 };
 
@@ -249,7 +255,7 @@ struct MomentSmem {
     float2 lead[kPad];                    // (threads of the ring read past the ends; what they collect is not stored)
     float2 f[T::NB][kMove][T::threads];   // moving populations of a plane
     float2 tail[kPad];
-    float2 rho[2][T::RY][kRX];            // density planes p + 1 and p + 2
+    float2 rho[T::NR][T::RY][kRX];        // density planes p + 1 and p + 2 (T::NR = 4: from p - 1 on)
 };
 
 // The direction with given components.
@@ -276,6 +282,7 @@ struct MoveSlot {
 template <int KIND>
 struct Collect {
     static constexpr int NP = RegMoments<PairF32, KIND>::n;
+    static constexpr float kShare = 7.f / 256.f;
     float2 rho, P[NP > 0 ? NP : 1];
     float jx, jy, jz;
     __device__ __forceinline__ void zero()
@@ -303,12 +310,24 @@ struct Collect {
         }
     }
     // the five populations of a group c_z = Z = +-1: the one that stays in its
-    // column, and those from the columns at -x, +x, -y, +y (moving the other way)
-    template <int Z>
-    __device__ __forceinline__ void add_group(float2 n0, float2 xp, float2 xm, float2 yp, float2 ym)
+    // column, and those from the columns at -x, +x, -y, +y (moving the other way).
+    // REF: less a share of the cell's density r one step before, which both groups of the
+    // cell know: they come two planes apart, and the z momentum would else be the
+    // difference of two sums of the populations' size.  (kShare is near w_7 and has three
+    // bits, so that the products are exact; with w_7 rounded what is left is a rounding
+    // with a sign of its own, and the density's sum swallows it: mass drifts.)  finish()
+    // adds the shares back.
+    template <int Z, bool REF>
+    __device__ __forceinline__ void add_group(float2 n0, float2 xp, float2 xm, float2 yp, float2 ym, float2 r)
     {
-        const float2 ex = vadd(xp, xm), dx = vsub(xp, xm), ey = vadd(yp, ym), dy = vsub(yp, ym);
-        const float2 s = vadd(n0, vadd(ex, ey));
+        const float2 dx = vsub(xp, xm), dy = vsub(yp, ym);
+        const float2 ex = vadd(xp, xm), ey = vadd(yp, ym);
+        float2 s = vadd(ex, ey);
+        if (REF) {
+            n0 = vfma(r, PairF32::dup(-2.f * kShare), n0);
+            s = vfma(r, PairF32::dup(-4.f * kShare), s);
+        }
+        s = vadd(n0, s);
         rho = vadd(rho, s);
         jx += dx.x + dx.y;
         jy += dy.x + dy.y;
@@ -321,6 +340,11 @@ struct Collect {
             P[4] = Z > 0 ? vadd(P[4], dx) : vsub(P[4], dx);
             P[5] = Z > 0 ? vadd(P[5], dy) : vsub(P[5], dy);
         }
+    }
+    __device__ __forceinline__ void finish(float2 r)
+    {
+        rho = vfma(r, PairF32::dup(12.f * kShare), rho);
+        if constexpr (NP > 0) P[2] = vfma(r, PairF32::dup(12.f * kShare), P[2]);
     }
 };
 
@@ -372,8 +396,8 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
     float2 r_next, h_next = make_float2(0.f, 0.f);
     {
         const unsigned o = offset(first - 1);
-        sm.rho[(first - 1) & 1][ey + 1][ex + 1] = present(first - 1, in.rho[o + col]);
-        if (rim) sm.rho[(first - 1) & 1][ry][rx] = present(first - 1, in.rho[o + rcol]);
+        sm.rho[(first - 1) & (T::NR - 1)][ey + 1][ex + 1] = present(first - 1, in.rho[o + col]);
+        if (rim) sm.rho[(first - 1) & (T::NR - 1)][ry][rx] = present(first - 1, in.rho[o + rcol]);
         const unsigned o1 = offset(first);
         r_next = in.rho[o1 + col];
         if (rim) h_next = in.rho[o1 + rcol];
@@ -382,9 +406,12 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
     float uz = 0.f;
     unsigned lw = 0, lw_p = 0;   // link words of the column at plane q + 1, q - 1
     RegMoments<PairF32, KIND> mo;
-    float2 S[3], lo[3], r_own = make_float2(0.f, 0.f);   // sums of plane p so far, and what plane p adds to p + 1's
-#pragma unroll
-    for (int d = 0; d < 3; ++d) S[d] = lo[d] = make_float2(0.f, 0.f);
+    // x and y sums of plane q so far, what it adds to q + 1's, its Laplacian's two
+    // predecessors, and the column's densities at q and q - 1
+    const float2 zero = make_float2(0.f, 0.f);
+    constexpr bool keep = T::NR == 2;
+    auto own = [&](int k) { return sm.rho[k & (T::NR - 1)][ey + 1][ex + 1]; };
+    float2 S[2] = {zero, zero}, lo[2] = {zero, zero}, L0 = zero, L1 = zero, r_own = zero, r_old = zero;
     Collect<KIND> c0, c1;   // planes p - 1 and p
     c0.zero();
     c1.zero();
@@ -395,9 +422,11 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
         // ---- a. plane q + 1's densities are in place: they complete plane q's
         //      sums and start plane q + 1's and q + 2's
         const bool collides = q >= first && !(WALLZ && (q < 0 || q >= nz));
-        // (density plane q + 2 into its slot; its last readers passed two barriers ago)
-        sm.rho[(q + 2) & 1][ey + 1][ex + 1] = present(q + 2, r_next);
-        if (rim) sm.rho[(q + 2) & 1][ry][rx] = present(q + 2, h_next);
+        // (density plane q + 2 into its slot, where plane q, of four held plane q - 2, was: the
+        // neighbours read it before the last iteration's barrier, so that their reads have to
+        // stay in section a; a thread's own() reads are of cells that it writes itself)
+        sm.rho[(q + 2) & (T::NR - 1)][ey + 1][ex + 1] = present(q + 2, r_next);
+        if (rim) sm.rho[(q + 2) & (T::NR - 1)][ry][rx] = present(q + 2, h_next);
         // loads for the next iteration
         const float2 uxy_c = uxy;
         const float uz_c = uz;
@@ -415,29 +444,31 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
         }
         float2 So[3], rc;
         {
-            const float2(*R)[kRX] = &sm.rho[(q + 1) & 1][ey];   // rows ey, ey + 1, ey + 2: y - 1, y, y + 1
+            const float2(*R)[kRX] = &sm.rho[(q + 1) & (T::NR - 1)][ey];   // rows ey, ey + 1, ey + 2: y - 1, y, y + 1
             const float2 xp = R[1][ex + 2], xm = R[1][ex], yp = R[2][ex + 1], ym = R[0][ex + 1];
             rc = R[1][ex + 1];
             const float2 dx = vsub(xp, xm), dy = vsub(yp, ym);
             const float2 a = vsub(R[2][ex + 2], R[0][ex]), b = vsub(R[0][ex + 2], R[2][ex]);   // (1,1), (1,-1)
-            const float2 Z = vfma(w1, rc, vmul(w2, vadd(vadd(xp, xm), vadd(yp, ym))));
+            // S_z = w_7 (6 (rho(q + 1) - rho(q - 1)) + L(q + 1) - L(q - 1)) with L the sum of the four
+            // neighbours less 4 rho: differences first, as in x and y (x_- - rho = x_+ - rho - dx)
+            const float2 L = vfma(vadd(vsub(xp, rc), vsub(yp, rc)), make_float2(2.f, 2.f), vsub(zero, vadd(dx, dy)));
             const float2 lx = vmul(w2, dx), ly = vmul(w2, dy);
             // plane q: this plane lies above it
             So[0] = vswap(vadd(S[0], lx));
             So[1] = vswap(vadd(S[1], ly));
-            So[2] = vswap(vadd(S[2], Z));
+            So[2] = vswap(vmul(w2, vfma(vsub(rc, keep ? r_old : own(q - 1)), make_float2(6.f, 6.f), vsub(L, L0))));
             // plane q + 1: its own plane
             S[0] = vadd(lo[0], vfma(w1, dx, vmul(w2, vadd(a, b))));
             S[1] = vadd(lo[1], vfma(w1, dy, vmul(w2, vsub(a, b))));
-            S[2] = lo[2];
             // plane q + 2: this plane lies below it
             lo[0] = lx;
             lo[1] = ly;
-            lo[2] = vsub(make_float2(0.f, 0.f), Z);
+            L0 = L1;
+            L1 = L;
         }
         float2 *const F = &sm.f[T::NB == 2 ? (q & 1) : 0][0][tid];
-        const float2 r = r_own;   // density of plane q at this column
-        r_own = rc;
+        const float2 r = keep ? r_own : own(q);   // density of plane q at this column
+        if (keep) r_own = rc;
         float2 f0, fu, fd;        // populations that stay in the column: c_z = 0, +1, -1
         if (collides) {
             auto get = [](int) { return make_float2(0.f, 0.f); };
@@ -457,6 +488,7 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
         }
         __syncthreads();
         // ---- b. what streams into this column
+        const float2 r_dn = keep ? r_old : own(q - 1);
         Collect<KIND> c2;         // plane q + 1
         c2.zero();
         if (collides) {
@@ -469,13 +501,17 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
                 c1.rho = vadd(c1.rho, f0);
                 c1.add_plane(xp, xm, yp, ym, a, b, c, d);
             }
-            c2.template add_group<1>(fu, LBM_FROM(1, 0, 1), LBM_FROM(-1, 0, 1), LBM_FROM(0, 1, 1), LBM_FROM(0, -1, 1));
-            c0.template add_group<-1>(fd, LBM_FROM(1, 0, -1), LBM_FROM(-1, 0, -1), LBM_FROM(0, 1, -1), LBM_FROM(0, -1, -1));
+            c2.template add_group<1, true>(fu, LBM_FROM(1, 0, 1), LBM_FROM(-1, 0, 1), LBM_FROM(0, 1, 1), LBM_FROM(0, -1, 1),
+                                           keep ? r_own : own(q + 1));
+            c0.template add_group<-1, true>(fd, LBM_FROM(1, 0, -1), LBM_FROM(-1, 0, -1), LBM_FROM(0, 1, -1),
+                                            LBM_FROM(0, -1, -1), r_dn);
             if (WALLZ) {   // half-way bounce-back: the cell's own populations come back reversed
                 if (q == 0)
-                    c1.template add_group<1>(fd, LBM_OWN(-1, 0, -1), LBM_OWN(1, 0, -1), LBM_OWN(0, -1, -1), LBM_OWN(0, 1, -1));
+                    c1.template add_group<1, true>(fd, LBM_OWN(-1, 0, -1), LBM_OWN(1, 0, -1), LBM_OWN(0, -1, -1),
+                                                   LBM_OWN(0, 1, -1), r);
                 if (q == nz - 1)
-                    c1.template add_group<-1>(fu, LBM_OWN(-1, 0, 1), LBM_OWN(1, 0, 1), LBM_OWN(0, -1, 1), LBM_OWN(0, 1, 1));
+                    c1.template add_group<-1, true>(fu, LBM_OWN(-1, 0, 1), LBM_OWN(1, 0, 1), LBM_OWN(0, -1, 1),
+                                                    LBM_OWN(0, 1, 1), r);
             }
             if (MASK && lw_c > 1u) {   // links into solid sites
 #define LBM_BACK(X, Y, Z) (((lw_c >> dir_of(X, Y, Z)) & 1u) ? LBM_OWN(-(X), -(Y), -(Z)) : make_float2(0.f, 0.f))
@@ -484,10 +520,11 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
                     const float2 a = LBM_BACK(1, 1, 0), b = LBM_BACK(-1, -1, 0), c = LBM_BACK(1, -1, 0), d = LBM_BACK(-1, 1, 0);
                     c1.add_plane(xp, xm, yp, ym, a, b, c, d);
                 }
-                c1.template add_group<1>(((lw_c >> kUp) & 1u) ? fd : make_float2(0.f, 0.f), LBM_BACK(1, 0, 1), LBM_BACK(-1, 0, 1),
-                                         LBM_BACK(0, 1, 1), LBM_BACK(0, -1, 1));
-                c1.template add_group<-1>(((lw_c >> kDown) & 1u) ? fu : make_float2(0.f, 0.f), LBM_BACK(1, 0, -1),
-                                          LBM_BACK(-1, 0, -1), LBM_BACK(0, 1, -1), LBM_BACK(0, -1, -1));
+                // (what takes the place of the zeros out of the solid sites, whose w_i t is off already)
+                c1.template add_group<1, false>(((lw_c >> kUp) & 1u) ? fd : make_float2(0.f, 0.f), LBM_BACK(1, 0, 1),
+                                                LBM_BACK(-1, 0, 1), LBM_BACK(0, 1, 1), LBM_BACK(0, -1, 1), zero);
+                c1.template add_group<-1, false>(((lw_c >> kDown) & 1u) ? fu : make_float2(0.f, 0.f), LBM_BACK(1, 0, -1),
+                                                 LBM_BACK(-1, 0, -1), LBM_BACK(0, 1, -1), LBM_BACK(0, -1, -1), zero);
 #undef LBM_BACK
             }
 #undef LBM_FROM
@@ -498,6 +535,7 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
             if (MASK && (lw_p & 1u)) {
                 out.put_solid(cell, rs, N32);
             } else {
+                c0.finish(r_dn);
                 const float inv = 1.0f / (c0.rho.x + c0.rho.y);
                 out.rho[cell] = c0.rho;
                 out.uxy[cell] = make_float2(c0.jx * inv, c0.jy * inv);
@@ -507,6 +545,7 @@ k_step_moment(const MomentState<KIND> in, MomentState<KIND> out, Phys<float> p, 
             }
         }
         lw_p = lw_c;
+        if (keep) r_old = r;
         c0 = c1;
         c1 = c2;
         if (T::NB == 1) __syncthreads();   // (two copies: a copy's readers passed the next plane's barrier)
