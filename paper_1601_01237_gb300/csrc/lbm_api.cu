@@ -32,6 +32,7 @@ struct lbm_lattice {
     double *partials_h;  // reduction partials (pinned host)
     long steps;
     int use_fused;
+    lbm::MomentPlan mplan;   // of runs of steps in moment space (choose_paths)
     int init_at_rest;    // current run started from lbm_init_fields with u = NULL
     // recording for the reverse pass
     void *ckpt;          // checkpoint store (rec_nck raw states)
@@ -141,6 +142,18 @@ lbm_status lbm_lattice_dirs(int c[19][3], double w[19])
     return LBM_OK;
 }
 
+namespace {
+
+// How the lattice steps, from its physics and mask, on the current device.
+void choose_paths(lbm_lattice *h)
+{
+    h->use_fused = env_flag("LBM_FUSED", 1) && lbm::fused_supported(h->phys);
+    h->mplan = h->use_fused ? lbm::moment_plan(h->phys) : lbm::MomentPlan();
+    if (h->mplan.bytes > lbm::state_bytes(h->phys.storage, h->phys.N)) h->mplan.bytes = 0;   // no copy holds a state
+}
+
+}  // namespace
+
 lbm_status lbm_create(const lbm_params *pp, lbm_lattice **out)
 {
     if (!pp || !out) return fail(LBM_EINVAL, "lbm_create: NULL argument");
@@ -195,7 +208,6 @@ lbm_status lbm_create(const lbm_params *pp, lbm_lattice **out)
     ph.rho_s[0] = p.rho_s[0]; ph.rho_s[1] = p.rho_s[1];
     ph.rho0 = p.rho0_dev;
     ph.ref_off = (long long)lbm::ref_offset(p.storage, N);
-    h->use_fused = env_flag("LBM_FUSED", 1) && lbm::fused_supported(ph);
     h->use_graphs = env_flag("LBM_GRAPHS", 1);
 
     cudaError_t e = cudaGetDevice(&h->device);
@@ -231,6 +243,7 @@ lbm_status lbm_create(const lbm_params *pp, lbm_lattice **out)
     }
     h->cur = 0;
     h->steps = 0;
+    choose_paths(h);
     *out = h;
     return LBM_OK;
 }
@@ -379,7 +392,7 @@ cudaError_t moment_run(lbm_lattice *h, long n, size_t bytes, cudaEvent_t *ev = n
     cudaError_t e = lbm::launch_moment_in(h->phys, h->f[h->cur], m[0], h->stream);
     if (ev) cudaEventRecord(*ev++, h->stream);
     for (long t = 1; t < n && e == cudaSuccess; ++t) {
-        e = lbm::launch_moment_step(h->phys, m[(t & 1) ^ 1], m[t & 1], h->stream);
+        e = lbm::launch_moment_step(h->phys, h->mplan, m[(t & 1) ^ 1], m[t & 1], h->stream);
         if (ev) cudaEventRecord(*ev++, h->stream);
     }
     if (e == cudaSuccess) e = lbm::launch_moment_out(h->phys, m[last], h->f[dst], h->stream);
@@ -399,16 +412,14 @@ bool capturing(cudaStream_t s)
     return false;
 }
 
-// Bytes of a moment state if the lattice's next n steps run in moment space (a
-// population copy holds one), else 0.  A run of even n over both copies leaves its
+// Bytes of a moment state if the lattice's next n steps run in moment space, else 0.  A run of even n over both copies leaves its
 // state in the other copy and moments in the one it began with, so that a caller's
 // graph of it could not be replayed; while one is captured such a run goes step by
 // step, which ends in the copy it began with.
 size_t moment_run_bytes(const lbm_lattice *h, long n)
 {
-    if (!h->use_fused) return 0;
-    const size_t b = lbm::moment_bytes(h->phys, n);
-    if (b == 0 || b > lbm::state_bytes(h->phys.storage, h->phys.N)) return 0;
+    if (!h->mplan.pays(n)) return 0;
+    const size_t b = h->mplan.bytes;
     return n % 2 == 0 && !moment_one_copy(h, b) && capturing(h->stream) ? 0 : b;
 }
 
@@ -635,10 +646,8 @@ lbm_status lbm_set_solid(lbm_lattice *h, const unsigned char *solid, int on_devi
     h->rec_steps = 0;
     free_workspace(h);
     free_mask(h);
-    if (!solid) {
-        h->use_fused = env_flag("LBM_FUSED", 1) && lbm::fused_supported(h->phys);
-        return LBM_OK;
-    }
+    choose_paths(h);
+    if (!solid) return LBM_OK;
     const size_t N = (size_t)h->phys.N;
     CK(cudaMalloc((void **)&h->solid, N), "lbm_set_solid: mask");
     CK(cudaMalloc((void **)&h->links, N * sizeof(unsigned)), "lbm_set_solid: link flags");
@@ -647,7 +656,7 @@ lbm_status lbm_set_solid(lbm_lattice *h, const unsigned char *solid, int on_devi
     CK(lbm::launch_link_flags(h->phys, h->solid, h->links, h->stream), "lbm_set_solid: link flags");
     h->phys.solid = h->solid;
     h->phys.links = h->links;
-    h->use_fused = env_flag("LBM_FUSED", 1) && lbm::fused_supported(h->phys);
+    choose_paths(h);
     {
         // wall densities (fused step) and the boundary lists of the mirror
         // model (fused step and reverse pass): count, then list
@@ -683,6 +692,7 @@ lbm_status lbm_set_solid(lbm_lattice *h, const unsigned char *solid, int on_devi
         cudaFree(cnt);
         if (e != cudaSuccess) {
             free_mask(h);
+            choose_paths(h);
             return cuda_fail(e, "lbm_set_solid: boundary lists");
         }
         h->phys.wall_rho = h->wall_rho;

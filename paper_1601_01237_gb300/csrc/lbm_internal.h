@@ -70,18 +70,29 @@ bool fused_supported(const HostPhys &p);
 // whether launch_step_fused takes it.
 cudaError_t launch_step_box(const HostPhys &p, const void *f_in, void *f_out, cudaStream_t s, void *s_out = nullptr);
 bool use_box(const HostPhys &p);
-// Runs of n >= 2 steps in moment space (lbm_moment.cu): the bytes of one moment
-// state of the lattice, 0 where its next n steps do not run that way; populations to
-// moments, a step on moments, and the last step from moments to populations.
-size_t moment_bytes(const HostPhys &h, long n);
+// Runs of n >= 2 steps in moment space (lbm_moment.cu): populations to moments,
+// steps on moments, and the last step from moments to populations.  The plan of a
+// lattice (on the current device; anew when its mask changes) holds the tile of the
+// steps and the estimated times, us, of a step on moments, of the two ends together and of
+// a step on populations.
+struct MomentPlan {
+    size_t bytes;         // of one moment state; 0: the lattice takes no such steps
+    int rows, ntx, lz;    // tile: thread rows, tiles along x, planes per CTA
+    long long cols;       // tile columns
+    double step_us, ends_us, fused_us;
+    bool pays(long n) const { return bytes && n >= 2 && ends_us + (double)(n - 1) * step_us < (double)n * fused_us; }
+};
+MomentPlan moment_plan(const HostPhys &h);
 cudaError_t launch_moment_in(const HostPhys &h, const void *f, void *m, cudaStream_t s);
-cudaError_t launch_moment_step(const HostPhys &h, const void *m_in, void *m_out, cudaStream_t s);
+cudaError_t launch_moment_step(const HostPhys &h, const MomentPlan &q, const void *m_in, void *m_out, cudaStream_t s);
 cudaError_t launch_moment_out(const HostPhys &h, const void *m, void *f, cudaStream_t s);
 
 // Planes per CTA of the fused step for a lattice of cols = ceil(nx/32) *
 // ceil(ny/8) tile columns and nz planes on a device with sms SMs.
 constexpr int kPlanesMax = 64, kPlanesMin = 8;
 int fused_planes(long long cols, int nz, int sms);
+// Estimated time of a marching step (launch_step_fused without the box step), us.
+double marching_us(const HostPhys &p);
 
 // Mask set-up for the fused step: wall_rho = rho_s at every solid site, and
 // the counts (lists == nullptr) or the lists themselves of the boundary cells

@@ -230,18 +230,16 @@ constexpr int kMove = 16;
 static_assert(kPad >= kEX + 1, "");
 // Tiles of EY thread rows.  NB = 2 copies of the moving populations leave one
 // barrier per plane instead of two, where shared memory holds them.  ns: measured
-// time per plane of an SM full of such CTAs, which is 69 to 77 ns per row at tau = 1
-// and 110 to 114 ns regularized whatever the tile, so that the tile with the fewest
-// rows of work (rings, ragged edges and the last wave counted) is taken:
-// us per step at tau = 1, tiles 12 / 16 / 24: 512^3 2802 / 2759 / 2892, 256^3 374 /
-// 386 / 386, 128^3 66 / 66 / 57, 96^3 35 / 37 / 35; regularized 12 / 16: 256^3 594 /
-// 608, 131 x 150 x 173 129 / 135, 384 x 512 x 512 with walls 3335 / 3182.  (One tile
-// of 16 rows and two barriers: 2810, 392, 68, 37; 599, 134, 3473.  Regularized tiles
-// of 18 or more rows spill: 1028 us at 256^3.)
+// time per plane of an SM full of such CTAs, so that the tile with the least work
+// (rings, ragged edges and the last wave counted) is taken.  us per step at tau = 1,
+// tiles 12 / 16 / 24: 512^3 3323 / 3252 / 3342, 256^3 414 / 422 / 417, 128^3 67 / 67 / 57,
+// 96^3 33 / 36 / 34; regularized 12 / 16: 256^3 651 / 649, 131 x 150 x 173 135 / 141,
+// 384 x 512 x 512 with walls 3754 / 3724.  Under a mask tiles of 16 rows spill at tau = 1
+// (256^3 835 us, the others 454 and 464), and regularized ones of 18 or more rows do.
 template <int KIND, int EY_>
 struct Tile {
     static constexpr int EY = EY_, ctas = KIND == COLL_EQ && EY <= 16 ? 2 : 1, NB = KIND == COLL_EQ && EY == 16 ? 1 : 2;
-    static constexpr int ns = KIND == COLL_EQ ? (EY == 12 ? 1656 : (EY == 16 ? 2345 : 1860)) : (EY == 12 ? 1320 : 1830);
+    static constexpr int ns = KIND == COLL_EQ ? (EY == 12 ? 1870 : (EY == 16 ? 2580 : 2060)) : (EY == 12 ? 1460 : 2005);
     static constexpr int threads = kEX * EY, OY = EY - 2, RY = EY + 2;
     static constexpr int rim = 2 * kRX + 2 * EY;   // cells of a density plane beyond the threads' own
     // density planes held: 4 leave a column's densities at q - 1, q and q + 1 in place
@@ -567,42 +565,48 @@ Phys<float> make_phys_m(const HostPhys &h)
     return p;
 }
 
-// Planes per CTA: equal chunks, the fewest waves x (planes + 4) (the collisions
-// beyond the two ends of a chunk and the density planes before it); cost: that
-// number.
-int moment_planes(long long cols, int nz, long long slots, long long *cost)
+// Planes per CTA: equal chunks of at most 128, the fewest waves x (planes + 4) (the
+// collisions beyond the two ends of a chunk and the density planes before it); waves:
+// their number.
+int moment_planes(long long cols, int nz, long long slots, long long *waves)
 {
     int best = nz;
-    *cost = -1;
-    for (int nch = (nz + 127) / 128; nch <= nz; ++nch) {
-        const int lz = (nz + nch - 1) / nch;
+    long long least = -1;
+    for (int most = nz < 128 ? nz : 128; most >= 1; --most) {   // (by length: few of them however tall the lattice)
+        const int nch = (nz + most - 1) / most, lz = (nz + nch - 1) / nch;
         if (lz < 4 && nch > 1) break;
-        const long long ctas = cols * ((nz + lz - 1) / lz), c = ((ctas + slots - 1) / slots) * (lz + 4);
-        if (*cost < 0 || c < *cost) { *cost = c; best = lz; }
+        const long long w = (cols * ((nz + lz - 1) / lz) + slots - 1) / slots;
+        if (least < 0 || w * (lz + 4) < least) { least = w * (lz + 4); best = lz; *waves = w; }
     }
     return best;
 }
 
-struct Plan {
-    int ntx, lz;
-    long long cols, ns;   // tile columns, estimated time
-};
+// Takes the tile of EY rows into the plan if it is the cheapest so far (cost: that of the others).
 template <int KIND, int EY>
-Plan plan_of(const HostPhys &h)
+void plan_tile(const HostPhys &h, MomentPlan &q, double &cost)
 {
     using T = Tile<KIND, EY>;
-    Plan q;
-    q.ntx = (h.nx + kOX - 1) / kOX;
-    q.cols = (long long)q.ntx * ((h.ny + T::OY - 1) / T::OY);
-    q.lz = moment_planes(q.cols, h.nz, (long long)T::ctas * current_device_sms(), &q.ns);
-    q.ns *= T::ns;
-    return q;
+    const int ntx = (h.nx + kOX - 1) / kOX;
+    const long long cols = (long long)ntx * ((h.ny + T::OY - 1) / T::OY);
+    long long waves = 1;
+    const int lz = moment_planes(cols, h.nz, (long long)T::ctas * current_device_sms(), &waves);
+    const double c = (double)waves * (lz + 4) * T::ns;
+    if (q.rows && !(c < cost)) return;
+    cost = c;
+    q.rows = EY;
+    q.ntx = ntx;
+    q.lz = lz;
+    q.cols = cols;
+    // (the planes beyond a chunk that do not collide cost less: all four count near four
+    // only regularized; at z walls there is no plane beyond)
+    const double planes = lz + (KIND == COLL_EQ ? 3.3 : 4.2) - (h.wall_z && lz == h.nz ? 1.0 : 0.0);
+    q.step_us = 1e-3 * (double)waves * planes * T::ns;
 }
 
 constexpr int kMaxAttrDevices = 64;
 
 template <int KIND, int FORCE, int EY, bool WALLZ, bool MASK>
-cudaError_t launch_tile(const HostPhys &h, const Plan &q, const void *in, void *out, cudaStream_t s)
+cudaError_t launch_tile(const HostPhys &h, const MomentPlan &q, const void *in, void *out, cudaStream_t s)
 {
     using T = Tile<KIND, EY>;
     static std::atomic<int> attr_set[kMaxAttrDevices];
@@ -636,19 +640,38 @@ cudaError_t launch_tile(const HostPhys &h, const Plan &q, const void *in, void *
 }
 
 template <int KIND, bool WALLZ, bool MASK>
-cudaError_t launch_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
+cudaError_t launch_step(const HostPhys &h, const MomentPlan &q, const void *in, void *out, cudaStream_t s)
 {
-    constexpr int E = FORCE_EDM;
-    const Plan a = plan_of<KIND, 12>(h);
-    // Guo's forcing takes the tile of 12 rows (it needs the registers of it)
-    if (h.forcing == FORCE_GUO) return launch_tile<KIND, FORCE_GUO, 12, WALLZ, MASK>(h, a, in, out, s);
-    const Plan b = plan_of<KIND, 16>(h);
+    if (h.forcing == FORCE_GUO) return launch_tile<KIND, FORCE_GUO, 12, WALLZ, MASK>(h, q, in, out, s);
+    if (q.rows == 12) return launch_tile<KIND, FORCE_EDM, 12, WALLZ, MASK>(h, q, in, out, s);
     if constexpr (KIND == COLL_EQ) {
-        const Plan c = plan_of<KIND, 24>(h);
-        if (c.ns < a.ns && c.ns < b.ns) return launch_tile<KIND, E, 24, WALLZ, MASK>(h, c, in, out, s);
+        if (q.rows == 24) return launch_tile<KIND, FORCE_EDM, 24, WALLZ, MASK>(h, q, in, out, s);
     }
-    return a.ns < b.ns ? launch_tile<KIND, E, 12, WALLZ, MASK>(h, a, in, out, s)
-                       : launch_tile<KIND, E, 16, WALLZ, MASK>(h, b, in, out, s);
+    if constexpr (KIND != COLL_EQ || !MASK) {
+        if (q.rows == 16) return launch_tile<KIND, FORCE_EDM, 16, WALLZ, MASK>(h, q, in, out, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <int KIND>
+MomentPlan plan_kind(const HostPhys &h)
+{
+    MomentPlan q = {};
+    double cost = 0;
+    plan_tile<KIND, 12>(h, q, cost);
+    if (h.forcing == FORCE_GUO) {   // (it needs the registers of that tile: 256^3 467 us, exact difference 414)
+        q.step_us *= 1.15;
+    } else {
+        if (KIND != COLL_EQ || !h.links) plan_tile<KIND, 16>(h, q, cost);
+        if constexpr (KIND == COLL_EQ) plan_tile<KIND, 24>(h, q, cost);
+    }
+    q.bytes = sizeof(float) * moment_floats<KIND>() * (size_t)h.N;
+    // the two ends are bound by their bytes: ps per cell (256^3: 410 + 448 us, 528 + 559;
+    // 16 bits 263 + 354, 366 + 464)
+    const bool f32 = h.storage == ST_F32;
+    q.ends_us = 4.0 + 1e-6 * (double)h.N * (KIND == COLL_EQ ? (f32 ? 52 : 38) : (f32 ? 66 : 51));
+    q.fused_us = marching_us(h);
+    return q;
 }
 
 bool tau_one(const HostPhys &h) { return (float)(1.0 / h.tau[0]) == 1.0f && (float)(1.0 / h.tau[1]) == 1.0f; }
@@ -657,25 +680,24 @@ inline unsigned grid_m(long long N) { return (unsigned)((N + kThreadsM - 1) / kT
 
 }  // namespace
 
-size_t moment_bytes(const HostPhys &h, long n)
+// A run of n steps takes the two ends and n - 1 steps on moments, where that is estimated
+// to be less than n steps on populations: lattices of a few planes, or much narrower than
+// a tile, collide too many cells twice.  us per step in runs of 20, populations / moments:
+// FP32 regularized 1 x 2100^2 395 / 640, 2 x 2100^2 631 / 829, 6 x 2100^2 1668 / 1437,
+// 20000 x 32 x 32 1029 / 1464, 256^3 878 / 653; tau = 1 1 x 2100^2 374 / 361; FP16 deviations tau = 1
+// 1 x 2100^2 275 / 358, 6 x 2100^2 1020 / 797, regularized 6 x 2100^2 1267 / 1416, 256^3 696 / 640
+// (two steps there 696 / 728).
+MomentPlan moment_plan(const HostPhys &h)
 {
-    // Short regularized runs of large lattices under Guo's forcing lose to the cost of
-    // the two ends (us at 256^3, step by step / in moment space: FP32 two 1771 / 1790,
-    // three 2654 / 2475, FP16 deviations three 2155 / 2205, ten 7178 / 7009); the others
-    // gain from two on (two steps, exact difference: FP16 deviations 1370 / 1345, FP32
-    // 1768 / 1657).
-    const int least = tau_one(h) || h.forcing != FORCE_GUO ? 2 : (h.storage == ST_F32 ? 3 : 6);
-    if (n < least) return 0;
+    const MomentPlan none = {};
     // The relative formats stay step by step: they hand out FP32 reference densities,
     // which carry every step's rounding to 16 bits.
-    if (h.storage != ST_F32 && h.storage != ST_F16_DEV && h.storage != ST_BF16_DEV) return 0;
-    if (!fused_supported(h) || use_box(h)) return 0;
+    if (h.storage != ST_F32 && h.storage != ST_F16_DEV && h.storage != ST_BF16_DEV) return none;
+    if (!tau_one(h) && h.collision != LBM_REGULARIZED) return none;
+    if (!fused_supported(h) || use_box(h)) return none;
     const long long cols = (long long)((h.nx + kOX - 1) / kOX) * ((h.ny + Tile<COLL_REG, 12>::OY - 1) / Tile<COLL_REG, 12>::OY);
-    if (cols >= (1LL << 31) || h.nz > 4 * 65535) return 0;   // grid limits
-    const size_t N = (size_t)h.N;
-    if (tau_one(h)) return sizeof(float) * moment_floats<COLL_EQ>() * N;
-    if (h.collision == LBM_REGULARIZED) return sizeof(float) * moment_floats<COLL_REG>() * N;
-    return 0;
+    if (cols >= (1LL << 31) || h.nz > 4 * 65535) return none;   // grid limits
+    return tau_one(h) ? plan_kind<COLL_EQ>(h) : plan_kind<COLL_REG>(h);
 }
 
 namespace {
@@ -698,11 +720,11 @@ cudaError_t moment_in_t(const HostPhys &h, const void *f, void *m, cudaStream_t 
 }
 
 template <int KIND>
-cudaError_t moment_step_t(const HostPhys &h, const void *in, void *out, cudaStream_t s)
+cudaError_t moment_step_t(const HostPhys &h, const MomentPlan &q, const void *in, void *out, cudaStream_t s)
 {
-    const cudaError_t e = h.wall_z ? launch_step<KIND, true, false>(h, in, out, s)
-                          : h.links ? launch_step<KIND, false, true>(h, in, out, s)
-                                    : launch_step<KIND, false, false>(h, in, out, s);
+    const cudaError_t e = h.wall_z ? launch_step<KIND, true, false>(h, q, in, out, s)
+                          : h.links ? launch_step<KIND, false, true>(h, q, in, out, s)
+                                    : launch_step<KIND, false, false>(h, q, in, out, s);
     return e == cudaSuccess ? moment_walls<KIND>(h, out, s) : e;
 }
 
@@ -740,9 +762,9 @@ cudaError_t launch_moment_in(const HostPhys &h, const void *f, void *m, cudaStre
     }
 }
 
-cudaError_t launch_moment_step(const HostPhys &h, const void *in, void *out, cudaStream_t s)
+cudaError_t launch_moment_step(const HostPhys &h, const MomentPlan &q, const void *in, void *out, cudaStream_t s)
 {
-    return tau_one(h) ? moment_step_t<COLL_EQ>(h, in, out, s) : moment_step_t<COLL_REG>(h, in, out, s);
+    return tau_one(h) ? moment_step_t<COLL_EQ>(h, q, in, out, s) : moment_step_t<COLL_REG>(h, q, in, out, s);
 }
 
 cudaError_t launch_moment_out(const HostPhys &h, const void *m, void *f, cudaStream_t s)
