@@ -5,6 +5,6 @@ namespace lbm {
 namespace adj {
 template cudaError_t adj_step_t<ST_F32>(const HostPhys &, const void *, const void *, int,
                                        const void *, const void *, void *, void *, void *, double *,
-                                       cudaStream_t);
+                                       cudaStream_t, bool);
 }  // namespace adj
 }  // namespace lbm

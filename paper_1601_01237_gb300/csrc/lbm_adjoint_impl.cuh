@@ -28,7 +28,8 @@
 // with one base per component and one vector jb for both: lambda_loc is then held
 // as these 5 values per cell instead of 38 (jb as 4-vectors [N], behind them
 // base[2][N]), and k_adj_D adds base to D, so that the next reverse step gathers
-//   mu_i(y) = D_a(y + c_i) + c_i . jb(y + c_i).
+//   mu_i(y) = D_a(y + c_i) + c_i . jb(y + c_i);
+// after the last reverse step the two stay apart, and k_adj_rho0 adds them in FP64.
 // us per reverse step with its replay, 38 values and 5: 96^3 184 / 150, 128^3 472 / 334,
 // masked 96^3 214 / 176; what is left waits on the 19 populations and 19 cached
 // sensitivities that each lane gathers.
@@ -768,12 +769,12 @@ k_adj_seed_eq(const G *__restrict__ g1, const G *__restrict__ g2, float *__restr
     reinterpret_cast<float4 *>(lam)[c] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// dL/drho^a_0 = sum_i w_i lambda^0_i = sum_i w_i lambda_loc^0_i + D^0_a (sum_i w_i = 1;
-// EQ instances, lam null: D has base, and sum_i w_i c_i = 0).
+// dL/drho^a_0 = sum_i w_i lambda^0_i = sum_i w_i lambda_loc^0_i + D^0_a (sum_i w_i = 1);
+// EQ instances: base in the place of the sum (sum_i w_i c_i = 0), lam null.
 template <class R>
 __global__ void __launch_bounds__(kThreadsA)
-k_adj_rho0(const R *__restrict__ lam, const R *__restrict__ D, double *__restrict__ g1, double *__restrict__ g2,
-           long long N, const unsigned char *__restrict__ solid)
+k_adj_rho0(const R *__restrict__ lam, const R *__restrict__ base, const R *__restrict__ D, double *__restrict__ g1,
+           double *__restrict__ g2, long long N, const unsigned char *__restrict__ solid)
 {
     const long long c = (long long)blockIdx.x * kThreadsA + threadIdx.x;
     if (c >= N) return;
@@ -782,7 +783,7 @@ k_adj_rho0(const R *__restrict__ lam, const R *__restrict__ D, double *__restric
         if (g2) g2[c] = 0.0;
         return;
     }
-    double s1 = 0, s2 = 0;
+    double s1 = base ? (double)base[c] : 0.0, s2 = base ? (double)base[N + c] : 0.0;
 #pragma unroll
     for (int i = 0; lam && i < Q; ++i) {
         s1 += wd(i) * (double)lam[(long long)i * N + c];
@@ -842,7 +843,8 @@ namespace adj {
 
 template <int S>
 cudaError_t adj_step_t(const HostPhys &h, const void *f, const void *rho, int rho_is_sums, const void *lam_next,
-                       const void *Dn, void *lam_loc, void *a, void *Dout, double *partials, cudaStream_t s)
+                       const void *Dn, void *lam_loc, void *a, void *Dout, double *partials, cudaStream_t s,
+                       bool last)
 {
     using T = typename Store<S>::T;
     using R = typename Store<S>::R;
@@ -879,7 +881,7 @@ cudaError_t adj_step_t(const HostPhys &h, const void *f, const void *rho, int rh
 #undef LBM_ADJ_REG
 #undef LBM_ADJ
 #undef LBM_ADJ_I
-    cudaError_t e = launch_adj_D<R>(h, (const R *)a, eq ? (const R *)lam_loc + 4 * h.N : nullptr, (R *)Dout, p, s);
+    cudaError_t e = launch_adj_D<R>(h, (const R *)a, eq && !last ? (const R *)lam_loc + 4 * h.N : nullptr, (R *)Dout, p, s);
     if (e == cudaSuccess && h.links && h.wall_mirror && h.n_bfluid > 0) {
         k_adj_D_wall<R><<<gridA(h.n_bfluid), kThreadsA, 0, s>>>((R *)Dout, h.solid, p, h.bfluid, h.n_bfluid);
         e = cudaGetLastError();

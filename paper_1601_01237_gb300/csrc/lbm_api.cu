@@ -908,8 +908,9 @@ lbm_status lbm_adjoint(lbm_lattice *h, const double *dL_drho1, const double *dL_
     // (la, da).
     // The segment's first state is read in place from the checkpoint store
     // (first); its later states go to the segment buffer (state t at slot t - 1).
-    auto enqueue_segment = [&](cudaStream_t st, long len, const void *first, void *la, void *lb, void *da,
-                               void *db) -> cudaError_t {
+    // last: the run's first segment, which the reverse pass ends with.
+    auto enqueue_segment = [&](cudaStream_t st, long len, const void *first, void *la, void *lb, void *da, void *db,
+                               bool last) -> cudaError_t {
         auto state = [&](long t) -> void * {
             return t == 0 ? const_cast<void *>(first) : (void *)((char *)seg + sb * (size_t)(t - 1));
         };
@@ -929,7 +930,7 @@ lbm_status lbm_adjoint(lbm_lattice *h, const double *dL_drho1, const double *dL_
             const void *fn = state(t);
             const void *rn = (char *)rseg + rstride * (size_t)t;
             // step t reads (la, da) and writes (lb, db)
-            er = lbm::launch_adjoint_step(h->phys, fn, rn, use_fused ? 1 : 0, la, da, lb, abuf, db, part, st);
+            er = lbm::launch_adjoint_step(h->phys, fn, rn, use_fused ? 1 : 0, la, da, lb, abuf, db, part, st, last && t == 0);
             std::swap(la, lb);
             std::swap(da, db);
         }
@@ -946,12 +947,12 @@ lbm_status lbm_adjoint(lbm_lattice *h, const double *dL_drho1, const double *dL_
         cs = nullptr;
         cudaGetLastError();
     }
-    auto segment_graph = [&](int par, const void *first) -> cudaGraphExec_t {
+    auto segment_graph = [&](int par, const void *first, bool last) -> cudaGraphExec_t {
         if (!cs || h->seg_graph_state[par] == -1) return nullptr;
         cudaGraph_t gr = nullptr;
         bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
         if (ok) {
-            const cudaError_t er = enqueue_segment(cs, E, first, lam, lam_loc, d_cur, d_nxt);
+            const cudaError_t er = enqueue_segment(cs, E, first, lam, lam_loc, d_cur, d_nxt, last);
             const cudaError_t ee = cudaStreamEndCapture(cs, &gr);
             ok = er == cudaSuccess && ee == cudaSuccess && gr;
         }
@@ -975,9 +976,9 @@ lbm_status lbm_adjoint(lbm_lattice *h, const double *dL_drho1, const double *dL_
         const long t1 = (t0 + E < h->rec_steps) ? t0 + E : h->rec_steps;
         const long len = t1 - t0;
         const void *first = (char *)h->ckpt + sb * (size_t)k;
-        cudaGraphExec_t gx = len == E ? segment_graph(lam == h->ws_lam ? 0 : 1, first) : nullptr;
+        cudaGraphExec_t gx = len == E ? segment_graph(lam == h->ws_lam ? 0 : 1, first, k == 0) : nullptr;
         if (gx) CKA(cudaGraphLaunch(gx, h->stream), "lbm_adjoint: segment graph");
-        else CKA(enqueue_segment(h->stream, len, first, lam, lam_loc, d_cur, d_nxt), "lbm_adjoint: segment");
+        else CKA(enqueue_segment(h->stream, len, first, lam, lam_loc, d_cur, d_nxt, k == 0), "lbm_adjoint: segment");
         if (len & 1) {
             std::swap(lam, lam_loc);
             std::swap(d_cur, d_nxt);

@@ -135,11 +135,12 @@ cudaError_t launch_step_split_noalloc(const HostPhys &p, const void *f_in, void 
 int adjoint_blocks(int storage);
 // Whether the reverse step keeps lambda_loc as 5 values per cell (tau = 1, the
 // exact-difference forcing, FP32 arithmetic, replayed sums): these are in the lambda
-// buffer, base_a added to D.
+// buffer, base_a added to D but for the last reverse step (last), after which
+// launch_adjoint_rho0 adds the two in FP64.
 bool adjoint_eq(const HostPhys &h, int rho_is_sums);
 cudaError_t launch_adjoint_step(const HostPhys &p, const void *f, const void *rho, int rho_is_sums,
                                 const void *lam_next, const void *Dn, void *lam_loc, void *a, void *Dout,
-                                double *partials, cudaStream_t s);
+                                double *partials, cudaStream_t s, bool last);
 // lambda_loc^N_i = dL/drho^a of the component of i (g1/g2 may be NULL); D^N, cleared by
 // the caller, takes it instead where adjoint_eq.
 cudaError_t launch_adjoint_seed(const HostPhys &p, const void *g1, const void *g2, int g_f64, void *lam, void *D,
