@@ -252,14 +252,15 @@ lbm_status lbm_sync(lbm_lattice *h);
  * forcing reading, every collision operator, periodic lattices, z walls and
  * solid masks.
  *
- * lbm_record runs n_steps >= 1 forward exactly as lbm_step does and keeps the
- * raw state every ckpt_every >= 1 steps (a library-owned checkpoint store of
- * ceil(n_steps / ckpt_every) states), and reserves the working memory of the
- * reverse pass (adjoint fields of 2 x 19 values per cell, one checkpoint
- * segment of states and of their densities); both are held until the next
- * lbm_record of another shape, lbm_set_solid or lbm_destroy, so that lbm_adjoint
- * allocates nothing.
- * Synchronizes.  Errors: LBM_EINVAL, LBM_ENOMEM, LBM_ECUDA. */
+ * lbm_record runs n_steps >= 1 forward as that many calls of lbm_step with one
+ * step each do, so that the reverse pass recomputes the same states bit for
+ * bit, keeps the raw state every ckpt_every >= 1 steps (a library-owned
+ * checkpoint store of ceil(n_steps / ckpt_every) states), and reserves the
+ * working memory of the reverse pass (adjoint fields of 2 x 19 values per cell,
+ * one checkpoint segment of states and of their densities); both are held until
+ * the next lbm_record of another shape, lbm_set_solid or lbm_destroy, so that
+ * lbm_adjoint allocates nothing.  (A call of lbm_step with all the steps may
+ * take them in moment space and then agrees to rounding.)  Synchronizes.  Errors: LBM_EINVAL, LBM_ENOMEM, LBM_ECUDA. */
 lbm_status lbm_record(lbm_lattice *h, long n_steps, int ckpt_every);
 
 /* Reverse pass over the last lbm_record.  Inputs dL_drho1, dL_drho2: N values

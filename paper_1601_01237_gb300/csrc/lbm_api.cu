@@ -412,10 +412,11 @@ bool capturing(cudaStream_t s)
     return false;
 }
 
-// Bytes of a moment state if the lattice's next n steps run in moment space, else 0.  A run of even n over both copies leaves its
-// state in the other copy and moments in the one it began with, so that a caller's
-// graph of it could not be replayed; while one is captured such a run goes step by
-// step, which ends in the copy it began with.
+// Bytes of a moment state if the lattice's next n steps run in moment space, else
+// 0.  A run of even n over both copies leaves its state in the other copy and
+// moments in the one it began with, so that a caller's graph of it could not be
+// replayed; while one is captured such a run goes step by step, which ends in the
+// copy it began with.
 size_t moment_run_bytes(const lbm_lattice *h, long n)
 {
     if (!h->mplan.pays(n)) return 0;
@@ -423,17 +424,9 @@ size_t moment_run_bytes(const lbm_lattice *h, long n)
     return n % 2 == 0 && !moment_one_copy(h, b) && capturing(h->stream) ? 0 : b;
 }
 
-}  // namespace
-
-lbm_status lbm_step(lbm_lattice *h, long n_steps)
+// n steps on populations, one launch of launch_one each.
+lbm_status population_steps(lbm_lattice *h, long n_steps)
 {
-    if (!h) return fail(LBM_EINVAL, "lbm_step: NULL handle");
-    if (n_steps < 0) return fail(LBM_EINVAL, "lbm_step: n_steps = %ld < 0", n_steps);
-    DeviceGuard g(h->device);
-    if (const size_t mb = moment_run_bytes(h, n_steps)) {
-        const cudaError_t e = moment_run(h, n_steps, mb);
-        return e == cudaSuccess ? LBM_OK : cuda_fail(e, "lbm_step: launch");
-    }
     long t = 0;
     auto plain = [&](long upto) -> lbm_status {
         for (; t < upto; ++t) {
@@ -460,6 +453,20 @@ lbm_status lbm_step(lbm_lattice *h, long n_steps)
         }
     }
     return plain(n_steps);
+}
+
+}  // namespace
+
+lbm_status lbm_step(lbm_lattice *h, long n_steps)
+{
+    if (!h) return fail(LBM_EINVAL, "lbm_step: NULL handle");
+    if (n_steps < 0) return fail(LBM_EINVAL, "lbm_step: n_steps = %ld < 0", n_steps);
+    DeviceGuard g(h->device);
+    if (const size_t mb = moment_run_bytes(h, n_steps)) {
+        const cudaError_t e = moment_run(h, n_steps, mb);
+        return e == cudaSuccess ? LBM_OK : cuda_fail(e, "lbm_step: launch");
+    }
+    return population_steps(h, n_steps);
 }
 
 lbm_status lbm_step_timed(lbm_lattice *h, long n_steps, double kernel_ms[4], long launches[4],
@@ -828,17 +835,13 @@ lbm_status lbm_record(lbm_lattice *h, long n_steps, int ckpt_every)
         h->ws_every = (long)E;
     }
     h->rec_at_rest = h->init_at_rest && h->steps == 0;
-    const bool rounds = h->phys.storage != lbm::ST_F32 && h->phys.storage != lbm::ST_F64;
     for (long t = 0; t < n_steps; t += ckpt_every) {
         CK(cudaMemcpyAsync((char *)h->ckpt + sb * (size_t)(t / ckpt_every), h->f[h->cur], sb,
                            cudaMemcpyDeviceToDevice, h->stream),
            "lbm_record: checkpoint");
-        // in 16 bits step by step: the reverse pass recomputes the same rounded states
-        const long n = std::min<long>(ckpt_every, n_steps - t), each = rounds ? 1 : n;
-        for (long k = 0; k < n; k += each) {
-            const lbm_status st = lbm_step(h, each);
-            if (st != LBM_OK) return st;
-        }
+        // on populations, as the reverse pass recomputes the states: the same bit for bit
+        const lbm_status st = population_steps(h, std::min<long>(ckpt_every, n_steps - t));
+        if (st != LBM_OK) return st;
     }
     CK(cudaStreamSynchronize(h->stream), "lbm_record: sync");
     h->rec_steps = n_steps;
