@@ -161,7 +161,11 @@ def measured_hbm_peak():
 
 
 # source files that define each timed kernel (a change to any of them voids
-# the committed DRAM-traffic figure of that kernel)
+# the committed DRAM-traffic figure of that kernel).  Under the name k_step_fused the
+# library times the single-pass step of either kind; the committed figures are of the
+# marching kernel, which lattices of TRAFFIC_MIN_SIDE cells or more along every axis take
+# (smaller and thinner ones may take the box step of lbm_box_impl.cuh).
+TRAFFIC_MIN_SIDE = 96
 KERNEL_SOURCES = {"k_step_fused": ("d3q19.cuh", "collide.cuh", "lbm_fused_impl.cuh"),
                   "k_density": ("d3q19.cuh", "lbm_forward.cu"),
                   "k_collide": ("d3q19.cuh", "lbm_forward.cu"),
@@ -182,9 +186,12 @@ def kernel_source_hash(kernel):
     return h.hexdigest()[:16]
 
 
-def ncu_traffic(kernel, storage, cells):
-    """DRAM bytes per launch from the committed ncu summary, scaled by cells,
-    or None when the kernels changed since the capture."""
+def ncu_traffic(kernel, storage, shape):
+    """DRAM bytes per launch from the committed ncu summary, scaled by cells, or
+    None when the kernels changed since the capture or the lattice is below
+    TRAFFIC_MIN_SIDE."""
+    if min(shape) < TRAFFIC_MIN_SIDE:
+        return None
     path = os.path.join(ROOT, "profiles", "dram_traffic.json")
     try:
         d = json.load(open(path))
@@ -193,7 +200,7 @@ def ncu_traffic(kernel, storage, cells):
     e = d.get("%s/%s" % (kernel, storage))
     if not e or e.get("kernel_source_sha") != kernel_source_hash(kernel):
         return None
-    return e["dram_bytes_per_cell"] * cells
+    return e["dram_bytes_per_cell"] * int(np.prod(shape))
 
 
 def algorithmic_bytes_per_cell(kernel, storage, tau_one=True):
@@ -430,7 +437,7 @@ def run_ours(args, rank, world, local_rank):
     achieved = alg / per_launch_s / 1e9
     # (steps in moment space are bound by shared memory and FP32 issue together)
     roofline = {"bound": "hbm" if dom != "k_step_moment" else "shared memory and issue", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": ncu_traffic(dom, storage, cells), "kernel": dom,
+                "traffic": ncu_traffic(dom, storage, shape), "kernel": dom,
                 "algorithmic_bytes_per_launch": alg, "launch_ms": per_launch_s * 1e3,
                 "peak_source": peak_src,
                 "kernels": {k: {"ms_per_launch": v[0] / v[1], "launches": v[1],

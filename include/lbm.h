@@ -154,8 +154,9 @@ lbm_status lbm_step(lbm_lattice *h, long n_steps);
  * lbm_step does, recording a CUDA event pair around every kernel launch on the
  * lattice's stream, then synchronizes.  kernel_ms[k] receives the total device
  * time of kernel kind k over the n_steps, launches[k] its launch count, and
- * names[k] (static strings) its name, for k < *n_kinds <= 4.  Used by the
- * benchmark for per-launch durations.  Errors: LBM_EINVAL, LBM_ECUDA. */
+ * names[k] (static strings) its name, for k < *n_kinds <= 4 ("k_step_fused": the
+ * single-pass step, as the marching kernel or, on small and thin lattices, the
+ * box kernel takes it).  Used by the benchmark for per-launch durations.  Errors: LBM_EINVAL, LBM_ECUDA. */
 lbm_status lbm_step_timed(lbm_lattice *h, long n_steps, double kernel_ms[4], long launches[4],
                           const char *names[4], int *n_kinds);
 
