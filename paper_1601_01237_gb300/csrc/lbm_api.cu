@@ -656,22 +656,22 @@ lbm_status lbm_set_solid(lbm_lattice *h, const unsigned char *solid, int on_devi
     choose_paths(h);
     if (!solid) return LBM_OK;
     const size_t N = (size_t)h->phys.N;
-    CK(cudaMalloc((void **)&h->solid, N), "lbm_set_solid: mask");
-    CK(cudaMalloc((void **)&h->links, N * sizeof(unsigned)), "lbm_set_solid: link flags");
-    CK(cudaMemcpyAsync(h->solid, solid, N, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                       h->stream), "lbm_set_solid: copy");
-    CK(lbm::launch_link_flags(h->phys, h->solid, h->links, h->stream), "lbm_set_solid: link flags");
-    h->phys.solid = h->solid;
-    h->phys.links = h->links;
-    choose_paths(h);
     {
-        // wall densities (fused step) and the boundary lists of the mirror
-        // model (fused step and reverse pass): count, then list
+        // mask and link flags, wall densities (fused step) and the boundary lists of
+        // the mirror model (fused step and reverse pass): count, then list.  The steps
+        // read all of it or none: whatever fails, the lattice is left without a mask.
         unsigned long long *cnt = nullptr, cnt_h[2] = {0, 0};
-        CK(cudaMalloc((void **)&h->wall_rho, 2 * N * sizeof(float)), "lbm_set_solid: wall densities");
-        CK(cudaMemsetAsync(h->wall_rho, 0, 2 * N * sizeof(float), h->stream), "lbm_set_solid: wall densities");
-        CK(cudaMalloc((void **)&cnt, 2 * sizeof(unsigned long long)), "lbm_set_solid: counters");
-        cudaError_t e = cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), h->stream);
+        cudaError_t e = cudaMalloc((void **)&h->solid, N);
+        if (e == cudaSuccess) e = cudaMalloc((void **)&h->links, N * sizeof(unsigned));
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(h->solid, solid, N, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = lbm::launch_link_flags(h->phys, h->solid, h->links, h->stream);
+        h->phys.solid = h->solid;
+        h->phys.links = h->links;
+        if (e == cudaSuccess) e = cudaMalloc((void **)&h->wall_rho, 2 * N * sizeof(float));
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->wall_rho, 0, 2 * N * sizeof(float), h->stream);
+        if (e == cudaSuccess) e = cudaMalloc((void **)&cnt, 2 * sizeof(unsigned long long));
+        if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), h->stream);
         if (e == cudaSuccess)
             e = lbm::launch_mask_setup(h->phys, h->solid, h->wall_rho, nullptr, nullptr, cnt, h->stream);
         if (e == cudaSuccess)
@@ -699,8 +699,7 @@ lbm_status lbm_set_solid(lbm_lattice *h, const unsigned char *solid, int on_devi
         cudaFree(cnt);
         if (e != cudaSuccess) {
             free_mask(h);
-            choose_paths(h);
-            return cuda_fail(e, "lbm_set_solid: boundary lists");
+            return cuda_fail(e, "lbm_set_solid: mask");
         }
         h->phys.wall_rho = h->wall_rho;
         h->phys.bfluid = h->bfluid;
@@ -708,7 +707,7 @@ lbm_status lbm_set_solid(lbm_lattice *h, const unsigned char *solid, int on_devi
         h->phys.n_bfluid = (long long)cnt_h[0];
         h->phys.n_bsolid = (long long)cnt_h[1];
     }
-    CK(cudaStreamSynchronize(h->stream), "lbm_set_solid: sync");
+    choose_paths(h);
     return LBM_OK;
 }
 
