@@ -253,8 +253,9 @@ static_assert(cx(7) == 1 && cy(7) == 1 && cz(11) == 1, "first diagonal of each a
 // 0.33 / 0.23, and in FP64 with q = rho times the rounded 1/36 a mean of -0.50 per step.
 // Parameter derivatives of 50 steps at 96^3 (six droplets, largest error over largest
 // value): with the last of these 6.5e-8 / 8.2e-8 / 7.6e-8 / 3.3e-8, here 2.0e-8 / 2.2e-8 /
-// 2.2e-8 / 3.1e-8.  us per step, that form and this one: 512^3 3052 / 3044, 256^3 393 /
-// 402, regularized 617 / 631, FP64 1 x 64 x 64 8.8 / 9.2.
+// 2.2e-8 / 3.1e-8.  us per step, that form and this one in the same kernels: runs in
+// moment space 512^3 3052 / 3044, 256^3 393 / 402, regularized 617 / 631, FP64 1 x 64 x 64
+// 8.8 / 9.1.
 template <class C, int REG, int FORCE, bool DEV, class GET, class PUT>
 __device__ __forceinline__ void collide_cell(const C &c, const Phys<typename C::R> &p, typename C::V r,
                                              typename C::R inv, typename C::R ux, typename C::R uy, typename C::R uz,

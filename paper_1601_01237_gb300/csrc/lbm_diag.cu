@@ -199,7 +199,6 @@ Geo<R> geo_of(const HostPhys &h)
 
 }  // namespace
 
-int diag_blocks() { return kDiagBlocks; }
 int diag_grid(long long N) { return (int)std::min<long long>(kDiagBlocks, (N + kThreadsD - 1) / kThreadsD); }
 int diag_slots() { return kSlots; }
 

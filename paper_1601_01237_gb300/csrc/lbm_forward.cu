@@ -306,7 +306,7 @@ k_collide(const typename Store<S>::T *__restrict__ fin, typename Store<S>::T *__
 //   - warps inside a wall do no arithmetic.
 // Of CTAs of 32, 64 and 128 threads the smallest leaves the least imbalance
 // (34^3 39.5 / 42.7 / 42.7 us per step).  us per step before and now: 1 x 64 x 64
-// 39.8 / 8.8, 1 x 300 x 300 115 / 60, 34^3 periodic 94.7 / 39.5, 128^3 2046 / 1225.
+// 39.8 / 9.1, 1 x 300 x 300 115 / 60, 34^3 periodic 94.7 / 39.5, 128^3 2046 / 1225.
 constexpr int kThreads64 = 32;
 
 struct Nbr32 {

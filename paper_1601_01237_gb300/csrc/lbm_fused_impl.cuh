@@ -270,7 +270,8 @@ __device__ __forceinline__ void decode_all(const typename Store<S>::Raw (&r)[Q],
     }
 }
 
-// Densities and momentum in the fixed order of collide_scalar: as density and momentum, with the two components added before the opposite
+// Densities and momentum in the fixed order of collide_scalar: the densities in
+// density()'s grouping, the momentum with the two components added before opposite
 // directions are subtracted.
 __device__ __forceinline__ void sums_scalar(const float2 (&v)[Q], float2 &r, float &jx, float &jy, float &jz)
 {

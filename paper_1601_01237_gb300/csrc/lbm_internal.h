@@ -23,8 +23,6 @@ struct HostPhys {
     double rho_s[2];
     double rho0;
     // N flags on the device, 1 = solid site (staircase walls); nullptr = none.
-    // Only the two-kernel step and its density, output and reduction kernels
-    // take a mask.
     const unsigned char *solid = nullptr;
     // N words of link flags derived from the mask: bit i set when the pull
     // source x - c_i of cell x is a solid site (bit 0: x itself is solid;
@@ -153,7 +151,6 @@ cudaError_t launch_density(const HostPhys &p, const void *f, void *rho, cudaStre
 
 // FP64 diagnostics over the density fields in rho (diag_grid(N) x
 // diag_slots() partial doubles).
-int diag_blocks();                  // at most
 int diag_grid(long long N);         // of a lattice of N cells
 int diag_slots();
 cudaError_t launch_pressure(const HostPhys &h, const void *rho, const double center[3], double r_in, double r_out,

@@ -17,9 +17,9 @@
 // 100 steps over those of population steps: 0.92 to 0.97, 0.89 to 0.94; u_z with plain sums
 // 1.04 to 1.13); the state at the end of the call is the population state.
 // us per step in calls of 10 (512^3), 20 (256^3) and 100 steps, population steps and
-// these: tau = 1 512^3 6723 / 2650, 256^3 842 / 371, 128^3 119 / 55, 96^3 52 / 33,
-// regularized 256^3 883 / 592, 384 x 512 x 512 with walls 5900 / 3190,
-// tau = 1 under a mask 256^3 1020 / 405.
+// these with their ends: tau = 1 512^3 6991 / 3251, 256^3 869 / 414, 128^3 122 / 57, 96^3
+// 55 / 33, regularized 256^3 873 / 649, 384 x 512 x 512 with walls 5424 / 3728, tau = 1 under
+// a mask 256^3 1042 / 455.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -177,7 +177,7 @@ k_moment_out(MomentState<KIND> m, typename Store<FMT>::T *__restrict__ f, Phys<f
 // Wall densities of the mirror model under a mask, after each new moment state:
 // each solid site with a fluid neighbour takes the w_i-weighted mean of its fluid
 // neighbours' densities plus rho_s (Eq. 13).  One thread per site: the sites are a
-// surface, so launch and one gather's latency bound it (8.5 us beside the 396 of a
+// surface, so launch and one gather's latency bound it (8.5 us beside the 425 of a
 // 256^3 step with an inclined slab).
 __global__ void __launch_bounds__(kThreadsM)
 k_moment_walls(float2 *__restrict__ rho, Phys<float> p, const unsigned *__restrict__ links,
